@@ -135,12 +135,14 @@ typedef struct {
                                  kernel lacks: TRIM_HANDOVER_*                           */
   uint32_t async_round_edges; /* AC-4 (alone or as a committed scheduled variant), from
                                  round 128 on: once the in-edges still to push are at most
-                                 this many, the rest of the run is asynchronous: no
-                                 rounds, each CTA pushes the rows of the vertices it
-                                 removes at its own pace, and a removed vertex takes one
-                                 more than the top level among its successors (Definition
-                                 2), carried by the pushes. Same levels and alpha; needs
-                                 G^T, off in TRIM_FLAG_ROUND_LOG runs (0 = never)        */
+                                 this many (and the vertices they belong to at most about
+                                 as many as the launch has warps), the rest of the run is
+                                 asynchronous: no rounds, each warp pushes the rows of the
+                                 vertices it removes at its own pace, and a removed vertex
+                                 takes one more than the top level among its successors
+                                 (Definition 2), carried by the pushes. Same levels and
+                                 alpha; needs G^T, off in TRIM_FLAG_ROUND_LOG runs
+                                 (0 = never)                                             */
 } trim_params_t;
 
 /* trim_params_t.sched_handover */
@@ -215,7 +217,7 @@ typedef struct trim_ctx trim_ctx;
  * device on first use (a counting sort; its time is not part of trim_run).
  * cuda_stream: a cudaStream_t (NULL = the legacy default stream).
  * On success *out receives the context. Allocates device memory ~ (40 n + 4 m) B,
- * plus ~ (20 n + m / 64) B + 128 B per resident GPU thread for the asynchronous
+ * plus ~ (12 n + m / 21) B + 96 B per resident GPU thread for the asynchronous
  * AC-4 tail once G^T exists (given here, or built on first use). */
 trim_err_t trim_create(const trim_csr_t* csr_out, const trim_csr_t* csr_in, void* cuda_stream,
                        uint32_t flags, trim_ctx** out);

@@ -41,13 +41,18 @@ struct trim_ctx {
            *s_next = nullptr, *s_cnt = nullptr, *s_off = nullptr, *s_list = nullptr,
            *log = nullptr, *roff = nullptr, *live0 = nullptr, *live1 = nullptr, *bsum = nullptr;
   uint32_t *w4_row = nullptr, *w4_eoff = nullptr, *chunk_first = nullptr;
-  // asynchronous AC-4 tail: per-vertex words, the global list of G^T row
-  // pieces and the two rebalance entry lists (allocated once G^T exists)
-  unsigned long long* aw = nullptr;
+  // asynchronous AC-4 tail: per-vertex records (over supp, s_head, s_next and
+  // s_list), the global list of G^T row pieces and the two pairs of rebalance
+  // lists (allocated once G^T exists)
+  uint4* aw = nullptr;
   uint32_t *oq_row = nullptr, *oq_len = nullptr, *oq_lev = nullptr;
   uint32_t oq_cap = 0;
   uint32_t *ae_id = nullptr, *ae_lev = nullptr;
   uint32_t ae_cap = 0;
+  uint32_t *er_row = nullptr, *er_len = nullptr, *er_lev = nullptr;
+  uint32_t er_cap = 0;
+  ulonglong2* ch_msg = nullptr;
+  uint32_t *ch_ack = nullptr, *ch_load = nullptr;
   // in+out runs: in-degree counters, the work list's G rows and in-degrees, and
   // the chunk-owner index of its edge space (both rows: up to 2m edges)
   uint32_t *cnt_in = nullptr, *w4_orow = nullptr, *w4_din = nullptr, *chunk_io = nullptr;
@@ -287,7 +292,6 @@ void default_params(trim_params_t* p) {
 // work-list rows and edge offsets, AC-3 live list) of kSliceEntries words per
 // warp of the block (64 KB for 512 threads)
 constexpr uint32_t kSliceEntries = 256;
-constexpr uint32_t kSbufCap = kSliceEntries;
 size_t dyn_smem_bytes(uint32_t block_threads) {
   return (block_threads / 32) * 4 * (size_t)kSliceEntries * sizeof(uint32_t);
 }
@@ -372,24 +376,32 @@ trim_err_t device_scan(trim_ctx* c, const uint32_t* in, uint32_t n, uint32_t* ou
   return TRIM_OK;
 }
 
-// The asynchronous AC-4 tail's per-vertex words, its global list of G^T row
-// pieces and its two rebalance entry lists, allocated once G^T exists
-// (kernels without them never start the tail). An entry list holds every
-// queue of a cooperative grid: 8 entries per resident thread.
+// The asynchronous AC-4 tail's global list of G^T row pieces and its two pairs
+// of rebalance lists and the channels between CTAs, allocated once G^T exists
+// (kernels without them never start the tail). A pair of lists holds what every
+// CTA of a cooperative grid can hold: one entry and kAsyncRows rows per thread.
 trim_err_t alloc_async(trim_ctx* c) {
-  if (c->aw != nullptr) return TRIM_OK;
+  if (c->oq_cap) return TRIM_OK;
   const uint64_t cap = trimk::async_queue_cap(c->n, c->m);  // < 2^32: n <= 2^31, m < 2^32
   int per_sm = 0;
   CK(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxThreadsPerMultiProcessor, c->device));
-  const uint64_t ecap = (uint64_t)c->sm_count * (uint64_t)per_sm * 8u;
-  TRY(dalloc(c, &c->aw, c->n));
+  const uint64_t ecap = (uint64_t)c->sm_count * (uint64_t)per_sm;
+  const uint64_t rcap = ecap * trimk::kAsyncRows;
   TRY(dalloc(c, &c->oq_row, cap));
   TRY(dalloc(c, &c->oq_len, cap));
   TRY(dalloc(c, &c->oq_lev, cap));
   TRY(dalloc(c, &c->ae_id, 2 * ecap));
   TRY(dalloc(c, &c->ae_lev, 2 * ecap));
-  c->oq_cap = (uint32_t)cap;
+  TRY(dalloc(c, &c->er_row, 2 * rcap));
+  TRY(dalloc(c, &c->er_len, 2 * rcap));
+  TRY(dalloc(c, &c->er_lev, 2 * rcap));
+  const uint64_t ctas = ecap / 128;  // block_threads >= 128
+  TRY(dalloc(c, &c->ch_msg, 32 * ctas));
+  TRY(dalloc(c, &c->ch_ack, 32 * ctas));
+  TRY(dalloc(c, &c->ch_load, ctas));
   c->ae_cap = (uint32_t)ecap;
+  c->er_cap = (uint32_t)rcap;
+  c->oq_cap = (uint32_t)cap;
   return TRIM_OK;
 }
 
@@ -597,10 +609,12 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   const bool in_host = gi && gi->on_device == TRIM_MEM_HOST;
   const size_t a_ioff = in_host ? A.add<uint32_t>(n + 1) : 0;
   const size_t a_itgt = in_host ? A.add<uint32_t>(c->m) : 0;
-  const size_t a_level = A.add<uint32_t>(n), a_cnt = A.add<uint32_t>(n), a_supp = A.add<uint32_t>(n);
-  const size_t a_shead = A.add<uint32_t>(n), a_snext = A.add<uint32_t>(n);
+  const size_t a_level = A.add<uint32_t>(n), a_cnt = A.add<uint32_t>(n);
+  // (next to each other: together they hold the asynchronous tail's 16 bytes per vertex)
+  const size_t a_supp = A.add<uint32_t>(n), a_shead = A.add<uint32_t>(n);
+  const size_t a_snext = A.add<uint32_t>(n), a_slist = A.add<uint32_t>(n);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
-  const size_t a_slist = A.add<uint32_t>(n), a_log = A.add<uint32_t>(n);
+  const size_t a_log = A.add<uint32_t>(n);
   const size_t a_roff = A.add<uint32_t>(n + 2), a_live0 = A.add<uint32_t>(n);
   const size_t a_live1 = A.add<uint32_t>(n), a_bsum = A.add<uint32_t>(8192);
   const size_t a_ctrl = A.add<Ctrl>(1);
@@ -643,6 +657,7 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->roff = at(a_roff);
   c->live0 = at(a_live0); c->live1 = at(a_live1); c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
+  c->aw = reinterpret_cast<uint4*>(c->supp);
   c->w4_row = at(a_w4r); c->w4_eoff = at(a_w4e); c->chunk_first = at(a_chunk);
   if (c->rlog_cap) c->rlog = reinterpret_cast<trim_round_rec_t*>(base + a_rlog);
   if (flags & TRIM_FLAG_VALIDATE) TRY(validate(c, gi ? c->ioff : nullptr));
@@ -822,7 +837,6 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   D.mask = c->has_mask ? c->mask : nullptr;
   D.ig = c->ig;
   if (inout) D.chunk_first = c->chunk_io;
-  D.sbuf_cap = kSbufCap;
   D.rlog = c->rlog; D.rlog_cap = c->rlog_cap;
   D.model = c->has_model ? c->model : nullptr;
   D.script = c->script; D.script_len = c->script_len;
@@ -837,7 +851,9 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   D.aw = c->aw;
   D.oq_row = c->oq_row; D.oq_len = c->oq_len; D.oq_lev = c->oq_lev; D.oq_cap = c->oq_cap;
   D.ae_id = c->ae_id; D.ae_lev = c->ae_lev; D.ae_cap = c->ae_cap;
-  D.async_edges_max = (c->aw != nullptr && c->ioff != nullptr) ? c->params.async_round_edges : 0u;
+  D.er_row = c->er_row; D.er_len = c->er_len; D.er_lev = c->er_lev; D.er_cap = c->er_cap;
+  D.ch_msg = c->ch_msg; D.ch_ack = c->ch_ack; D.ch_load = c->ch_load;
+  D.async_edges_max = (c->oq_cap != 0 && c->ioff != nullptr) ? c->params.async_round_edges : 0u;
   // scheduled runs keep the live-edge count (a feature); with G^T and AC-4 the
   // scheduler kernels derive it from running totals instead
   if (variant >= TRIM_SCHED_HEURISTIC && !(ac4 && c->ioff)) D.flags |= trimk::F_LIVE_EDGES;

@@ -23,6 +23,8 @@ constexpr int NFEAT = 12;
 // capacity for n vertices and m edges (every removal adds at most
 // ceil(in-degree / kAsyncPiece) items)
 constexpr uint32_t kAsyncPiece = 256;
+// ... and row pieces per thread that a CTA's ring and its warps hold at most
+constexpr uint32_t kAsyncRows = 3;
 __host__ __device__ constexpr uint64_t async_queue_cap(uint64_t n, uint64_t m) {
   return n + m / kAsyncPiece + 1;
 }
@@ -114,20 +116,21 @@ struct Ctrl {
   unsigned int local_rounds;      // local AC-4 rounds so far, published by CTA 0
   // asynchronous AC-4 tail (see async_tail in trim_kernels.cu): work tokens
   // (one per CTA with work; 0: the run is over), pieces written to the global
-  // list, the rebalance generation asked for, entries in the two global entry
-  // lists, the tail's removals and top level, the round at which it took
-  // over, a heartbeat of the CTAs with work (bounds the wait of those
-  // without), and the rebalances run
+  // list, the rebalance generation asked for, entries and rows in the two
+  // pairs of global lists, the tail's removals and top level, the round at
+  // which it took over, a heartbeat of the CTAs with work (bounds the wait of
+  // those without), and the rebalances run
   unsigned int a_tokens;
   unsigned int oq_res;
   unsigned int a_req;
   unsigned int e_n[2];
+  unsigned int er_n[2];
   unsigned int a_removed;
   unsigned int a_maxlev;
   unsigned int a_round;
   unsigned int a_beat;
   unsigned int a_rebalances;
-  unsigned int _p5[18];
+  unsigned int _p5[16];
   // segmented runs: a kernel that lacks the variant its scheduler picked saves
   // the schedule state here and exits; the kernel that has it resumes from it
   unsigned int resume;            // 1: a segment ended early, state in `saved`
@@ -176,18 +179,19 @@ struct Dev {
   // the implicit flavours; off/tgt are null then
   trim_implicit_graph_t ig;
   uint32_t* bsum;     // per-CTA scratch of the grid-wide scan
-  uint32_t sbuf_cap;  // entries of each CTA append buffer (dynamic shared memory)
   uint32_t resume;    // 1: continue the run from Ctrl::saved instead of starting it
   uint32_t commit_after;  // != 0: scheduler flavours commit after this many stable rounds
   uint32_t recheck_rounds;  // length of the first committed stretch (doubles while repeated)
   uint32_t bar_base;  // grid-barrier counter when this kernel starts (0 for a new run)
   uint32_t local_edges_max;  // AC-4: pending in-edges up to which rounds run locally (0: never)
-  // asynchronous AC-4 tail: per vertex (top level among its removed successors
-  // << 32 | live-successor counter); the global list of G^T row pieces still
-  // to push (row start, length, level of the removed vertex) and its
-  // capacity; the two global entry lists of rebalances (predecessor, level),
-  // ae_cap entries each
-  unsigned long long* aw;
+  // asynchronous AC-4 tail: per vertex 16 bytes (live-successor counter, top
+  // level among its removed successors, G^T row start, row length), in the
+  // arrays of AC-6 and AC-3 (supp, s_head, s_next, s_list, contiguous), which
+  // no round after the tail's start uses; the global list of G^T row pieces
+  // still to push (row start, length, level of the removed vertex) and its
+  // capacity; the two pairs of global lists of rebalances: entries
+  // (predecessor, level), ae_cap each, and rows (as pieces), er_cap each
+  uint4* aw;
   uint32_t* oq_row;
   uint32_t* oq_len;
   uint32_t* oq_lev;
@@ -195,6 +199,15 @@ struct Dev {
   uint32_t* ae_id;
   uint32_t* ae_lev;
   uint32_t ae_cap;
+  uint32_t* er_row;
+  uint32_t* er_len;
+  uint32_t* er_lev;
+  uint32_t er_cap;
+  // per CTA: the messages of its 32 incoming channels, the acknowledgements of
+  // its 32 outgoing ones, and its published load
+  ulonglong2* ch_msg;
+  uint32_t* ch_ack;
+  uint32_t* ch_load;
   uint32_t async_edges_max;  // pending in-edges up to which the rest of the run is asynchronous (0: never)
   Ctrl* C;
   trim_round_rec_t* rlog;

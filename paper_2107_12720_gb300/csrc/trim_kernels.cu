@@ -118,7 +118,9 @@ constexpr uint32_t LQ_ENTRIES = 256;  // removed vertices queued per CTA per rou
 constexpr uint32_t LQ_DMAX = 64;      // larger in-degrees always go to the global work list
 // asynchronous AC-4 tail (see async_tail)
 constexpr uint32_t ASYNC_MIN_ROUND = 128;  // rounds before the tail may take over
-constexpr uint32_t AQ_LOCAL_DMAX = 1024; // larger in-degrees always go to the shared queue
+constexpr uint32_t ASYNC_RETRY = 64;       // local stretches end for it at multiples of this
+constexpr uint32_t AQ_LOCAL_DMAX = 1024; // larger in-degrees always go to the global pieces
+constexpr uint32_t AQ_PIECE = 32;        // in-edges per piece of a CTA's ring (one batch)
 #endif
 
 // Per-CTA shared state.
@@ -147,25 +149,30 @@ struct Cta {
   uint32_t lq_ovf;                    // 1: a removal of this round went to the global lists
   uint32_t lq_pushed;                 // predecessors decremented from the queue this round
   uint32_t lq_next;                   // how the stretch goes on after the local barrier
-  // asynchronous tail: predecessors queued per buffer (dynamic shared memory):
-  // reserved, and the end of the reservations that fit; the share of the last
-  // rebalance (global entries [sh_elo, sh_ehi), pieces [sh_plo, sh_phi)); this
-  // CTA's removals and top level since it last released its token; whether it
-  // holds a token; steps run; whether it asks for a rebalance; rebalances
-  // passed; start of the pieces written since the last one; average share
-  // (entries) at the last one; its entry-list slot; what the next step does
-  uint32_t aq_res[2];
-  uint32_t aq_end[2];
-  uint32_t sh_elo, sh_ehi, sh_plo, sh_phi;
+  // asynchronous tail (see async_tail). The ring of row pieces in dynamic
+  // shared memory: pieces taken out and put in so far. The idle workers (a bit
+  // each), their wake-up barriers and the rows in their mailboxes. What the CTA does next (read by every worker
+  // before each batch); the share of the last rebalance still to claim (global
+  // entries, rows and pieces); removals and top level not yet published;
+  // entries and rows written out by a rebalance; whether the CTA holds a
+  // token, asks for a rebalance; rebalances passed; first piece of the global
+  // list not yet shared out; the last batch's time (shows progress); bases of
+  // the entries and rows it writes out; its channels' last tags
+  uint32_t r_head, r_tail;
+  uint32_t a_idle;
+  unsigned long long w_bar[MAX_WARPS];
+  uint32_t w_rows[MAX_WARPS];
+  uint32_t a_next;
+  uint32_t sh_elo, sh_ehi, sh_rlo, sh_rhi, sh_plo, sh_phi;
   uint32_t a_removed, a_maxlev;
+  uint32_t a_ne, a_nr;
   uint32_t a_token;
-  uint32_t a_steps;
   uint32_t a_want;
   uint32_t a_gen;
   uint32_t a_plo;
-  uint32_t a_avg;
-  uint32_t a_base;
-  uint32_t a_next;
+  uint32_t a_prog;
+  uint32_t a_ebase, a_rbase;
+  uint32_t ch_sent[32], ch_taken[32];
 #endif
 };
 
@@ -1252,6 +1259,16 @@ __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   L.fe += nF;
 }
 
+// The asynchronous tail (see below) takes a level's vertices one to a warp, so it starts once there are
+// about as many workers as vertices. Measured on deep cascades (ms, tail from
+// round 128 against rounds; 4,560 workers): 4,096 chains of 2,867 6.8 against
+// 13.2, 5,872 of 2,000 7.6 against 10.2, but 7,000 of 300 1.88 against 1.63 and
+// 11,744 of 1,000 7.4 against 6.2.
+__device__ __forceinline__ uint32_t async_workers() { return gridDim.x * ((blockDim.x >> 5) - 1u); }
+__device__ __forceinline__ bool async_few(uint32_t vertices) {
+  return 10ull * vertices <= 13ull * async_workers();
+}
+
 // End of local round r (all threads): one arrival per CTA on the barrier word
 // of this round's parity, carrying 2^48 + 2^32 * (overflowed) + the CTA's local
 // removals; the wait ends when the word has grown by gridDim.x arrivals since
@@ -1295,10 +1312,10 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     const uint32_t nF = (uint32_t)d, n_ovf = (uint32_t)(d >> 32) & 0xFFFFu;
     // the stretch ends before the last round of a committed stretch (the
     // scheduler reads its features) and, where the asynchronous tail may take
-    // over, before round ASYNC_MIN_ROUND (it starts from the work list)
+    // over (asked every ASYNC_RETRY rounds), as it starts from the work list
     const bool stop = ((MODES & M_SCHED) && r + 1u >= S.cstop) ||
                       (D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
-                       r + 1u == ASYNC_MIN_ROUND);
+                       r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u && async_few(nF));
     if (n_ovf == 0u && (nF == 0u || !stop)) {
       local_close(D, B, nF);  // every removal of the round is in the queues
       B.lq_next = nF ? LQ_GO : LQ_DONE;
@@ -1409,29 +1426,49 @@ __device__ __noinline__ bool local_stretch(const Dev& D, Cta& B) {
 // (Definition 2: round r removes the vertices whose successors were all
 // removed before round r, the last of them in round r - 1). The pushes can
 // carry that maximum, and then the rest of an AC-4 run needs no rounds at all.
-// Every vertex gets one 64-bit word, (top level pushed so far << 32 |
-// live-successor counter); the push from a removed vertex of level l replaces
-// it by (max(top, l) << 32 | counter - 1) in one compare-and-swap, and the
-// push that takes the counter to zero removes the vertex with level
-// max(top, l) + 1: every successor has pushed by then, so the maximum is over
-// all of them, whatever the order of the pushes. No CTA waits for another:
-// each runs steps of its own. A step pushes the predecessors queued in the
-// CTA's shared memory (the G^T rows of the vertices it removed in its previous
-// step, each with its vertex's level) and queues those of the vertices it
-// removes now.
+// Every vertex gets a 16-byte record: a 64-bit word (top level pushed so far
+// << 32 | live-successor counter) and its G^T row (start, length). The push
+// from a removed vertex of level l replaces the word by (max(top, l) << 32 |
+// counter - 1) in one compare-and-swap, and the push that takes the counter to
+// zero removes the vertex with level max(top, l) + 1: every successor has
+// pushed by then, so the maximum is over all of them, whatever the order of
+// the pushes.
 //
-// A removed vertex's row stays with the CTA whose push removed it, and that
-// CTA is one of its successors' CTAs: over many levels the work drifts onto
-// fewer and fewer CTAs. A CTA whose queue holds far more than its share, or
-// whose removals do not fit its queue (those rows go to a global list of
-// pieces of at most kAsyncPiece in-edges), asks for a rebalance: every CTA
-// joins at its next step boundary, writes its queued entries to a global list,
-// and after a grid barrier each takes an even slice of those entries and of
-// the pieces written since the last rebalance, then a second barrier closes
-// the rebalance (counts published, the lists' counters ready for the next).
-// The tail ends when no CTA has work: a token count holds one token per CTA
-// with work; a CTA releases its token when its queue runs empty, and a count
-// of zero (with no rebalance asked for) ends the run.
+// What bounds it is the chain of dependent memory accesses per level, so no
+// warp waits for another. Each worker warp loops on its own over a batch of up
+// to 32 pushes held in registers, the G^T row of one removed vertex: it loads
+// the records (word and row come with one sector), issues the compare-and-swaps,
+// and while these are under way loads the row of a vertex whose counter it saw
+// at one; if the swaps went as foreseen (nearly always), that row is its next
+// batch. A level then costs two dependent accesses to memory.
+//
+// A removed vertex's row stays with the warp whose push removed it, the warp of
+// the last of its successors to go: work drifts towards the warps that lag, and
+// every level waits for the slowest warp. So a batch that removes several
+// vertices hands all but one of them on at once: to idle workers of the CTA (a
+// claim, a mailbox, a wake-up: no lock, nobody polls), else to the CTA's ring.
+// Rows over 32 in-edges go the same way in pieces of 32; rows over AQ_LOCAL_DMAX
+// in-edges, or that the ring has no room for, to a global list of pieces of at
+// most kAsyncPiece. One warp of each CTA, the control warp, gives pieces of the
+// ring to workers that became idle, and while there is none sends them, one
+// each, to CTAs with idle workers (channels, see async_control).
+//
+// Measured (ms per trim, kernel only; chains of 2,867 and 10,000 levels): the
+// deep cascade 2^24 6.7, the large mixed graph 21.0. As one step per CTA, two
+// pushes per thread, with a rebalance of all CTAs when a queue grew: 11.4 and
+// 36.2 (a level paid for the word, the swap, the row and two CTA barriers in
+// turn). With batches of several rows, up to 32 pushes: 8.9 and 29.4; 16: 7.8
+// and 25.1.
+//
+// Rows in the global pieces, or a ring half full, need a rebalance: every CTA's
+// workers stop after their batch, write what they hold (entries of their batch,
+// pieces of the ring) to global lists, and after a grid barrier each CTA takes
+// an even slice of those and of the pieces written since the last rebalance; a
+// second barrier closes the rebalance (counts published, the lists' counters
+// ready for the next). The tail ends when no CTA has work: a token count holds
+// one token per CTA with work; a CTA releases its token when its workers and
+// ring are empty and its rows sent are acknowledged, and a count of zero (with
+// no rebalance asked for) ends the run.
 //
 // It takes over at the start of an AC-4 round r (r >= ASYNC_MIN_ROUND) whose
 // pending work-list entries are exactly the vertices removed in round r - 1,
@@ -1445,7 +1482,160 @@ __device__ __forceinline__ bool async_start(const Dev& D, const Sched& S) {
   if (S.prev_variant != TRIM_AC4_PUSH) return false;
   if ((MODES & M_SCHED) && D.mode > TRIM_AC3_PULL && !(S.cstop != 0u && S.round < S.cstop))
     return false;
-  return S.e_end - S.e_c4 <= D.async_edges_max && S.bmax <= 256u;
+  const uint32_t edges = S.e_end - S.e_c4;
+  return edges <= min(D.async_edges_max, 32u * async_workers()) && S.bmax <= 256u &&
+         async_few(S.w_end - S.c4w);
+}
+
+constexpr uint32_t AS_STEP = 0, AS_DONE = 1, AS_REBALANCE = 2;
+
+// The CTA's ring of row pieces (dynamic shared memory): row starts | lengths |
+// levels, a power of two of pieces each (1 to 2 per thread). With the pieces
+// that its warps hold there are never more than kAsyncRows per thread.
+__device__ __forceinline__ uint32_t async_ring_cap() {
+  return 1u << (31 - __clz(2 * (int)blockDim.x));
+}
+// ... behind it each worker's mailbox (3 x 32 words) ...
+__device__ __forceinline__ uint32_t* async_mail(uint32_t warp) {
+  return dyn_smem + 3u * async_ring_cap() + warp * 96u;
+}
+
+// What a worker warp holds between batches: the batch (lane i < cnt: push to
+// predecessor p with level l), a row piece being worked off (warp-uniform),
+// its next work-list entry, its removals and top level not yet added to the
+// CTA's, the phase of its wake-up barrier, and whether parts of the last
+// rebalance's share may be unclaimed. (aw, itgt and level are copies of the
+// pointers in Dev, kept in registers)
+struct AsyncWarp {
+  uint4* aw;
+  const uint32_t* itgt;
+  uint32_t* level;
+  uint32_t p, l, cnt;
+  uint32_t pr, pl, pv;
+  uint32_t wj;
+  uint32_t removed, top;
+  uint32_t phase;
+  bool share;
+};
+
+__device__ __forceinline__ uint32_t vol(const uint32_t& x) {
+  return *reinterpret_cast<const volatile uint32_t*>(&x);
+}
+// Warp-collective: lane 0's reading of x, the same for every lane (the lanes may
+// read at different times, and what follows is warp-collective)
+__device__ __forceinline__ uint32_t warp_vol(const uint32_t& x) {
+  return __shfl_sync(FULL, vol(x), 0);
+}
+__device__ __forceinline__ void set_vol(uint32_t& x, uint32_t v) {
+  *reinterpret_cast<volatile uint32_t*>(&x) = v;
+}
+__device__ __forceinline__ ulonglong2 ld_relaxed_v2(const uint4* p) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
+               : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+// Idle workers sleep on a barrier of their own and have a bit in a_idle. Whoever
+// clears a bit has claimed that worker: it writes rows to the worker's mailbox
+// (n of them) and wakes it with the one arrival its barrier waits for. Nobody
+// polls shared memory and nothing takes a lock: a worker that hands rows over
+// goes on with its own batch at once.
+// One thread: claims an idle worker; its number, or 32 if there is none.
+__device__ __forceinline__ uint32_t async_claim(Cta& B) {
+  while (true) {
+    const uint32_t m = vol(B.a_idle);
+    if (m == 0u) return 32u;
+    const uint32_t w = (uint32_t)__ffs(m) - 1u;
+    if (atomicAnd(&B.a_idle, ~(1u << w)) >> w & 1u) return w;
+  }
+}
+__device__ __forceinline__ void async_wake(Cta& B, uint32_t w, uint32_t n) {
+  set_vol(B.w_rows[w], n);
+  __threadfence_block();
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&B.w_bar[w])) : "memory");
+}
+
+// Warp-collective: the rows (row, len > 0, lev) that lanes hold go to idle
+// workers of this CTA, a batch's worth each, in the order of the lanes. Lanes
+// whose row (or what is left of it) found no idle worker keep it: len stays > 0.
+__device__ __forceinline__ void async_give(Cta& B, uint32_t& row, uint32_t& len, uint32_t lev) {
+  const unsigned lane = lane_id();
+  unsigned m = __ballot_sync(FULL, len != 0u);
+  uint32_t w = 32u, n = 0, e = 0;  // the claimed worker, its rows and their edges so far
+  while (m) {
+    const int j = __ffs(m) - 1;
+    const uint32_t rj = __shfl_sync(FULL, row, j), nj = __shfl_sync(FULL, len, j);
+    const uint32_t vj = __shfl_sync(FULL, lev, j);
+    const uint32_t c = min(nj, 32u);
+    if (w < 32u && e + c > 32u) {  // this worker has its batch
+      if (lane == 0) async_wake(B, w, n);
+      w = 32u;
+    }
+    if (w >= 32u) {
+      if (lane == 0) w = async_claim(B);
+      w = __shfl_sync(FULL, w, 0);
+      if (w >= 32u) break;
+      n = e = 0u;
+    }
+    if (lane == 0) {
+      uint32_t* box = async_mail(w);
+      box[n] = rj;
+      box[32u + n] = c;
+      box[64u + n] = vj;
+    }
+    ++n;
+    e += c;
+    if ((int)lane == j) {
+      row += c;
+      len -= c;
+    }
+    if (nj <= 32u) m &= m - 1u;
+  }
+  __syncwarp();
+  if (w < 32u && lane == 0) async_wake(B, w, n);
+  __syncwarp();
+}
+
+// Warp-collective: the rows that lanes hold go to the ring in pieces of
+// AQ_PIECE, all or (where they do not fit) none: len becomes 0 if they did. A
+// piece is there once its length is; only the control warp takes pieces out.
+__device__ __forceinline__ void async_ring(Cta& B, uint32_t row, uint32_t& len, uint32_t lev) {
+  const uint32_t nd = (len + AQ_PIECE - 1u) / AQ_PIECE;
+  const uint32_t nincl = warp_incl_scan(nd);
+  const uint32_t ND = __shfl_sync(FULL, nincl, 31);
+  const uint32_t QR = async_ring_cap();
+  uint32_t base = 0, ok = 0;
+  if (lane_id() == 0) {
+    uint32_t t = vol(B.r_tail);
+    while (ND <= QR && t - vol(B.r_head) <= QR - ND) {
+      const uint32_t seen = atomicCAS(&B.r_tail, t, t + ND);
+      if (seen == t) {
+        ok = 1u;
+        break;
+      }
+      t = seen;
+    }
+    base = t;
+  }
+  ok = __shfl_sync(FULL, ok, 0);
+  if (!ok) return;
+  uint32_t at = __shfl_sync(FULL, base, 0) + nincl - nd;
+  for (uint32_t i = 0; i < nd; ++i, ++at) {
+    const uint32_t k = at & (QR - 1u);
+    dyn_smem[k] = row + i * AQ_PIECE;
+    dyn_smem[2u * QR + k] = lev;
+    __threadfence_block();
+    set_vol(dyn_smem[QR + k], min(AQ_PIECE, len - i * AQ_PIECE));
+  }
+  len = 0u;
+  __syncwarp();
 }
 
 // Warp-collective: lanes with ovf set removed a vertex (G^T row start row,
@@ -1461,7 +1651,7 @@ __device__ __noinline__ void async_spill(const Dev& D, Cta& B, bool ovf, uint32_
   uint32_t s = 0;
   if (lane == 0) {
     s = atomicAdd(&D.C->oq_res, tot);
-    B.a_want = 1u;
+    set_vol(B.a_want, 1u);
   }
   s = __shfl_sync(FULL, s, 0);
   // (cannot fail: every removal adds at most ceil(din / kAsyncPiece) pieces)
@@ -1479,174 +1669,276 @@ __device__ __noinline__ void async_spill(const Dev& D, Cta& B, bool ovf, uint32_
   }
 }
 
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+// Warp-collective: the G^T rows (row, len) that the lanes hold, laid end to end
+// with exclusive prefix excl: element lane - at of them (at <= lane < at +
+// total) becomes this lane's push, with its row's level.
+__device__ __forceinline__ void async_take(AsyncWarp& A, uint32_t at, uint32_t total,
+                                           uint32_t excl, uint32_t row, uint32_t lev) {
+  const uint32_t j = lane_id() - at;
+  const unsigned o = owner_of(excl, j);
+  const uint32_t ro = __shfl_sync(FULL, row, o), xo = __shfl_sync(FULL, excl, o);
+  const uint32_t lo = __shfl_sync(FULL, lev, o);
+  if (j < total) {
+    A.p = __ldg(&A.itgt[ro + (j - xo)]);
+    A.l = lo;
+  }
 }
 
-// Warp-collective: lanes with `removed` set removed vertex p with level lev
-// (G^T row start row, in-degree din). The level is written and the
-// predecessors are queued in buffer nxt with that level, all of the warp's
-// rows at once (each lane loads entries of the flattened rows), each
-// predecessor's word and row bounds prefetched into L2 for the step that
-// pushes it; a row longer than AQ_LOCAL_DMAX, or one that does not fit, goes
-// to the global pieces.
-__device__ __forceinline__ void async_append(const Dev& D, Cta& B, bool removed, uint32_t p,
-                                             uint32_t lev, uint32_t row, uint32_t din,
-                                             uint32_t nxt, uint32_t QA) {
-  const unsigned lane = lane_id();
-  const unsigned mask = __ballot_sync(FULL, removed);
-  if (mask == 0u) return;
-  if (removed) D.level[p] = lev;
-  const uint32_t top = __reduce_max_sync(FULL, removed ? lev : 0u);
-  if (lane == 0) {
-    atomicAdd(&B.a_removed, (unsigned)__popc(mask));
-    atomicMax(&B.a_maxlev, top);
+// Warp-collective: lanes in `rows` hold the G^T row of a removed vertex. The
+// first, or with `many` all that fit, join this warp's next batch, of which
+// `total` lanes are taken: their pushes are loaded (A.p, A.l). Returns the lanes
+// whose row is left over. (All of them while the last rebalance's share is
+// unclaimed: the share comes first, so that a warp asked to stop can.)
+__device__ __forceinline__ unsigned async_pick(AsyncWarp& A, unsigned rows, uint32_t row,
+                                               uint32_t len, uint32_t lev, bool many,
+                                               uint32_t& total) {
+  if (A.share) return rows;
+  unsigned left = 0;
+  const uint32_t k0 = lane_id() - total;
+  uint32_t at = 0, sum = 0;
+  while (rows) {  // (seldom more than three rows)
+    const int j = __ffs(rows) - 1;
+    const uint32_t rj = __shfl_sync(FULL, row, j), nj = __shfl_sync(FULL, len, j);
+    const uint32_t vj = __shfl_sync(FULL, lev, j);
+    if (nj <= 32u - total - sum && (many || total + sum == 0u)) {
+      const uint32_t k = k0 - sum;
+      if (k < nj) {
+        at = rj + k;
+        A.l = vj;
+      }
+      sum += nj;
+    } else {
+      left |= 1u << j;
+    }
+    rows &= rows - 1u;
   }
-  const bool want = removed && din > 0u && din <= AQ_LOCAL_DMAX;
-  bool ovf = removed && din > AQ_LOCAL_DMAX;
-  const unsigned wm = __ballot_sync(FULL, want);
-  if (wm) {
-    const unsigned ew = want ? din : 0u;
-    const unsigned eincl = warp_incl_scan(ew);
-    const unsigned esum = __shfl_sync(FULL, eincl, 31);
-    const unsigned excl = eincl - ew;
-    uint32_t be = 0;
-    if (lane == 0) be = atomicAdd(&B.aq_res[nxt], esum);
-    be = __shfl_sync(FULL, be, 0);
-    if ((uint64_t)be + esum <= QA) {  // warp-uniform
-      if (lane == 0) atomicMax(&B.aq_end[nxt], be + esum);
-      uint32_t* ids = dyn_smem + nxt * QA;
-      uint32_t* lv = dyn_smem + (2u + nxt) * QA;
-      for (uint32_t j0 = 0; j0 < esum; j0 += 128u) {
-        uint32_t t[4], l[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t j = j0 + (uint32_t)q * 32u + lane;
-          const unsigned o = owner_of(excl, j);
-          const uint32_t ro = __shfl_sync(FULL, row, o), xo = __shfl_sync(FULL, excl, o);
-          l[q] = __shfl_sync(FULL, lev, o);
-          t[q] = j < esum ? __ldg(&D.itgt[ro + (j - xo)]) : 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t j = j0 + (uint32_t)q * 32u + lane;
-          if (j < esum) {
-            ids[be + j] = t[q];
-            lv[be + j] = l[q];
-            prefetch_l2(&D.aw[t[q]]);  // for the step that pushes it
-            prefetch_l2(&D.ioff[t[q]]);
-          }
-        }
+  if (k0 < sum) A.p = __ldg(&A.itgt[at]);
+  total += sum;
+  return left;
+}
+
+// Warp-collective: rows left over by async_pick go to idle workers, one each,
+// else to the ring, else (rows over AQ_LOCAL_DMAX in-edges at once) to the
+// global pieces. A row of a batch or less is placed by its own lane.
+__device__ __forceinline__ void async_surplus(const Dev& D, Cta& B, unsigned left, uint32_t row,
+                                              uint32_t len, uint32_t lev) {
+  const bool mine = left >> lane_id() & 1u;
+  uint32_t el = mine ? len : 0u;
+  if (mine && el <= 32u) {
+    const uint32_t w = async_claim(B);
+    if (w < 32u) {
+      uint32_t* box = async_mail(w);
+      box[0] = row;
+      box[32] = el;
+      box[64] = lev;
+      async_wake(B, w, 1u);
+      el = 0u;
+    }
+  }
+  __syncwarp();
+  if (!__any_sync(FULL, el != 0u)) return;
+  const bool ovf = el > AQ_LOCAL_DMAX;
+  if (ovf) el = 0u;
+  if (__any_sync(FULL, el > 32u)) async_give(B, row, el, lev);
+  if (__any_sync(FULL, el != 0u)) async_ring(B, row, el, lev);
+  if (__any_sync(FULL, ovf || el != 0u))
+    async_spill(D, B, ovf || el != 0u, row, ovf ? len : el, lev);
+}
+
+// Warp-collective: a worker that found nothing to do adds its counts to the
+// CTA's, sets its idle bit and sleeps until it is claimed; the rows it is given
+// become its batch. (The wait ends: the control warp, whose own waits are
+// bounded, claims every idle worker when it ends the stretch.)
+__device__ __forceinline__ void async_idle(const Dev& D, Cta& B, AsyncWarp& A) {
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  A.top = __reduce_max_sync(FULL, A.top);
+  uint32_t n = 0;
+  if (lane == 0) {
+    if (A.removed) {
+      atomicAdd(&B.a_removed, A.removed);
+      atomicMax(&B.a_maxlev, A.top);
+    }
+    __threadfence_block();
+    atomicOr(&B.a_idle, 1u << warp);
+    __threadfence_block();
+    if (vol(B.a_next) != AS_STEP && (atomicAnd(&B.a_idle, ~(1u << warp)) >> warp & 1u)) {
+      // (claimed itself: the control warp may have passed this bit by)
+    } else {
+      uint32_t done = 0;
+      while (!done) {
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+            " selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(done) : "r"(smem_addr(&B.w_bar[warp])), "r"(A.phase & 1u), "r"(10000u) : "memory");
+        if (!done && vol(B.a_next) == AS_DONE) break;  // (nobody wakes it any more)
+      }
+      if (done) n = vol(B.w_rows[warp]) | 0x80000000u;
+    }
+  }
+  n = __shfl_sync(FULL, n, 0);
+  A.removed = 0u;
+  A.top = 0u;
+  if (n >> 31) A.phase ^= 1u;
+  n &= 0x7FFFFFFFu;
+  if (n) {
+    __threadfence_block();
+    const uint32_t* box = async_mail(warp);
+    const bool in = lane < n;
+    const uint32_t row = in ? box[lane] : 0u, len = in ? box[32u + lane] : 0u;
+    const uint32_t lev = in ? box[64u + lane] : 0u;
+    const uint32_t incl = warp_incl_scan(len);
+    A.cnt = __shfl_sync(FULL, incl, 31);  // (at most 32)
+    async_take(A, 0u, A.cnt, incl - len, row, lev);
+  }
+}
+
+// Warp-collective: fills the batch's free lanes from the piece being worked
+// off; a warp without any work claims a part of the last rebalance's share (32
+// entries, a row or a piece) or a pending work-list entry first.
+__device__ __forceinline__ void async_fill(const Dev& D, Cta& B, AsyncWarp& A, uint32_t nwork) {
+  const unsigned lane = lane_id();
+  if (A.cnt == 0u && A.pl == 0u && A.share) {
+    const size_t par = (size_t)((B.a_gen - 1u) & 1u);
+    uint32_t e = 0, r = 0, q = 0;
+    if (lane == 0) e = atomicAdd(&B.sh_elo, 32u);
+    e = __shfl_sync(FULL, e, 0);
+    if (e < B.sh_ehi) {
+      A.cnt = min(32u, B.sh_ehi - e);
+      if (lane < A.cnt) {
+        A.p = ldcg(&D.ae_id[par * D.ae_cap + e + lane]);
+        A.l = ldcg(&D.ae_lev[par * D.ae_cap + e + lane]);
       }
     } else {
-      ovf = ovf || want;
-    }
-  }
-  if (__ballot_sync(FULL, ovf)) async_spill(D, B, ovf, row, din, lev);
-}
-
-// Warp-collective: pushes from removed vertices to their predecessors p[q]
-// (lanes with valid[q] set), each carrying its removed vertex's level l[q],
-// by compare-and-swap on the predecessors' words; the row bounds of every
-// predecessor load alongside its word, so a removal costs no further
-// dependent load before its row is queued. A word whose counter is zero
-// belongs to a vertex that is not live (masked): it is left alone.
-template <int Q>
-__device__ __forceinline__ void async_push(const Dev& D, Cta& B, const bool (&valid)[Q],
-                                           const uint32_t (&p)[Q], const uint32_t (&l)[Q],
-                                           uint32_t nxt, uint32_t QA, Counters& K) {
-  unsigned long long w[Q];
-  uint32_t p0[Q], p1[Q], lev[Q];
-  bool pend[Q], removed[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    w[q] = valid[q] ? ld_relaxed64(&D.aw[p[q]]) : 0ull;
-    p0[q] = valid[q] ? __ldg(&D.ioff[p[q]]) : 0u;
-    p1[q] = valid[q] ? __ldg(&D.ioff[p[q] + 1u]) : 0u;
-  }
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    pend[q] = valid[q] && (uint32_t)w[q] != 0u;
-    removed[q] = false;
-    lev[q] = 0u;
-    K.pushed += valid[q] ? 1u : 0u;
-  }
-  // a failed compare-and-swap means another push on the same word succeeded,
-  // so the loop ends; the bound only guards against a broken invariant
-  for (uint32_t it = 0;; ++it) {
-    bool any = false;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) any = any || pend[q];
-    if (!__any_sync(FULL, any)) break;
-    if (it == (1u << 22)) {
-      if (lane_id() == 0) set_error(D, TRIM_ERR_TIMEOUT, 6);
-      break;
-    }
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      if (!pend[q]) continue;
-      const uint32_t top = max((uint32_t)(w[q] >> 32), l[q]);
-      const uint32_t cnt = (uint32_t)w[q];
-      const unsigned long long nw = ((unsigned long long)top << 32) | (cnt - 1u);
-      const unsigned long long prev = atomicCAS(&D.aw[p[q]], w[q], nw);
-      if (prev == w[q]) {
-        pend[q] = false;
-        removed[q] = cnt == 1u;
-        lev[q] = top + 1u;
-      } else {
-        w[q] = prev;
-        if ((uint32_t)prev == 0u) pend[q] = false;
+      if (lane == 0) {
+        atomicSub(&B.sh_elo, 32u);  // (the cursor stays near its end)
+        r = atomicAdd(&B.sh_rlo, 1u);
+        q = r < B.sh_rhi ? 0xFFFFFFFFu : atomicAdd(&B.sh_plo, 1u);
+      }
+      r = __shfl_sync(FULL, r, 0);
+      q = __shfl_sync(FULL, q, 0);
+      if (r < B.sh_rhi) {
+        A.pr = ldcg(&D.er_row[par * D.er_cap + r]);
+        A.pl = ldcg(&D.er_len[par * D.er_cap + r]);
+        A.pv = ldcg(&D.er_lev[par * D.er_cap + r]);
+      } else if (q < B.sh_phi) {
+        A.pr = ldcg(&D.oq_row[q]);
+        A.pl = ldcg(&D.oq_len[q]);
+        A.pv = ldcg(&D.oq_lev[q]);
+      } else if (A.wj < B.S.w_end) {
+        const uint32_t eo = ldcg(&D.w4_eoff[A.wj]);
+        const uint32_t ee = (A.wj + 1u < B.S.w_end) ? ldcg(&D.w4_eoff[A.wj + 1u]) : B.S.e_end;
+        A.pr = ldcg(&D.w4_row[A.wj]);
+        A.pl = ee - eo;
+        A.pv = B.S.round - 1u;
+        A.wj += nwork;
       }
     }
+    // what no warp has claimed yet (a claimed part is its warp's to finish)
+    A.share = vol(B.sh_elo) < B.sh_ehi || vol(B.sh_rlo) < B.sh_rhi || vol(B.sh_plo) < B.sh_phi ||
+              A.wj < B.S.w_end;
+    A.share = __any_sync(FULL, A.share);
   }
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-    async_append(D, B, removed[q], p[q], lev[q], p0[q], p1[q] - p0[q], nxt, QA);
+  if (A.pl != 0u && A.cnt < 32u) {
+    const uint32_t k = min(32u - A.cnt, A.pl), j = lane - A.cnt;
+    if (j < k) {
+      A.p = __ldg(&A.itgt[A.pr + j]);
+      A.l = A.pv;
+    }
+    A.pr += k;
+    A.pl -= k;
+    A.cnt += k;
+  }
 }
 
-// Warp-collective: pushes the in-edges [row, row + len) of G^T, all carrying level l.
-__device__ __forceinline__ void async_piece(const Dev& D, Cta& B, uint32_t row, uint32_t len,
-                                            uint32_t l, uint32_t nxt, uint32_t QA,
-                                            Counters& K) {
+// Warp-collective: one batch. The compare-and-swaps are issued before the rows
+// of the vertices they should remove are loaded, and checked after: the row
+// accesses do not wait for them. A word whose counter is zero belongs to a
+// vertex that is not live (masked): it is left alone.
+__device__ __forceinline__ void async_batch(const Dev& D, Cta& B, AsyncWarp& A, Counters& K) {
   const unsigned lane = lane_id();
-  for (uint32_t k0 = 0; k0 < len; k0 += 64u) {
-    bool valid[2];
-    uint32_t p[2], lv[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t e = k0 + (uint32_t)q * 32u + lane;
-      valid[q] = e < len;
-      p[q] = valid[q] ? __ldg(&D.itgt[row + e]) : 0u;
-      lv[q] = l;
+  const bool valid = lane < A.cnt;
+  const uint32_t p = A.p, l = A.l;
+  ulonglong2 a = make_ulonglong2(0ull, 0ull);
+  if (valid) a = ld_relaxed_v2(&A.aw[p]);
+  unsigned long long* word = reinterpret_cast<unsigned long long*>(&A.aw[p]);
+  const uint32_t cnt = (uint32_t)a.x, row = (uint32_t)a.y, len = (uint32_t)(a.y >> 32);
+  const bool live = valid && cnt != 0u;
+  uint32_t lev = max((uint32_t)(a.x >> 32), l);
+  K.pushed += valid ? 1u : 0u;
+  unsigned long long prev = a.x;
+  if (live) prev = atomicCAS(word, a.x, ((unsigned long long)lev << 32) | (cnt - 1u));
+  uint32_t total = 0;
+  const unsigned seen = __ballot_sync(FULL, live && cnt == 1u && len != 0u);
+  // One row per batch: a warp that keeps several is slower (it waits for the
+  // latest of more accesses), and every level waits for the slowest. Only where
+  // rows pile up in the ring (more than there are warps for) are batches filled.
+  const bool many = (seen & (seen - 1u)) != 0u &&
+                    __shfl_sync(FULL, vol(B.r_tail) - vol(B.r_head), 0) >= (blockDim.x >> 5);
+  unsigned left = async_pick(A, seen, row, len, lev + 1u, many, total);
+  bool pend = live && prev != a.x;
+  bool removed = live && !pend && cnt == 1u;
+  const bool clean = !__any_sync(FULL, pend);
+  if (!clean) {
+    // a failed compare-and-swap means another push on the same word succeeded,
+    // so the loop ends; the bound only guards against a broken invariant
+    for (uint32_t it = 0; pend; ++it) {
+      const unsigned long long w = prev;
+      if ((uint32_t)w == 0u) break;
+      if (it == (1u << 22)) {
+        set_error(D, TRIM_ERR_TIMEOUT, 6);
+        break;
+      }
+      lev = max((uint32_t)(w >> 32), l);
+      prev = atomicCAS(word, w, ((unsigned long long)lev << 32) | ((uint32_t)w - 1u));
+      if (prev == w) {
+        removed = (uint32_t)w == 1u;
+        pend = false;
+      }
     }
-    async_push<2>(D, B, valid, p, lv, nxt, QA, K);
+    __syncwarp();
+  }
+  const unsigned rm = __ballot_sync(FULL, removed);
+  if (!clean) {
+    // not all as foreseen: rows of vertices that another push removed leave the
+    // batch, rows of vertices removed after all join it
+    const unsigned rows = __ballot_sync(FULL, removed && len != 0u);
+    if (seen & ~rows) {
+      total = 0u;
+      left = async_pick(A, rows, row, len, lev + 1u, many, total);
+    } else if (rows & ~seen) {
+      left |= async_pick(A, rows & ~seen, row, len, lev + 1u, many, total);
+    }
+  }
+  if (rm) {
+    if (removed) {
+      A.level[p] = lev + 1u;
+      A.top = max(A.top, lev + 1u);
+    }
+    A.removed += __popc(rm);
+  }
+  A.cnt = total;
+  if (left) async_surplus(D, B, left, row, len, lev + 1u);
+}
+
+// A worker warp: batches until the control warp ends the stretch (and the last
+// rebalance's share is claimed).
+__device__ __forceinline__ void async_work(const Dev& D, Cta& B, AsyncWarp& A, uint32_t nwork,
+                                           Counters& K) {
+  while (true) {
+    const uint32_t next = warp_vol(B.a_next);
+    if (next == AS_DONE || (next != AS_STEP && !A.share)) break;
+    async_fill(D, B, A, nwork);
+    if (A.cnt == 0u) {
+      if (!A.share) async_idle(D, B, A);
+      continue;
+    }
+    async_batch(D, B, A, K);
+    if (lane_id() == 0) set_vol(B.a_prog, (uint32_t)clock());  // (shows that this CTA goes on)
   }
 }
 
-// All threads: pushes the entries [lo, hi) of a list of (predecessor, level)
-// pairs, two per thread at a time (warps past the end skip the pass).
-__device__ __forceinline__ void async_entries(const Dev& D, Cta& B, const uint32_t* ids,
-                                              const uint32_t* lv, uint32_t lo, uint32_t hi,
-                                              bool global, uint32_t nxt, uint32_t QA,
-                                              Counters& K) {
-  for (uint32_t base = lo; base < hi; base += 2u * blockDim.x) {  // CTA-uniform
-    if (base + (threadIdx.x & ~31u) >= hi) break;  // (warp-uniform: later bases are larger)
-    bool valid[2];
-    uint32_t p[2], l[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t k = base + (uint32_t)q * blockDim.x + threadIdx.x;
-      valid[q] = k < hi;
-      p[q] = valid[q] ? (global ? ldcg(&ids[k]) : ids[k]) : 0u;
-      l[q] = valid[q] ? (global ? ldcg(&lv[k]) : lv[k]) : 0u;
-    }
-    async_push<2>(D, B, valid, p, l, nxt, QA, K);
-  }
-}
-
-constexpr uint32_t AS_STEP = 0, AS_DONE = 1, AS_REBALANCE = 2;
-
-// Thread 0: releases this CTA's token, after publishing its removals and top
+// One thread: releases this CTA's token, after publishing its removals and top
 // level (CTA 0 reads the totals once the token count is zero).
 __device__ __forceinline__ void async_release(const Dev& D, Cta& B) {
   Ctrl* C = D.C;
@@ -1661,130 +1953,274 @@ __device__ __forceinline__ void async_release(const Dev& D, Cta& B) {
   B.a_token = 0u;
 }
 
-// Thread 0, before each step: buffer cur holds the predecessors the next step
-// pushes. A CTA with work asks for a rebalance when its removals did not fit
-// its queue or its queue holds more than max(half its threads, 2 x the
-// average share at the last rebalance): steps stay short (a step takes as long
-// as its CTA's slowest chain of loads, and one push per thread or less keeps
-// that to a single pass), and joins one when the hints (the requested
-// generation and the error flag, loaded during the previous step) show one. A
-// CTA without work publishes its counts, releases its token, and waits until
-// a rebalance is asked for or the token count is zero (the run is over). The
-// wait is bounded: spin_limit_ns without a heartbeat from a working CTA
-// (every 256 of its steps) ends the run with TRIM_ERR_TIMEOUT.
-__device__ void async_decide(const Dev& D, Cta& B, uint32_t cur, uint32_t h_req,
-                             uint32_t h_err) {
+// Rows on their way to another CTA travel on channels: lane i of a control warp
+// sends to the CTA async_offset(i) further on, one row at a time, and receives
+// from the one as far back. A channel is a 16-byte message in the receiver's
+// line (row start, length and a tag; level and the tag again: each 64-bit half
+// says by itself whether it has arrived, so no fence is needed) and the tag it
+// acknowledged in the sender's line.
+__device__ __forceinline__ uint32_t async_offset(uint32_t i) {
+  return gridDim.x > 32u ? 1u + i * ((gridDim.x - 1u) / 32u) : i + 1u;
+}
+struct AsyncChannel {
+  uint32_t to, from;      // CTAs (to == this one: no channel)
+  uint32_t sent, taken;   // tags of the last message sent and received
+};
+
+// The control warp: receives and dispatches rows, and watches until the stretch
+// ends, then sets a_next and wakes the idle workers.
+// Rows that arrive go to idle workers or the ring. Pieces in the ring go to
+// idle workers, and where there are none to CTAs that have some. Rows in the global pieces, or a
+// ring half full, ask for a rebalance. A CTA without work and
+// with every row it sent acknowledged publishes its counts, releases its token,
+// and waits until rows arrive, a rebalance is asked for or
+// the token count is zero (the run is over). Every wait is bounded:
+// spin_limit_ns without a heartbeat from a working CTA (or, with work, without
+// a batch of its own workers) ends the run with TRIM_ERR_TIMEOUT.
+__device__ __noinline__ void async_control(const Dev& D, Cta& B) {
   Ctrl* C = D.C;
-  B.aq_res[cur ^ 1u] = 0u;  // read by the previous step: the next one fills it
-  B.aq_end[cur ^ 1u] = 0u;
-  B.sh_elo = B.sh_ehi = B.sh_plo = B.sh_phi = 0u;  // the last rebalance's share is pushed
-  B.a_next = AS_STEP;
-  const uint32_t qe = B.aq_end[cur];
-  const bool over = qe > max(blockDim.x / 2u, 2u * B.a_avg);
-  if (qe != 0u || B.a_want) {
-    if ((++B.a_steps & 255u) == 0u) red_relaxed_add(&C->a_beat, 1u);
-    if (h_err != 0u) {
-      B.err = h_err;
-      B.a_next = AS_DONE;
-    } else if (B.a_want || over) {
-      atomicMax(&C->a_req, B.a_gen + 1u);
-      B.a_next = AS_REBALANCE;
-    } else if ((int)(h_req - B.a_gen) > 0) {
-      B.a_next = AS_REBALANCE;
+  const unsigned lane = lane_id();
+  const uint32_t QR = async_ring_cap(), nwk = (blockDim.x >> 5) - 1u, all = (1u << nwk) - 1u;
+  const uint32_t G = gridDim.x, off = async_offset(lane);
+  AsyncChannel ch;
+  ch.to = off < G ? (blockIdx.x + off) % G : blockIdx.x;
+  ch.from = off < G ? (blockIdx.x + G - off) % G : blockIdx.x;
+  ch.sent = B.ch_sent[lane];
+  ch.taken = B.ch_taken[lane];
+  const ulonglong2* in = &D.ch_msg[32u * blockIdx.x + lane];
+  uint64_t t0 = globaltimer(), tb = t0;
+  uint32_t beat = ld_relaxed(&C->a_beat), prog = vol(B.a_prog), next = AS_STEP;
+  uint32_t load = 0xFFFFFFFFu;
+  for (uint32_t turn = 0; next == AS_STEP; ++turn) {
+    // everything this turn looks at, under way together
+    unsigned long long m0, m1;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(m0), "=l"(m1) : "l"(in) : "memory");
+    const uint32_t ack = ld_relaxed(&D.ch_ack[32u * blockIdx.x + lane]);
+    const bool watch = (turn & 3u) == 0u || __shfl_sync(FULL, B.a_token, 0) == 0u;
+    uint32_t err = 0, req = 0, tok = 0, bt = 0;
+    if (watch && lane == 0) {
+      err = ld_relaxed(&C->err);
+      req = ld_relaxed(&C->a_req);
+      tok = ld_relaxed(&C->a_tokens);
+      bt = ld_relaxed(&C->a_beat);
     }
-    return;
+    // rows that arrived
+    const uint32_t tag = ch.taken + 1u;
+    const bool here = (uint32_t)(m1 >> 32) == tag && (uint32_t)(m0 >> 40) == (tag & 0xFFFFFFu);
+    const unsigned hm = __ballot_sync(FULL, here);
+    if (hm) {
+      uint32_t row = (uint32_t)m0, len = here ? (uint32_t)(m0 >> 32) & 0xFFu : 0u;
+      const uint32_t lev = (uint32_t)m1;
+      async_give(B, row, len, lev);
+      if (__any_sync(FULL, len != 0u)) async_ring(B, row, len, lev);
+      // (a row that even the ring has no room for stays where it is)
+      const bool took = here && len == 0u;
+      // a CTA without a token takes one before it acknowledges: until then the
+      // sender's covers the row
+      uint32_t tokens = 1u;
+      if (lane == 0 && B.a_token == 0u) {
+        B.a_token = 1u;
+        tokens = atomicAdd(&C->a_tokens, 1u);
+      }
+      tokens = __shfl_sync(FULL, tokens, 0);
+      if (took && tokens != 0u) {  // (0: never, the sender holds one; the test waits for the addition)
+        ch.taken = tag;
+        st_relaxed(&D.ch_ack[32u * ch.from + lane], tag);
+      }
+      __syncwarp();
+    }
+    // pieces in the ring (all workers idle before it is seen empty: then
+    // nothing but this warp adds to it, and there is no work at all)
+    const uint32_t mask = warp_vol(B.a_idle);
+    __threadfence_block();
+    const uint32_t head = __shfl_sync(FULL, B.r_head, 0), rows = warp_vol(B.r_tail) - head;
+    const bool idle = mask == all && rows == 0u && !__any_sync(FULL, ack != ch.sent);
+    const uint32_t now_load = nwk - __popc(mask) + min(rows, 255u);
+    if (now_load != load) {
+      load = now_load;
+      if (lane == 0) st_relaxed(&D.ch_load[blockIdx.x], load);
+    }
+    if (rows != 0u) {
+      const uint32_t k = (head + lane) & (QR - 1u);
+      uint32_t len = vol(dyn_smem[QR + k]);  // (0: not there yet)
+      const unsigned rm = __ballot_sync(FULL, len != 0u);
+      const uint32_t n = rm == FULL ? 32u : (uint32_t)__ffs(~rm) - 1u;  // leading pieces
+      if (n) {
+        __threadfence_block();
+        if (lane >= n) len = 0u;
+        uint32_t row = dyn_smem[k];
+        const uint32_t lev = dyn_smem[2u * QR + k];
+        async_give(B, row, len, lev);
+        const unsigned left = __ballot_sync(FULL, len != 0u);
+        uint32_t done = left ? (uint32_t)__ffs(left) - 1u : n;
+        if (left && rows > 1u) {  // (a single row waits for a worker here)
+          // the i-th lane whose channel is free and leads to idle workers
+          // sends the i-th piece left; nearly idle CTAs first
+          const uint32_t their = ld_relaxed(&D.ch_load[ch.to]);
+          const bool can = ch.to != blockIdx.x && ack == ch.sent && their < nwk;
+          const unsigned lo = __ballot_sync(FULL, can && their <= nwk / 2u);
+          const unsigned cm = lo ? lo : __ballot_sync(FULL, can);
+          const uint32_t from = done + __popc(cm & ((1u << lane) - 1u));
+          const bool send = (cm >> lane & 1u) && from < n;
+          const uint32_t sr = __shfl_sync(FULL, row, from & 31u), sv = __shfl_sync(FULL, lev, from & 31u);
+          const uint32_t sl = __shfl_sync(FULL, len, from & 31u);
+          const uint32_t ns = __popc(__ballot_sync(FULL, send));
+          if (send) {
+            ch.sent += 1u;
+            const unsigned long long s0 = (unsigned long long)sr | ((unsigned long long)sl << 32) |
+                                          ((unsigned long long)(ch.sent & 0xFFFFFFu) << 40);
+            const unsigned long long s1 = (unsigned long long)sv | ((unsigned long long)ch.sent << 32);
+            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&D.ch_msg[32u * ch.to + lane]),
+                         "l"(s0), "l"(s1) : "memory");
+          }
+          done += ns;
+        }
+        if (lane < done) set_vol(dyn_smem[QR + k], 0u);
+        __threadfence_block();
+        __syncwarp();
+        if (lane == 0) set_vol(B.r_head, head + done);
+      }
+    }
+    __syncwarp();
+    if (lane == 0 && (watch || idle)) {
+      const uint64_t now = globaltimer();
+      const uint32_t pr = vol(B.a_prog);
+      if (err != 0u) {
+        B.err = err;
+        next = AS_DONE;
+      } else if (vol(B.a_want) || rows > QR / 2u) {
+        atomicMax(&C->a_req, B.a_gen + 1u);
+        next = AS_REBALANCE;
+      } else if (watch && (int)(req - B.a_gen) > 0) {
+        next = AS_REBALANCE;
+      } else if (B.a_token) {
+        if (idle) {
+          async_release(D, B);
+          t0 = now;
+        } else if (pr != prog) {
+          prog = pr;
+          t0 = now;
+          if (now - tb > 100000u) {  // a heartbeat every 100 us
+            tb = now;
+            red_relaxed_add(&C->a_beat, 1u);
+          }
+        }
+      } else if (watch && tok == 0u) {
+        // (a CTA that asks for a rebalance holds its token until the
+        // rebalance, so a zero count means no rebalance can come)
+        next = AS_DONE;
+      } else if (watch && bt != beat) {
+        beat = bt;
+        t0 = now;
+      }
+      if (next == AS_STEP && now > t0 && now - t0 > D.spin_limit_ns) {
+        set_error(D, TRIM_ERR_TIMEOUT, 4);
+        B.err = TRIM_ERR_TIMEOUT;
+        next = AS_DONE;
+      }
+    }
+    next = __shfl_sync(FULL, next, 0);
+    // (polls and sends take from the workers: 6.7 ms on the deep cascade with
+    // 1,600 ns and two rows, 9.2 with 200 ns and two, 10.6 with 200 ns and one)
+    if (next == AS_STEP) __nanosleep(1600);
   }
-  if (B.a_token) async_release(D, B);
-  uint64_t t0 = globaltimer();
-  uint32_t beat = ld_relaxed(&C->a_beat);
-  while (true) {
-    const uint32_t err = ld_relaxed(&C->err);
-    const uint32_t req = ld_relaxed(&C->a_req);
-    const uint32_t tok = ld_relaxed(&C->a_tokens);
-    const uint32_t bt = ld_relaxed(&C->a_beat);
-    if (err != 0u) {
-      B.err = err;
-      B.a_next = AS_DONE;
-      return;
-    }
-    if ((int)(req - B.a_gen) > 0) {
-      B.a_next = AS_REBALANCE;
-      return;
-    }
-    // (a CTA that asks for a rebalance holds its token until the rebalance,
-    // so a zero count means no rebalance can come)
-    if (tok == 0u) {
-      B.a_next = AS_DONE;
-      return;
-    }
-    const uint64_t now = globaltimer();
-    if (bt != beat) {
-      beat = bt;
-      t0 = now;
-    } else if (now - t0 > D.spin_limit_ns) {
-      set_error(D, TRIM_ERR_TIMEOUT, 4);
-      B.err = TRIM_ERR_TIMEOUT;
-      B.a_next = AS_DONE;
-      return;
-    }
-    __nanosleep(256);
+  B.ch_sent[lane] = ch.sent;
+  B.ch_taken[lane] = ch.taken;
+  __syncwarp();
+  if (lane == 0) {
+    set_vol(B.a_next, next);
+    __threadfence_block();
+    // (a worker that sets its bit after this sees a_next and does not sleep)
+    for (uint32_t w = async_claim(B); w < 32u; w = async_claim(B)) async_wake(B, w, 0u);
   }
+  __syncwarp();
 }
 
-// All threads, every CTA (generation g = B.a_gen): writes the entries of
-// buffer cur to the global entry list of parity g & 1; after a grid barrier
-// every CTA takes an even slice of those entries and of the pieces written
-// since the last rebalance; tokens follow the new shares and CTA 0 clears the
-// other parity's list (last read after rebalance g - 1, by every CTA before
-// this rebalance's first barrier); a second barrier publishes both before any
-// CTA writes to the lists again. Returns false on an error.
-__device__ __noinline__ bool async_rebalance(const Dev& D, Cta& B, uint32_t cur, uint32_t QA) {
+// All threads, every CTA (generation g = B.a_gen): writes the workers' entries
+// and pieces and the ring's pieces to the global lists of parity g & 1; after
+// a grid barrier every CTA takes an even slice of those and of the pieces
+// written since the last rebalance; tokens follow the new shares and CTA 0
+// clears the other parity's counters (last read after rebalance g - 1, by every
+// CTA before this rebalance's first barrier); a second barrier publishes both
+// before any CTA writes to the lists again. Returns false on an error.
+__device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp& A) {
   Ctrl* C = D.C;
+  const unsigned lane = lane_id();
   const uint32_t par = B.a_gen & 1u;
-  const uint32_t qe = B.aq_end[cur];
-  uint32_t* eid = D.ae_id + (size_t)par * D.ae_cap;
-  uint32_t* elv = D.ae_lev + (size_t)par * D.ae_cap;
-  if (threadIdx.x == 0) {
-    B.a_base = qe ? atomicAdd(&C->e_n[par], qe) : 0u;
-    // (cannot fail: a list holds every CTA's whole queue)
-    if ((uint64_t)B.a_base + qe > D.ae_cap) set_error(D, TRIM_ERR_STATE, 7);
-  }
-  __syncthreads();
-  const uint32_t base = B.a_base;
-  if ((uint64_t)base + qe <= D.ae_cap) {
-    const uint32_t* ids = dyn_smem + cur * QA;
-    const uint32_t* lv = dyn_smem + (2u + cur) * QA;
-    for (uint32_t k = threadIdx.x; k < qe; k += blockDim.x) {
-      eid[base + k] = ids[k];
-      elv[base + k] = lv[k];
+  const uint32_t QR = async_ring_cap();
+  uint32_t eo = 0, ro = 0;
+  A.top = __reduce_max_sync(FULL, A.top);
+  if (lane == 0) {
+    if (A.cnt) eo = atomicAdd(&B.a_ne, A.cnt);
+    if (A.pl) ro = atomicAdd(&B.a_nr, 1u);
+    if (A.removed) {
+      atomicAdd(&B.a_removed, A.removed);
+      atomicMax(&B.a_maxlev, A.top);
     }
   }
+  eo = __shfl_sync(FULL, eo, 0);
+  A.removed = 0u;
+  A.top = 0u;
+  __syncthreads();
+  const uint32_t head = B.r_head, nring = B.r_tail - head, ne = B.a_ne, nr = B.a_nr + nring;
+  if (threadIdx.x == 0) {
+    B.a_ebase = ne ? atomicAdd(&C->e_n[par], ne) : 0u;
+    B.a_rbase = nr ? atomicAdd(&C->er_n[par], nr) : 0u;
+    // (cannot fail: the lists hold what every CTA can hold)
+    if ((uint64_t)B.a_ebase + ne > D.ae_cap || (uint64_t)B.a_rbase + nr > D.er_cap)
+      set_error(D, TRIM_ERR_STATE, 7);
+  }
+  __syncthreads();
+  if ((uint64_t)B.a_ebase + ne <= D.ae_cap && (uint64_t)B.a_rbase + nr <= D.er_cap) {
+    const size_t e0 = (size_t)par * D.ae_cap + B.a_ebase, r0 = (size_t)par * D.er_cap + B.a_rbase;
+    if (lane < A.cnt) {
+      D.ae_id[e0 + eo + lane] = A.p;
+      D.ae_lev[e0 + eo + lane] = A.l;
+    }
+    for (uint32_t i = threadIdx.x; i < nring; i += blockDim.x) {
+      const uint32_t k = (head + i) & (QR - 1u);
+      D.er_row[r0 + i] = dyn_smem[k];
+      D.er_len[r0 + i] = dyn_smem[QR + k];
+      D.er_lev[r0 + i] = dyn_smem[2u * QR + k];
+      dyn_smem[QR + k] = 0u;
+    }
+    if (lane == 0 && A.pl) {
+      D.er_row[r0 + nring + ro] = A.pr;
+      D.er_len[r0 + nring + ro] = A.pl;
+      D.er_lev[r0 + nring + ro] = A.pv;
+    }
+  }
+  A.cnt = 0u;
+  A.pl = 0u;
+  A.share = true;
   if (!grid_barrier(D, B)) return false;
   if (threadIdx.x == 0) {
     const uint64_t G = gridDim.x, b = blockIdx.x;
-    const uint64_t tE = ld_relaxed(&C->e_n[par]);
+    const uint64_t tE = ld_relaxed(&C->e_n[par]), tR = ld_relaxed(&C->er_n[par]);
     const uint32_t p_hi = ld_relaxed(&C->oq_res);
     const uint64_t tP = p_hi - B.a_plo;
     B.sh_elo = (uint32_t)(b * tE / G);
     B.sh_ehi = (uint32_t)((b + 1u) * tE / G);
+    B.sh_rlo = (uint32_t)(b * tR / G);
+    B.sh_rhi = (uint32_t)((b + 1u) * tR / G);
     B.sh_plo = B.a_plo + (uint32_t)(b * tP / G);
     B.sh_phi = B.a_plo + (uint32_t)((b + 1u) * tP / G);
     B.a_plo = p_hi;
-    const uint64_t avg = (tE + tP * kAsyncPiece) / G;
-    B.a_avg = avg < (1u << 24) ? (uint32_t)avg : (1u << 24);
-    B.aq_res[cur] = 0u;  // the queue went to the list
-    B.aq_end[cur] = 0u;
+    B.r_head = B.r_tail;  // the ring went to the list
+    B.a_ne = 0u;
+    B.a_nr = 0u;
     B.a_want = 0u;
     B.a_gen += 1u;
-    const uint32_t busy = (B.sh_ehi > B.sh_elo || B.sh_phi > B.sh_plo) ? 1u : 0u;
+    B.a_next = AS_STEP;
+    const bool busy = B.sh_ehi > B.sh_elo || B.sh_rhi > B.sh_rlo || B.sh_phi > B.sh_plo;
+    // (a CTA left without work releases its token later, if it may)
     if (busy && !B.a_token) {
       atomicAdd(&C->a_tokens, 1u);
       B.a_token = 1u;
-    } else if (!busy && B.a_token) {
-      async_release(D, B);
     }
     if (blockIdx.x == 0) {
       C->e_n[par ^ 1u] = 0u;
+      C->er_n[par ^ 1u] = 0u;
       C->a_rebalances = B.a_gen;
     }
   }
@@ -1792,86 +2228,85 @@ __device__ __noinline__ bool async_rebalance(const Dev& D, Cta& B, uint32_t cur,
 }
 
 // Runs the rest of the run asynchronously from round B.S.round = r0 (all
-// threads): every vertex's word is set from its counter, the pending
-// work-list entries (level r0 - 1) are pushed, one per warp, and then the
-// CTA runs steps (and rebalances) until the token count is zero. CTA 0 then
-// publishes the run's totals: alpha = top level + 1 (r0 if the tail removed
-// nothing), and one AC-4 round for each of rounds r0 .. alpha. Returns false
-// on an error.
+// threads): every vertex's record is set from its counter and its G^T row, and
+// the workers push the pending work-list entries (level r0 - 1) and what
+// follows from them until the token count is zero. CTA 0 then publishes the
+// run's totals: alpha = top level + 1 (r0 if the tail removed nothing), and
+// one AC-4 round for each of rounds r0 .. alpha. Returns false on an error.
 __device__ __noinline__ bool async_tail(const Dev& D, Cta& B) {
   Counters K;
   Ctrl* C = D.C;
-  const unsigned warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint32_t QA = nw * D.sbuf_cap;  // entries per buffer: the four slices' space
-  const uint32_t r0 = B.S.round;
+  const unsigned warp = threadIdx.x >> 5, nwk = (blockDim.x >> 5) - 1u;  // the last warp controls
+  const uint32_t r0 = B.S.round, nwork = gridDim.x * nwk;
   {
-    // four counters per 16-byte load where both arrays allow it
-    const bool vec = ((reinterpret_cast<uintptr_t>(D.cnt) | reinterpret_cast<uintptr_t>(D.aw)) & 15u) == 0u;
-    const uint32_t n4 = vec ? D.n >> 2 : 0u, stride = gridDim.x * blockDim.x;
-    const uint4* c4 = reinterpret_cast<const uint4*>(D.cnt);
-    ulonglong2* w2 = reinterpret_cast<ulonglong2*>(D.aw);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-      const uint4 c = __ldcg(&c4[i]);
-      w2[2u * i] = make_ulonglong2(c.x, c.y);
-      w2[2u * i + 1u] = make_ulonglong2(c.z, c.w);
+    constexpr int U = 4;  // records in flight per thread
+    const uint32_t stride = gridDim.x * blockDim.x;
+    for (uint32_t v0 = blockIdx.x * blockDim.x + threadIdx.x; v0 < D.n; v0 += U * stride) {
+      uint32_t c[U], s[U], e[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const uint64_t v = (uint64_t)v0 + (uint64_t)q * stride;
+        const bool has = v < D.n;
+        c[q] = has ? ldcg(&D.cnt[v]) : 0u;
+        s[q] = has ? __ldg(&D.ioff[v]) : 0u;
+        e[q] = has ? __ldg(&D.ioff[v + 1u]) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const uint64_t v = (uint64_t)v0 + (uint64_t)q * stride;
+        if (v < D.n) D.aw[v] = make_uint4(c[q], 0u, s[q], e[q] - s[q]);
+      }
     }
-    for (uint32_t v = (n4 << 2) + blockIdx.x * blockDim.x + threadIdx.x; v < D.n; v += stride)
-      D.aw[v] = (unsigned long long)ldcg(&D.cnt[v]);
+  }
+  for (uint32_t i = threadIdx.x; i < async_ring_cap(); i += blockDim.x)
+    dyn_smem[async_ring_cap() + i] = 0u;
+  if (threadIdx.x < 32u) {
+    B.ch_sent[threadIdx.x] = B.ch_taken[threadIdx.x] = 0u;
+    D.ch_msg[32u * blockIdx.x + threadIdx.x] = make_ulonglong2(0ull, 0ull);
+    D.ch_ack[32u * blockIdx.x + threadIdx.x] = 0u;
   }
   if (threadIdx.x == 0) {
-    B.aq_res[0] = B.aq_res[1] = 0u;
-    B.aq_end[0] = B.aq_end[1] = 0u;
-    B.sh_elo = B.sh_ehi = B.sh_plo = B.sh_phi = 0u;
+    B.r_head = B.r_tail = 0u;
+    B.a_idle = 0u;
+    for (uint32_t w = 0; w < MAX_WARPS; ++w)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&B.w_bar[w])) : "memory");
+    B.a_next = AS_STEP;
+    B.sh_elo = B.sh_ehi = B.sh_rlo = B.sh_rhi = B.sh_plo = B.sh_phi = 0u;
     B.a_removed = 0u;
     B.a_maxlev = 0u;
+    B.a_ne = B.a_nr = 0u;
     B.a_token = 1u;
-    B.a_steps = 0u;
     B.a_want = 0u;
     B.a_gen = 0u;
     B.a_plo = 0u;
-    B.a_avg = (B.S.e_end - B.S.e_c4) / gridDim.x;
+    B.a_prog = 0u;
+    D.ch_load[blockIdx.x] = nwk;
     if (blockIdx.x == 0) {
       C->a_tokens = gridDim.x;
       C->a_round = r0;
     }
   }
   if (!grid_barrier(D, B, false)) return false;
-  {
-    const uint32_t ia = B.S.c4w, ib = B.S.w_end, eb = B.S.e_end;
-    for (uint32_t j = ia + warp * gridDim.x + blockIdx.x; j < ib; j += gridDim.x * nw) {
-      const uint32_t row = ldcg(&D.w4_row[j]);
-      const uint32_t eo = ldcg(&D.w4_eoff[j]);
-      const uint32_t ee = (j + 1u < ib) ? ldcg(&D.w4_eoff[j + 1u]) : eb;
-      async_piece(D, B, row, ee - eo, r0 - 1u, 0u, QA, K);
-    }
-  }
-  uint32_t cur = 0, h_req = 0, h_err = 0;
+  AsyncWarp A;
+  A.aw = D.aw;
+  A.itgt = D.itgt;
+  A.level = D.level;
+  A.p = A.l = A.cnt = 0u;
+  A.pr = A.pl = A.pv = 0u;
+  A.wj = warp < nwk ? B.S.c4w + warp * gridDim.x + blockIdx.x : B.S.w_end;
+  A.removed = A.top = 0u;
+  A.phase = 0u;
+  A.share = true;
   bool ok = true;
   while (true) {
+    if (warp < nwk) async_work(D, B, A, nwork, K);
+    else async_control(D, B);
     __syncthreads();
-    if (threadIdx.x == 0) async_decide(D, B, cur, h_req, h_err);
-    __syncthreads();
-    const uint32_t next = B.a_next;
-    if (next == AS_DONE) break;
-    if (next == AS_REBALANCE && !async_rebalance(D, B, cur, QA)) {
+    if (B.a_next == AS_DONE) break;
+    if (!async_rebalance(D, B, A)) {
       ok = false;
       break;
     }
-    if (threadIdx.x == 0) {  // hints for the next decision, in flight during the step
-      h_req = ld_relaxed(&C->a_req);
-      h_err = ld_relaxed(&C->err);
-    }
-    const uint32_t nxt = cur ^ 1u;
-    // a rebalance's share: entries of the global list, then pieces (one per warp)
-    if (B.sh_ehi > B.sh_elo) {
-      const size_t o = (size_t)((B.a_gen - 1u) & 1u) * D.ae_cap;
-      async_entries(D, B, D.ae_id + o, D.ae_lev + o, B.sh_elo, B.sh_ehi, true, nxt, QA, K);
-    }
-    for (uint32_t i = B.sh_plo + warp; i < B.sh_phi; i += nw)
-      async_piece(D, B, ldcg(&D.oq_row[i]), ldcg(&D.oq_len[i]), ldcg(&D.oq_lev[i]), nxt, QA, K);
-    async_entries(D, B, dyn_smem + cur * QA, dyn_smem + (2u + cur) * QA, 0u, B.aq_end[cur],
-                  false, nxt, QA, K);
-    cur = nxt;
   }
   stats_flush(D, B, K);
   if (threadIdx.x == 0) {

@@ -143,7 +143,6 @@ extern "C" trim_err_t trim_run_ac4_noalloc(const uint32_t* offsets, const uint32
   D.C = reinterpret_cast<trimk::Ctrl*>(base);
   D.mode = TRIM_AC4_PUSH;
   D.flags = trimk::F_AC4_POSSIBLE;
-  D.sbuf_cap = kSliceEntries;
   D.spin_limit_ns = 5ull * 1000 * 1000 * 1000;
   D.heur_push_ratio = 1.0f;
   D.heur_ac6_ratio = 1.0f;
