@@ -1,19 +1,37 @@
-// trim_scc.cu -- kernels of the SCC decomposition that trimming feeds
-// (Section 1: FW-BW with trimming, as in ISPAN): size-2 SCC trimming and the
-// steps of a colour-partitioned forward-backward search. The host driver is
-// trim_run_scc in trim_api.cu; size-1 SCCs come from in+out trimming.
+// trim_scc.cu -- the SCC decomposition that trimming feeds (Section 1: FW-BW
+// with trimming, as in ISPAN), in one cooperative launch behind the in+out
+// trimming that finds the size-1 components: size-2 trimming, trimming passes,
+// and forward-backward steps until no vertex is open. The host driver is
+// trim_run_scc in trim_api.cu.
 //
 // State: comp[v] = the smallest vertex id of v's component once known, else
-// SCC_OPEN. A step works on every open vertex at once: its forward part labels
-// each open vertex with the smallest open vertex that reaches it (label
-// propagation along G, i.e. forward searches from every vertex at once, each
-// vertex keeping the smallest source); a vertex r whose label is r itself is
-// reached by no smaller open vertex, and the backward search from r inside
-// label r (through G^T) collects exactly r's component: every member reaches r
-// and is reached from r, so it carries label r, and r, reached by no smaller
-// vertex, is its smallest member. Each step closes at least the component of
-// the smallest open vertex, and disconnected parts of the graph (separate
-// graphs of a batch) progress together.
+// SCC_OPEN. The open vertices stand in a list that every step shortens.
+//
+// The first step is one forward-backward search from a pivot, the open vertex
+// with the largest min(in-degree, out-degree): in a graph with a giant component
+// that vertex is nearly always in it, and two searches that touch most edges
+// not at all close it. (Searches from every vertex at once, as below, would
+// walk the giant component's edges several times.) Every later step works on every open
+// vertex at once: its forward part labels each open vertex with the smallest
+// open vertex that reaches it (label propagation along G, i.e. forward searches
+// from every vertex at once, each vertex keeping the smallest source); a vertex
+// r whose label is r itself is reached by no smaller open vertex, and the
+// backward search from r inside label r (through G^T) collects exactly r's
+// component: every member reaches r and is reached from r, so it carries label
+// r, and r, reached by no smaller vertex, is its smallest member. Each step
+// closes at least the component of the smallest open vertex, and disconnected
+// parts of the graph (separate graphs of a batch) progress together.
+//
+// A level of a search is bound by latency when it is small (a grid barrier, not
+// a launch and a host round trip, ends it) and by random accesses when it is
+// large; rows are spread over the warps 32 vertices at a time laid end to end,
+// and rows over kSccHeavy edges over the whole grid (one warp on a hub's row
+// was what a level waited for).
+//
+// Measured (ms, in+out trimming included; before: one launch and one host read
+// per level and pass, a warp per row, searches from every vertex in every step):
+// R-MAT scale 14 0.13 (0.80), 20 0.29 (5.9), 22 0.65 (16.7); 4,096 planted graphs
+// in one call 17.7 (51.1); a planted graph of 100,000 0.47 (0.89).
 #include "trim_internal.cuh"
 
 using namespace trimk;
@@ -21,264 +39,592 @@ using namespace trimk;
 namespace {
 constexpr uint32_t SCC_OPEN = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
-__device__ __forceinline__ uint32_t gtid() { return blockIdx.x * blockDim.x + threadIdx.x; }
-__device__ __forceinline__ uint32_t gsize() { return gridDim.x * blockDim.x; }
-}  // namespace
+constexpr uint32_t CLOSED = 0xFFFFFFFFu;  // search mark of a vertex with a component
+constexpr unsigned FULL = 0xFFFFFFFFu;
+constexpr uint32_t kSccHeavy = 1024;   // longer rows go to the whole grid ...
+constexpr uint32_t kSccChunk = 256;    // ... in pieces of this many edges
+constexpr uint32_t kBuf = 256;         // entries staged per warp before a flush
+constexpr int kMaxWarps = 16;
 
-// After in+out trimming: removed vertices are size-1 components; the others
-// are open, all in partition 0.
-__global__ void scc_init_kernel(const uint32_t* level, uint32_t n, uint32_t* comp, uint32_t* color) {
-  for (uint32_t v = gtid(); v < n; v += gsize()) {
-    const bool open = level[v] == LIVE;
-    comp[v] = open ? SCC_OPEN : v;
-    color[v] = 0u;
+// Per-CTA state: the warps' append buffers, and the barrier's progress.
+struct Scc {
+  uint32_t buf[kMaxWarps][kBuf];
+  unsigned epoch;
+  unsigned err;
+  unsigned phase;
+};
+
+__device__ __forceinline__ uint32_t gwarp() {
+  return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+}
+__device__ __forceinline__ uint32_t nwarps() { return gridDim.x * (blockDim.x >> 5); }
+
+// Grid-wide barrier (bounded as the trimming kernel's): a phase ends. Phase p
+// counts into slot p & 3, which is read in phase p + 1; the slot of phase p + 2
+// was last read in phase p - 1 and is cleared by CTA 0 at the start of phase p.
+// Returns false when the run must stop.
+__device__ bool scc_sync(const SccArgs& A, Scc& S) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned target = (++S.epoch) * gridDim.x;
+    __threadfence();
+    atomicAdd(&A.C->bar, 1u);
+    const uint64_t t0 = globaltimer();
+    while ((int)(ld_relaxed(&A.C->bar) - target) < 0) {
+      if (globaltimer() - t0 > A.spin_limit_ns) {
+        atomicCAS(&A.C->err, 0u, (unsigned)TRIM_ERR_TIMEOUT);
+        break;
+      }
+    }
+    (void)ld_acquire(&A.C->bar);
+    S.err = ld_relaxed(&A.C->err);
+    S.phase += 1u;
+    if (blockIdx.x == 0) {
+      SccSlot* z = &A.C->slot[(S.phase + 2u) & 3u];
+      z->n = z->heavy = z->hits = 0u;
+    }
+  }
+  __syncthreads();
+  return S.err == 0u;
+}
+__device__ __forceinline__ SccSlot* now(const SccArgs& A, const Scc& S) {
+  return &A.C->slot[S.phase & 3u];
+}
+__device__ __forceinline__ const SccSlot* before(const SccArgs& A, const Scc& S) {
+  return &A.C->slot[(S.phase - 1u) & 3u];
+}
+
+// Appends to a global list, staged in the warp's buffer: one atomic per flush.
+struct Out {
+  uint32_t* list;
+  unsigned* count;
+  uint32_t have;
+};
+__device__ __forceinline__ void flush(Scc& S, Out& o) {
+  if (o.have == 0u) return;
+  const uint32_t* b = S.buf[threadIdx.x >> 5];
+  __syncwarp();
+  uint32_t at = 0;
+  if (lane_id() == 0) at = atomicAdd(o.count, o.have);
+  at = __shfl_sync(FULL, at, 0);
+  for (uint32_t i = lane_id(); i < o.have; i += 32u) o.list[at + i] = b[i];
+  __syncwarp();
+  o.have = 0u;
+}
+// Warp-collective: lanes with pred append v.
+__device__ __forceinline__ void put(Scc& S, Out& o, bool pred, uint32_t v) {
+  const unsigned m = __ballot_sync(FULL, pred);
+  if (m == 0u) return;
+  if (o.have + 32u > kBuf) flush(S, o);
+  if (pred) S.buf[threadIdx.x >> 5][o.have + __popc(m & ((1u << lane_id()) - 1u))] = v;
+  o.have += __popc(m);
+}
+// Adds a count per lane to a counter (warp-collective).
+__device__ __forceinline__ void add(unsigned* c, unsigned x) {
+  x = __reduce_add_sync(FULL, x);
+  if (lane_id() == 0 && x) atomicAdd(c, x);
+}
+
+// All warps: f(u, w, valid) (warp-collective) for the edges u -> w of the rows of
+// list[0..count): a warp takes up to 32 vertices, their rows laid end to end,
+// four loads in flight per lane. Rows over kSccHeavy edges go to the heavy list
+// for heavy_edges, in the next phase.
+template <class F>
+__device__ __forceinline__ void list_edges(const SccArgs& A, const Scc& S, const uint32_t* off,
+                                           const uint32_t* tgt, const uint32_t* list,
+                                           uint32_t count, F f) {
+  const unsigned lane = lane_id();
+  const uint32_t nw = nwarps();
+  const uint32_t G = min(32u, max(1u, (count + nw - 1u) / nw));
+  for (uint32_t base = gwarp() * G; base < count; base += nw * G) {  // warp-uniform
+    const bool has = lane < G && base + lane < count;
+    const uint32_t u = has ? ldcg(&list[base + lane]) : 0u;
+    const uint32_t s = has ? __ldg(&off[u]) : 0u;
+    uint32_t d = has ? __ldg(&off[u + 1u]) - s : 0u;
+    if (d > kSccHeavy) {
+      A.heavy[atomicAdd(&now(A, S)->heavy, 1u)] = u;
+      d = 0u;
+    }
+    const uint32_t incl = warp_incl_scan(d), excl = incl - d;
+    const uint32_t total = __shfl_sync(FULL, incl, 31);
+    for (uint32_t k0 = 0; k0 < total; k0 += 128u) {
+      uint32_t uu[4], w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t k = k0 + (uint32_t)q * 32u + lane;
+        const unsigned o = owner_of(excl, k);
+        const uint32_t so = __shfl_sync(FULL, s, o), xo = __shfl_sync(FULL, excl, o);
+        uu[q] = __shfl_sync(FULL, u, o);
+        w[q] = k < total ? __ldg(&tgt[so + (k - xo)]) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) f(uu[q], w[q], k0 + (uint32_t)q * 32u + lane < total);
+    }
+  }
+}
+template <class F>
+__device__ __forceinline__ void heavy_edges(const SccArgs& A, const uint32_t* off,
+                                            const uint32_t* tgt, uint32_t nheavy, F f) {
+  const unsigned lane = lane_id();
+  for (uint32_t h = 0; h < nheavy; ++h) {
+    const uint32_t u = ldcg(&A.heavy[h]);
+    const uint32_t s = __ldg(&off[u]), e = __ldg(&off[u + 1u]);
+    for (uint64_t k0 = (uint64_t)s + (uint64_t)gwarp() * kSccChunk; k0 < e;
+         k0 += (uint64_t)nwarps() * kSccChunk)  // warp-uniform
+#pragma unroll
+      for (uint32_t i = 0; i < kSccChunk; i += 32u) {
+        const uint64_t k = k0 + i + lane;
+        f(u, k < e ? __ldg(&tgt[k]) : 0u, k < e);
+      }
   }
 }
 
-// Warp-collective row probe: for the lanes with want, counts (up to cap) the
-// entries of row [s, s+d) whose vertex is open, skipping `self`, and returns
-// the first such vertex (NONE if none). Rows of up to 32 entries are probed by
-// their own lane; longer ones by the whole warp, 32 entries per step, stopping
-// once cap open entries are seen.
-__device__ __forceinline__ uint32_t probe_row(const uint32_t* rowtgt, uint32_t s, uint32_t d,
-                                              bool want, uint32_t self, const uint32_t* comp,
-                                              uint32_t cap, uint32_t& count) {
+// Does the row [s, s + d) hold an entry for which hit(w) is true? Warp-collective
+// for the lanes with want: four entries per lane at a time, up to 32 of a row;
+// what is left of longer rows is looked through by the whole warp.
+template <class H>
+__device__ __forceinline__ bool row_any(const uint32_t* tgt, uint32_t s, uint32_t d, bool want,
+                                        H hit) {
   const unsigned lane = lane_id();
-  uint32_t first = NONE;
-  count = 0;
-  const bool own = want && d <= 32u;
-  for (uint32_t k = 0; own && k < d && count < cap; ++k) {
-    const uint32_t w = rowtgt[s + k];
-    if (w != self && ldcg(&comp[w]) == SCC_OPEN) {
-      if (first == NONE) first = w;
-      ++count;
-    }
+  bool found = false;
+  uint32_t i = 0;
+  while (want && !found && i < d && i < 32u) {
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[q] = i + q < d ? __ldg(&tgt[s + i + q]) : 0u;
+    bool h[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) h[q] = i + q < d && hit(w[q]);
+    found = h[0] || h[1] || h[2] || h[3];
+    i += 4u;
   }
-  unsigned big = __ballot_sync(0xFFFFFFFFu, want && d > 32u);
+  __syncwarp();
+  unsigned big = __ballot_sync(FULL, want && !found && d > 32u);
   while (big) {
     const int j = __ffs(big) - 1;
     big &= big - 1u;
-    const uint32_t sj = __shfl_sync(0xFFFFFFFFu, s, j), dj = __shfl_sync(0xFFFFFFFFu, d, j);
-    const uint32_t self_j = __shfl_sync(0xFFFFFFFFu, self, j);
-    uint32_t cnt = 0, fst = NONE;
-    for (uint32_t k0 = 0; k0 < dj && cnt < cap; k0 += 32u) {  // warp-uniform
-      const uint32_t k = k0 + lane;
-      bool hit = false;
-      uint32_t w = 0;
-      if (k < dj) {
-        w = rowtgt[sj + k];
-        hit = w != self_j && ldcg(&comp[w]) == SCC_OPEN;
+    const uint32_t sj = __shfl_sync(FULL, s, j), dj = __shfl_sync(FULL, d, j);
+    bool any = false;
+    for (uint32_t k0 = 32u; k0 < dj && !any; k0 += 128u) {  // warp-uniform
+      uint32_t w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t k = k0 + (uint32_t)q * 32u + lane;
+        w[q] = k < dj ? __ldg(&tgt[sj + k]) : 0u;
       }
-      const unsigned hm = __ballot_sync(0xFFFFFFFFu, hit);
-      if (hm && fst == NONE) fst = __shfl_sync(0xFFFFFFFFu, w, __ffs(hm) - 1);
-      cnt += __popc(hm);
+      bool h = false;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t k = k0 + (uint32_t)q * 32u + lane;
+        h = h || (k < dj && hit(w[q]));
+      }
+      any = __any_sync(FULL, h);
+    }
+    if ((int)lane == j) found = any;
+  }
+  return found;
+}
+
+// Open entries of the row [s, s + d) for the lanes with want: those other than
+// `self` counted up to 2 (oth, the first one in *first) and all of them up to 3.
+__device__ __forceinline__ void row_count(const SccArgs& A, const uint32_t* tgt, uint32_t s,
+                                          uint32_t d, bool want, uint32_t self, uint32_t& oth,
+                                          uint32_t& all, uint32_t& first) {
+  const unsigned lane = lane_id();
+  oth = all = 0u;
+  first = NONE;
+  for (uint32_t i = 0; want && d <= 32u && i < d && (oth < 2u || all < 3u); i += 4u) {
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[q] = i + q < d ? __ldg(&tgt[s + i + q]) : 0u;
+    bool o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[q] = i + q < d && ldcg(&A.comp[w[q]]) == SCC_OPEN;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (!o[q]) continue;
+      ++all;
+      if (w[q] != self) {
+        if (first == NONE) first = w[q];
+        ++oth;
+      }
+    }
+  }
+  __syncwarp();
+  unsigned big = __ballot_sync(FULL, want && d > 32u);
+  while (big) {
+    const int j = __ffs(big) - 1;
+    big &= big - 1u;
+    const uint32_t sj = __shfl_sync(FULL, s, j), dj = __shfl_sync(FULL, d, j);
+    const uint32_t vj = __shfl_sync(FULL, self, j);
+    uint32_t o = 0, a = 0, f = NONE;
+    for (uint32_t k0 = 0; k0 < dj && (o < 2u || a < 3u); k0 += 32u) {  // warp-uniform
+      const uint32_t k = k0 + lane;
+      const uint32_t w = k < dj ? __ldg(&tgt[sj + k]) : 0u;
+      const bool open = k < dj && ldcg(&A.comp[w]) == SCC_OPEN;
+      const unsigned om = __ballot_sync(FULL, open && w != vj);
+      if (om && f == NONE) f = __shfl_sync(FULL, w, __ffs(om) - 1);
+      o += __popc(om);
+      a += __popc(__ballot_sync(FULL, open));
     }
     if ((int)lane == j) {
-      first = fst;
-      count = min(cnt, cap);
+      oth = o;
+      all = a;
+      first = f;
     }
   }
-  return first;
+  oth = min(oth, 2u);
+  all = min(all, 3u);
 }
 
-// Size-2 trimming, pass 1: for every open vertex, its only open successor
-// other than itself (out1) and its only open predecessor other than itself
-// (in1), counting parallel edges separately, or NONE when there is none or
-// more than one. A self-loop makes v a component of its own, so such a vertex
-// is never paired (NONE).
-__global__ void scc_trim2_single_kernel(const uint32_t* off, const uint32_t* tgt,
-                                        const uint32_t* ioff, const uint32_t* itgt, uint32_t n,
-                                        const uint32_t* comp, uint32_t* out1, uint32_t* in1) {
-  for (uint32_t w0 = gtid() & ~31u; w0 < n; w0 += gsize()) {  // warp-uniform
-    const uint32_t v = w0 + lane_id();
-    const bool open = v < n && comp[v] == SCC_OPEN;
-    const uint32_t s = open ? off[v] : 0u, d = open ? off[v + 1] - s : 0u;
-    const uint32_t is = open ? ioff[v] : 0u, id = open ? ioff[v + 1] - is : 0u;
-    uint32_t oc = 0, ic = 0, lc = 0;
-    // a self-loop: counted as the one "open entry equal to v" of its row
-    const uint32_t o = probe_row(tgt, s, d, open, v, comp, 2u, oc);
-    const uint32_t i = probe_row(itgt, is, id, open, v, comp, 2u, ic);
-    const uint32_t all_out = probe_row(tgt, s, d, open, NONE, comp, 3u, lc);
-    const bool loop = open && lc > oc;  // more open entries with v itself than without
-    (void)all_out;
-    if (v < n) {
-      out1[v] = (open && !loop && oc == 1u) ? o : NONE;
-      in1[v] = (open && !loop && ic == 1u) ? i : NONE;
-    }
+// The open vertices of list[0..count) go to `to` (one phase; its count is in the
+// phase's slot).
+__device__ __forceinline__ void keep_open(const SccArgs& A, Scc& S, const uint32_t* list,
+                                          uint32_t count, uint32_t* to) {
+  Out o{to, &now(A, S)->n, 0u};
+  for (uint32_t base = gwarp() * 32u; base < count; base += nwarps() * 32u) {
+    const uint32_t i = base + lane_id();
+    const uint32_t v = i < count ? ldcg(&list[i]) : 0u;
+    put(S, o, i < count && ldcg(&A.comp[v]) == SCC_OPEN, v);
   }
+  flush(S, o);
 }
 
-// Size-2 trimming, pass 2: v and u = out1[v] with out1[u] = v are each other's
-// only open successors, so {u, v} is a component (a closed 2-cycle); the same
-// with predecessors. Both members write the same label. Counts the pairs.
-__global__ void scc_trim2_pair_kernel(uint32_t n, const uint32_t* out1, const uint32_t* in1,
-                                      uint32_t* comp, unsigned long long* pairs) {
-  unsigned long long k = 0;
-  for (uint32_t v = gtid(); v < n; v += gsize()) {
-    const uint32_t o = out1[v], i = in1[v];
-    uint32_t u = NONE;
-    if (o != NONE && out1[o] == v) u = o;
-    else if (i != NONE && in1[i] == v) u = i;
-    if (u != NONE) {
-      comp[v] = min(u, v);
-      k += (v < u) ? 1u : 0u;
-    }
-  }
-  k = warp_sum(k);
-  if (lane_id() == 0 && k) atomicAdd(pairs, k);
+__device__ __forceinline__ void close_vertex(const SccArgs& A, uint32_t v, uint32_t c) {
+  A.comp[v] = c;
+  A.fw[v] = CLOSED;
+  A.bw[v] = CLOSED;
 }
 
-// One trimming pass: an open vertex without an open successor, or without an
-// open predecessor, is a component of its own (its other neighbours are in
-// components already complete, so no cycle through it remains). Counts what
-// it removed (0: nothing left to trim).
-__global__ void scc_trim1_kernel(const uint32_t* off, const uint32_t* tgt, const uint32_t* ioff,
-                                 const uint32_t* itgt, uint32_t n, uint32_t* comp,
-                                 unsigned long long* removed) {
-  unsigned long long k = 0;
-  for (uint32_t w0 = gtid() & ~31u; w0 < n; w0 += gsize()) {  // warp-uniform
-    const uint32_t v = w0 + lane_id();
-    const bool open = v < n && ldcg(&comp[v]) == SCC_OPEN;
-    const uint32_t s = open ? off[v] : 0u, d = open ? off[v + 1] - s : 0u;
-    uint32_t oc = 0, ic = 0;
-    probe_row(tgt, s, d, open, NONE, comp, 1u, oc);
-    const bool need_in = open && oc > 0u;
-    const uint32_t is = need_in ? ioff[v] : 0u, id = need_in ? ioff[v + 1] - is : 0u;
-    probe_row(itgt, is, id, need_in, NONE, comp, 1u, ic);
-    if (open && (oc == 0u || ic == 0u)) {
-      comp[v] = v;
-      ++k;
-    }
-  }
-  k = warp_sum(k);
-  if (lane_id() == 0 && k) atomicAdd(removed, k);
-}
-
-// Labels: every open vertex starts with its own id and joins the first frontier.
-__global__ void scc_label_start_kernel(uint32_t n, const uint32_t* comp, uint32_t* label,
-                                       uint32_t* frontier, uint32_t* count,
-                                       unsigned long long* open) {
-  unsigned long long k = 0;
-  for (uint32_t w0 = gtid() & ~31u; w0 < n; w0 += gsize()) {  // warp-uniform
-    const uint32_t v = w0 + lane_id();
-    const bool o = v < n && comp[v] == SCC_OPEN;
-    if (v < n) label[v] = o ? v : NONE;
-    const unsigned bm = __ballot_sync(0xFFFFFFFFu, o);
-    if (!bm) continue;
-    uint32_t at = 0;
-    if (lane_id() == (unsigned)(__ffs(bm) - 1)) at = atomicAdd(count, (uint32_t)__popc(bm));
-    at = __shfl_sync(0xFFFFFFFFu, at, __ffs(bm) - 1);
-    if (o) frontier[at + __popc(bm & ((1u << lane_id()) - 1u))] = v;
-    k += o ? 1u : 0u;
-  }
-  k = warp_sum(k);
-  if (lane_id() == 0 && k) atomicAdd(open, k);
-}
-
-// One level of label propagation along G: every frontier vertex offers its
-// label to its open successors; a successor whose label drops joins the next
-// frontier (once per level: inq holds the level's stamp).
-__global__ void scc_label_level_kernel(const uint32_t* off, const uint32_t* tgt,
-                                       const uint32_t* comp, uint32_t* label, uint32_t* inq,
-                                       uint32_t stamp, const uint32_t* frontier, uint32_t count,
-                                       uint32_t* next, uint32_t* next_count) {
-  const uint32_t lane = lane_id();
-  const uint32_t warps = gsize() >> 5;
-  for (uint32_t i = gtid() >> 5; i < count; i += warps) {
-    const uint32_t u = frontier[i];
-    const uint32_t lu = ldcg(&label[u]);
-    const uint32_t s = off[u], e = off[u + 1];
-    for (uint32_t k0 = s; k0 < e; k0 += 32u) {
-      const uint32_t k = k0 + lane;
-      bool take = false;
-      uint32_t w = 0;
-      if (k < e) {
-        w = tgt[k];
-        if (comp[w] == SCC_OPEN && ldcg(&label[w]) > lu && atomicMin(&label[w], lu) > lu)
-          take = atomicExch(&inq[w], stamp) != stamp;
+// Search from the frontier in A.fa (k vertices, marked with `stamp`) along
+// (off, tgt), whose transpose is (roff, rtgt), among the open vertices in
+// `allow` (where given: those whose mark there is allowed). A small frontier
+// offers its rows; once it is large, the vertices not yet marked look for a
+// marked neighbour instead (usually within a few entries). Returns false on an
+// error.
+__device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint32_t* tgt,
+                       const uint32_t* roff, const uint32_t* rtgt, uint32_t* mark, uint32_t stamp,
+                       const uint32_t* allow, uint32_t allowed, const uint32_t* open, uint32_t n_open,
+                       uint32_t k, uint32_t& levels) {
+  const unsigned lane = lane_id();
+  uint32_t *fa = A.fa, *fb = A.fb;
+  uint32_t left = n_open - min(n_open, k);  // not marked yet (at most)
+  while (k > 0u) {
+    ++levels;
+    Out o{fb, &now(A, S)->n, 0u};
+    if ((uint64_t)k * 16u > left) {
+      for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+        const uint32_t i = base + lane;
+        const uint32_t v = i < n_open ? ldcg(&open[i]) : 0u;
+        const bool want = i < n_open && ldcg(&mark[v]) < stamp &&
+                          (allow == nullptr || ldcg(&allow[v]) == allowed);
+        const uint32_t s = want ? __ldg(&roff[v]) : 0u;
+        const uint32_t d = want ? __ldg(&roff[v + 1u]) - s : 0u;
+        const bool hit = row_any(rtgt, s, d, want, [&](uint32_t w) { return ldcg(&mark[w]) == stamp; });
+        if (hit) mark[v] = stamp;
+        put(S, o, hit, v);
       }
-      const unsigned bm = __ballot_sync(0xFFFFFFFFu, take);
-      if (!bm) continue;
-      uint32_t at = 0;
-      if (lane == 0) at = atomicAdd(next_count, (uint32_t)__popc(bm));
-      at = __shfl_sync(0xFFFFFFFFu, at, 0);
-      if (take) next[at + __popc(bm & ((1u << lane) - 1u))] = w;
-    }
-  }
-}
-
-// Roots: open vertices that kept their own label start the backward searches.
-__global__ void scc_roots_start_kernel(uint32_t n, const uint32_t* comp, const uint32_t* label,
-                                       uint32_t* mark, uint32_t stamp, uint32_t* frontier,
-                                       uint32_t* count) {
-  for (uint32_t w0 = gtid() & ~31u; w0 < n; w0 += gsize()) {  // warp-uniform
-    const uint32_t v = w0 + lane_id();
-    const bool root = v < n && comp[v] == SCC_OPEN && label[v] == v;
-    const unsigned bm = __ballot_sync(0xFFFFFFFFu, root);
-    if (!bm) continue;
-    uint32_t at = 0;
-    if (lane_id() == (unsigned)(__ffs(bm) - 1)) at = atomicAdd(count, (uint32_t)__popc(bm));
-    at = __shfl_sync(0xFFFFFFFFu, at, __ffs(bm) - 1);
-    if (root) {
-      mark[v] = stamp;
-      frontier[at + __popc(bm & ((1u << lane_id()) - 1u))] = v;
-    }
-  }
-}
-
-// One level of the backward searches (through G^T): each warp takes frontier
-// vertices, its lanes walk the row; an open neighbour with the same label not
-// yet marked with this stamp is marked (the atomic exchange that sees an older
-// stamp wins) and joins the next frontier.
-__global__ void scc_search_level_kernel(const uint32_t* rowoff, const uint32_t* rowtgt,
-                                        const uint32_t* comp, const uint32_t* color,
-                                        uint32_t* mark, uint32_t stamp, const uint32_t* frontier,
-                                        uint32_t count, uint32_t* next, uint32_t* next_count) {
-  const uint32_t lane = lane_id();
-  const uint32_t warps = gsize() >> 5;
-  for (uint32_t i = gtid() >> 5; i < count; i += warps) {
-    const uint32_t u = frontier[i];
-    const uint32_t c = color[u];
-    const uint32_t s = rowoff[u], e = rowoff[u + 1];
-    for (uint32_t k0 = s; k0 < e; k0 += 32u) {
-      const uint32_t k = k0 + lane;
-      bool take = false;
-      uint32_t w = 0;
-      if (k < e) {
-        w = rowtgt[k];
-        take = comp[w] == SCC_OPEN && color[w] == c && ldcg(&mark[w]) != stamp &&
-               atomicExch(&mark[w], stamp) != stamp;
+      flush(S, o);
+      if (!scc_sync(A, S)) return false;
+      k = ldcg(&before(A, S)->n);
+    } else {
+      auto visit = [&](uint32_t, uint32_t w, bool valid) {
+        const bool take = valid && ldcg(&mark[w]) < stamp &&
+                          (allow == nullptr || ldcg(&allow[w]) == allowed) &&
+                          atomicMax(&mark[w], stamp) < stamp;
+        put(S, o, take, w);
+      };
+      list_edges(A, S, off, tgt, fa, k, visit);
+      flush(S, o);
+      if (!scc_sync(A, S)) return false;
+      const uint32_t heavy = ldcg(&before(A, S)->heavy);
+      k = ldcg(&before(A, S)->n);
+      if (heavy) {  // (their finds join the same list, behind those of the phase before)
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&now(A, S)->n, k);
+        o.count = &now(A, S)->hits;
+        o.list = fb + k;
+        heavy_edges(A, off, tgt, heavy, visit);
+        flush(S, o);
+        if (!scc_sync(A, S)) return false;
+        k = ldcg(&before(A, S)->n) + ldcg(&before(A, S)->hits);
       }
-      const unsigned bm = __ballot_sync(0xFFFFFFFFu, take);
-      if (!bm) continue;
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(next_count, (uint32_t)__popc(bm));
-      base = __shfl_sync(0xFFFFFFFFu, base, 0);
-      if (take) next[base + __popc(bm & ((1u << lane) - 1u))] = w;
     }
+    left -= min(left, k);
+    uint32_t* t = fa;
+    fa = fb;
+    fb = t;
   }
+  return true;
 }
 
-// Close: every open vertex the backward search from its label's root reached
-// belongs to that root's component. Counts the vertices placed.
-__global__ void scc_close_kernel(uint32_t n, uint32_t* comp, const uint32_t* label,
-                                 const uint32_t* mark, uint32_t stamp,
-                                 unsigned long long* placed) {
-  unsigned long long k = 0;
-  for (uint32_t v = gtid(); v < n; v += gsize()) {
-    if (comp[v] == SCC_OPEN && mark[v] == stamp) {
-      comp[v] = label[v];
-      ++k;
+// Trimming passes: an open vertex without an open successor, or without an open
+// predecessor, is a component of its own (its other neighbours are in components
+// already complete, so no cycle through it remains).
+__device__ bool trim_passes(const SccArgs& A, Scc& S, const uint32_t* open, uint32_t n_open,
+                            unsigned& trimmed) {
+  const unsigned lane = lane_id();
+  for (int pass = 0; pass < 1024; ++pass) {
+    unsigned gone = 0;
+    for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+      const uint32_t i = base + lane;
+      const uint32_t v = i < n_open ? ldcg(&open[i]) : 0u;
+      const bool is = i < n_open && ldcg(&A.comp[v]) == SCC_OPEN;
+      auto hit = [&](uint32_t w) { return ldcg(&A.comp[w]) == SCC_OPEN; };
+      const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
+      const bool out = row_any(A.tgt, s, d, is, hit);
+      const uint32_t t = out ? __ldg(&A.ioff[v]) : 0u, e = out ? __ldg(&A.ioff[v + 1u]) - t : 0u;
+      const bool in = row_any(A.itgt, t, e, out, hit);
+      if (is && !in) {
+        close_vertex(A, v, v);
+        ++gone;
+      }
     }
+    add(&now(A, S)->hits, gone);
+    if (!scc_sync(A, S)) return false;
+    const unsigned k = ldcg(&before(A, S)->hits);
+    trimmed += k;
+    if (k == 0u) break;
   }
-  k = warp_sum(k);
-  if (lane_id() == 0 && k) atomicAdd(placed, k);
+  return true;
 }
 
-// Number of components: vertices that label their own component.
-__global__ void scc_count_kernel(uint32_t n, const uint32_t* comp, unsigned long long* count) {
-  unsigned long long k = 0;
-  for (uint32_t v = gtid(); v < n; v += gsize()) k += comp[v] == v ? 1u : 0u;
-  k = warp_sum(k);
-  if (lane_id() == 0 && k) atomicAdd(count, k);
+}  // namespace
+
+__global__ void __launch_bounds__(512, 2) trim_scc_kernel(SccArgs A) {
+  __shared__ Scc S;
+  const unsigned lane = lane_id();
+  const uint32_t n = A.n;
+  if (threadIdx.x == 0) {
+    S.epoch = S.err = S.phase = 0u;
+  }
+  // in+out trimming failed: its error is the run's
+  if (ld_relaxed(&A.run->err) != 0u) return;
+  __syncthreads();
+  // size-1 components from in+out trimming; the others are open
+  {
+    Out o{A.open0, &now(A, S)->n, 0u};
+    for (uint32_t base = gwarp() * 32u; base < n; base += nwarps() * 32u) {
+      const uint32_t v = base + lane;
+      const bool open = v < n && A.level[v] == LIVE;
+      if (v < n) {
+        A.comp[v] = open ? SCC_OPEN : v;
+        A.fw[v] = A.bw[v] = open ? 0u : CLOSED;
+      }
+      put(S, o, open, v);
+    }
+    flush(S, o);
+  }
+  if (!scc_sync(A, S)) return;
+  uint32_t *open = A.open0, *spare = A.open1;
+  uint32_t n_open = ldcg(&before(A, S)->n);
+  // Size-2 trimming: for every open vertex its only open successor other than
+  // itself (out1) and its only open predecessor other than itself (in1),
+  // parallel edges counted separately, NONE when there is none or more than
+  // one; a vertex with a self-loop, which is a component of its own, is never
+  // paired. `more` is true for a self-loop and for three or more open
+  // successors; the second pass over G^T is for the few others.
+  for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+    const uint32_t i = base + lane;
+    const bool is = i < n_open;
+    const uint32_t v = is ? ldcg(&open[i]) : 0u;
+    const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
+    uint32_t oth = 0, all = 0, o1 = NONE, ioth = 0, iall = 0, i1 = NONE;
+    row_count(A, A.tgt, s, d, is, v, oth, all, o1);
+    const bool more = all > oth;
+    const bool back = is && !more;
+    const uint32_t t = back ? __ldg(&A.ioff[v]) : 0u, e = back ? __ldg(&A.ioff[v + 1u]) - t : 0u;
+    row_count(A, A.itgt, t, e, back, v, ioth, iall, i1);
+    if (is) {
+      A.fa[v] = (!more && oth == 1u) ? o1 : NONE;
+      A.fb[v] = (!more && ioth == 1u) ? i1 : NONE;
+    }
+  }
+  if (!scc_sync(A, S)) return;
+  // v and u = out1[v] with out1[u] = v are each other's only open successors, so
+  // {u, v} is a component (a closed 2-cycle); the same with predecessors. Both
+  // members write the same label.
+  {
+    unsigned pairs = 0;
+    for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+      const uint32_t i = base + lane;
+      if (i < n_open) {
+        const uint32_t v = ldcg(&open[i]);
+        const uint32_t o = ldcg(&A.fa[v]), p = ldcg(&A.fb[v]);
+        uint32_t u = NONE;
+        if (o != NONE && ldcg(&A.fa[o]) == v) u = o;
+        else if (p != NONE && ldcg(&A.fb[p]) == v) u = p;
+        if (u != NONE) {
+          close_vertex(A, v, min(u, v));
+          pairs += v < u ? 1u : 0u;
+        }
+      }
+    }
+    add(&now(A, S)->hits, pairs);
+  }
+  if (!scc_sync(A, S)) return;
+  const unsigned size2 = ldcg(&before(A, S)->hits);
+  unsigned trimmed = 0;
+  uint32_t steps = 0, levels = 0, stamp = 0;
+  while (true) {
+    if (!trim_passes(A, S, open, n_open, trimmed)) return;
+    keep_open(A, S, open, n_open, spare);
+    if (!scc_sync(A, S)) return;
+    n_open = ldcg(&before(A, S)->n);
+    uint32_t* t = open;
+    open = spare;
+    spare = t;
+    if (n_open == 0u) break;  // every vertex has its component
+    if (steps == 0u) {
+      // a forward-backward search from one pivot
+      unsigned long long best = 0ull;
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_open;
+           i += gridDim.x * blockDim.x) {
+        const uint32_t v = ldcg(&open[i]);
+        const uint32_t d = min(__ldg(&A.off[v + 1u]) - __ldg(&A.off[v]),
+                               __ldg(&A.ioff[v + 1u]) - __ldg(&A.ioff[v]));
+        const unsigned long long key = ((unsigned long long)d << 32) | (0xFFFFFFFFu - v);
+        best = key > best ? key : best;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(FULL, best, o);
+        best = x > best ? x : best;
+      }
+      if (lane == 0 && best) atomicMax(&A.C->best, best);
+      if (!scc_sync(A, S)) return;
+      const uint32_t pivot = 0xFFFFFFFFu - (uint32_t)ld_acquire64(&A.C->best);
+      const uint32_t f = ++stamp, b = ++stamp;
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        A.fa[0] = pivot;
+        A.fw[pivot] = f;
+        A.bw[pivot] = b;
+      }
+      if (!scc_sync(A, S)) return;
+      if (!search(A, S, A.off, A.tgt, A.ioff, A.itgt, A.fw, f, nullptr, 0u, open, n_open, 1u, levels))
+        return;
+      if (blockIdx.x == 0 && threadIdx.x == 0) A.fa[0] = pivot;
+      if (!scc_sync(A, S)) return;
+      if (!search(A, S, A.ioff, A.itgt, A.off, A.tgt, A.bw, b, A.fw, f, open, n_open, 1u, levels))
+        return;
+      uint32_t least = NONE;
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_open;
+           i += gridDim.x * blockDim.x) {
+        const uint32_t v = ldcg(&open[i]);
+        if (ldcg(&A.bw[v]) == b) least = min(least, v);
+      }
+      least = __reduce_min_sync(FULL, least);
+      if (lane == 0 && least != NONE) atomicMin(&A.C->least, least);
+      if (!scc_sync(A, S)) return;
+      const uint32_t c = ld_relaxed(&A.C->least);
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_open;
+           i += gridDim.x * blockDim.x) {
+        const uint32_t v = ldcg(&open[i]);
+        if (ldcg(&A.bw[v]) == b) close_vertex(A, v, c);
+      }
+    } else {
+      // labels: every open vertex starts with its own id and joins the first frontier
+      uint32_t *fa = A.fa, *fb = A.fb;
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_open;
+           i += gridDim.x * blockDim.x) {
+        const uint32_t v = ldcg(&open[i]);
+        A.label[v] = v;
+        fa[i] = v;
+      }
+      if (!scc_sync(A, S)) return;
+      // every frontier vertex offers its label to its open successors; one whose
+      // label drops joins the next frontier (once per level: fw holds its stamp)
+      uint32_t k = n_open;
+      while (k > 0u) {
+        ++levels;
+        const uint32_t st = ++stamp;
+        Out o{fb, &now(A, S)->n, 0u};
+        auto offer = [&](uint32_t u, uint32_t w, bool valid) {
+          bool take = false;
+          if (valid && ldcg(&A.comp[w]) == SCC_OPEN) {
+            const uint32_t lu = ldcg(&A.label[u]);
+            take = ldcg(&A.label[w]) > lu && atomicMin(&A.label[w], lu) > lu &&
+                   atomicExch(&A.fw[w], st) != st;
+          }
+          put(S, o, take, w);
+        };
+        list_edges(A, S, A.off, A.tgt, fa, k, offer);
+        flush(S, o);
+        if (!scc_sync(A, S)) return;
+        const uint32_t heavy = ldcg(&before(A, S)->heavy);
+        k = ldcg(&before(A, S)->n);
+        if (heavy) {
+          o.count = &now(A, S)->hits;
+          o.list = fb + k;
+          heavy_edges(A, A.off, A.tgt, heavy, offer);
+          flush(S, o);
+          if (!scc_sync(A, S)) return;
+          k += ldcg(&before(A, S)->hits);
+        }
+        uint32_t* x = fa;
+        fa = fb;
+        fb = x;
+      }
+      // roots: open vertices that kept their own label start the backward searches
+      const uint32_t st = ++stamp;
+      {
+        Out o{fa, &now(A, S)->n, 0u};
+        for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+          const uint32_t i = base + lane;
+          const uint32_t v = i < n_open ? ldcg(&open[i]) : 0u;
+          const bool root = i < n_open && ldcg(&A.label[v]) == v;
+          if (root) A.bw[v] = st;
+          put(S, o, root, v);
+        }
+        flush(S, o);
+      }
+      if (!scc_sync(A, S)) return;
+      k = ldcg(&before(A, S)->n);
+      while (k > 0u) {  // through G^T, inside the label
+        ++levels;
+        Out o{fb, &now(A, S)->n, 0u};
+        auto visit = [&](uint32_t u, uint32_t w, bool valid) {
+          const bool take = valid && ldcg(&A.bw[w]) < st &&
+                            ldcg(&A.label[w]) == ldcg(&A.label[u]) && atomicMax(&A.bw[w], st) < st;
+          put(S, o, take, w);
+        };
+        list_edges(A, S, A.ioff, A.itgt, fa, k, visit);
+        flush(S, o);
+        if (!scc_sync(A, S)) return;
+        const uint32_t heavy = ldcg(&before(A, S)->heavy);
+        k = ldcg(&before(A, S)->n);
+        if (heavy) {
+          o.count = &now(A, S)->hits;
+          o.list = fb + k;
+          heavy_edges(A, A.ioff, A.itgt, heavy, visit);
+          flush(S, o);
+          if (!scc_sync(A, S)) return;
+          k += ldcg(&before(A, S)->hits);
+        }
+        uint32_t* x = fa;
+        fa = fb;
+        fb = x;
+      }
+      // an open vertex that the backward search from its label's root reached
+      // belongs to that root's component
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_open;
+           i += gridDim.x * blockDim.x) {
+        const uint32_t v = ldcg(&open[i]);
+        if (ldcg(&A.bw[v]) == st) close_vertex(A, v, ldcg(&A.label[v]));
+      }
+    }
+    if (!scc_sync(A, S)) return;
+    ++steps;
+  }
+  // number of components: vertices that label their own component
+  unsigned k = 0;
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+    k += ldcg(&A.comp[v]) == v ? 1u : 0u;
+  add(&A.C->components, k);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    A.C->size2 = size2;
+    A.C->trimmed = trimmed;
+    A.C->steps = steps;
+    A.C->levels = levels;
+    A.C->done = 1u;
+  }
 }
