@@ -332,16 +332,16 @@ __device__ __forceinline__ void set_error(const Dev& D, unsigned code, unsigned 
 
 // kernels (trim_kernels.cu, one flavour per variant set; trim_aux.cu), launched from trim_api.cu
 __global__ void trim_probe_atomic_kernel(const uint32_t* idx, uint64_t n, uint32_t* counters);
-__global__ void trim_persistent_kernel_m1(trimk::Dev D);   // AC-4 only
-__global__ void trim_persistent_kernel_m2(trimk::Dev D);   // AC-6 only
-__global__ void trim_persistent_kernel_m4(trimk::Dev D);   // AC-3 only
-__global__ void trim_persistent_kernel_m9(trimk::Dev D);   // AC-4 + schedulers (segments)
-__global__ void trim_persistent_kernel_m10(trimk::Dev D);  // AC-6 + schedulers (segments)
-__global__ void trim_persistent_kernel_m12(trimk::Dev D);  // AC-3 + schedulers (segments)
-__global__ void trim_persistent_kernel_m15(trimk::Dev D);  // all variants + schedulers
-__global__ void trim_persistent_kernel_m17(trimk::Dev D);  // in+out trimming (AC-4 pushes on G and G^T)
-__global__ void trim_persistent_kernel_m34(trimk::Dev D);  // AC-6 on an implicit graph
-__global__ void trim_persistent_kernel_m36(trimk::Dev D);  // AC-3 on an implicit graph
+__global__ void trim_persistent_kernel_m1(const __grid_constant__ trimk::Dev P);   // AC-4 only
+__global__ void trim_persistent_kernel_m2(const __grid_constant__ trimk::Dev P);   // AC-6 only
+__global__ void trim_persistent_kernel_m4(const __grid_constant__ trimk::Dev P);   // AC-3 only
+__global__ void trim_persistent_kernel_m9(const __grid_constant__ trimk::Dev P);   // AC-4 + schedulers (segments)
+__global__ void trim_persistent_kernel_m10(const __grid_constant__ trimk::Dev P);  // AC-6 + schedulers (segments)
+__global__ void trim_persistent_kernel_m12(const __grid_constant__ trimk::Dev P);  // AC-3 + schedulers (segments)
+__global__ void trim_persistent_kernel_m15(const __grid_constant__ trimk::Dev P);  // all variants + schedulers
+__global__ void trim_persistent_kernel_m17(const __grid_constant__ trimk::Dev P);  // in+out trimming (AC-4 pushes on G and G^T)
+__global__ void trim_persistent_kernel_m34(const __grid_constant__ trimk::Dev P);  // AC-6 on an implicit graph
+__global__ void trim_persistent_kernel_m36(const __grid_constant__ trimk::Dev P);  // AC-3 on an implicit graph
 __global__ void trim_implicit_degree_sum_kernel(trimk::Dev D, unsigned long long* m);
 __global__ void trim_reset_ctrl_kernel(trimk::Ctrl* C);
 __global__ void trim_status_kernel(const uint32_t* level, uint32_t n, uint8_t* status);
