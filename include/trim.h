@@ -118,7 +118,7 @@ typedef struct {
                                  with TRIM_ERR_TIMEOUT                                       */
   float heur_push_ratio;      /* heuristic: push while sum(indeg F) < ratio * n_live        */
   float heur_ac6_ratio;       /* heuristic (no G^T): AC-6 while |F| < ratio * n_live        */
-  uint32_t local_round_edges; /* AC-4-only kernel: once the in-edges still to push fit a
+  uint32_t local_round_edges; /* AC-4 and in+out kernels: once the in-edges still to push fit a
                                  small round (at most this many, one work-list entry per
                                  warp), rounds run CTA-locally: each CTA queues the vertices
                                  it removes in shared memory and pushes them itself in the
@@ -338,13 +338,14 @@ trim_err_t trim_set_dead_mask(trim_ctx* ctx, const uint8_t* mask, int on_device)
  * smaller of the vertex's Definition-2 levels in G and in G^T). Survivors are
  * exactly the vertices that reach a directed cycle and are reached from one.
  * Needs G^T (csr_in, or built on the device on first use, outside the timing).
- * Runs as one persistent launch that pushes, for every removed vertex, both
- * its G^T row (out-degree counters of its predecessors) and its G row
- * (in-degree counters of its successors). Results are read with trim_status /
- * trim_level like those of trim_run; stats may be NULL (in_edges_pushed counts
- * the G^T pushes, edges_inspected the G pushes). Graphs with 2m > 2^32 - 64 are
- * refused with TRIM_ERR_TOO_LARGE (the work list counts both rows of a vertex in
- * uint32 edge offsets). */
+ * Runs as one persistent launch that pushes, for every removed vertex, the row
+ * that can still hold live vertices: the G^T row (out-degree counters of its
+ * predecessors) of a vertex without live successors, the G row (in-degree
+ * counters of its successors) of one without live predecessors. Results are
+ * read with trim_status / trim_level like those of trim_run; stats may be NULL
+ * (in_edges_pushed counts the in-edges of the removed vertices, edges_inspected
+ * their out-edges). Graphs with 2m > 2^32 - 64 are refused with
+ * TRIM_ERR_TOO_LARGE. */
 trim_err_t trim_run_inout(trim_ctx* ctx, trim_run_stats_t* stats);
 
 /* Enqueues the same work as trim_run without waiting (no host synchronisation,

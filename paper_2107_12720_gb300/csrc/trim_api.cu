@@ -55,7 +55,8 @@ struct trim_ctx {
   uint32_t *ch_ack = nullptr, *ch_load = nullptr;
   // in+out runs: in-degree counters, the work list's G rows and in-degrees, and
   // the chunk-owner index of its edge space (both rows: up to 2m edges)
-  uint32_t *cnt_in = nullptr, *w4_orow = nullptr, *w4_din = nullptr, *chunk_io = nullptr;
+  unsigned long long* cnt_io = nullptr;
+  uint32_t *w4_dir = nullptr, *chunk_io = nullptr;
   uint8_t* mask = nullptr;  // trim_set_dead_mask: device copy of the dead mask
   bool has_mask = false;
   bool implicit = false;      // trim_create_implicit: successors computed, no CSR
@@ -747,16 +748,15 @@ trim_err_t ensure_work_list(trim_ctx* c) {
   return TRIM_OK;
 }
 
-// In+out trimming's arrays: in-degree counters and the work list's out-CSR
-// row starts and in-degrees; allocated on first use.
+// In+out trimming's arrays: both counters of every vertex and the directions of
+// the work list's rows; allocated on first use.
 trim_err_t ensure_inout(trim_ctx* c) {
-  if (c->cnt_in) return TRIM_OK;
+  if (c->chunk_io) return TRIM_OK;  // the last of them
   // the work list's edge offsets are uint32 and cover both rows of every vertex
   if (2 * c->m > (1ull << 32) - 64)
     return fail(c, TRIM_ERR_TOO_LARGE, "in+out trimming needs 2m <= 2^32 - 64");
-  TRY(dalloc(c, &c->cnt_in, c->n));
-  TRY(dalloc(c, &c->w4_orow, c->n));
-  TRY(dalloc(c, &c->w4_din, c->n));
+  TRY(dalloc(c, &c->cnt_io, c->n));
+  TRY(dalloc(c, &c->w4_dir, c->n));
   TRY(dalloc(c, &c->chunk_io, ((2 * c->m) >> 5) + 2));
   return TRIM_OK;
 }
@@ -835,7 +835,7 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   D.s_list = c->s_list; D.log = c->log; D.roff = c->roff; D.live0 = c->live0;
   D.live1 = c->live1; D.w4_row = c->w4_row; D.w4_eoff = c->w4_eoff;
   D.chunk_first = c->chunk_first; D.bsum = c->bsum; D.C = c->ctrl;
-  D.cnt_in = c->cnt_in; D.w4_orow = c->w4_orow; D.w4_din = c->w4_din;
+  D.cnt_io = c->cnt_io; D.w4_dir = c->w4_dir;
   D.mask = c->has_mask ? c->mask : nullptr;
   D.ig = c->ig;
   if (inout) D.chunk_first = c->chunk_io;

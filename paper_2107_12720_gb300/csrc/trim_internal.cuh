@@ -166,12 +166,11 @@ struct Dev {
   uint32_t* w4_row;
   uint32_t* w4_eoff;
   uint32_t* chunk_first;  // [c]: work-list entry that owns edge 32c of the prefix
-  // in+out trimming (trim_run_inout): in-degree counters, and per work-list
-  // entry the vertex's out-CSR row start and in-degree (its edge range covers
-  // its G^T row, then its G row)
-  uint32_t* cnt_in;
-  uint32_t* w4_orow;
-  uint32_t* w4_din;
+  // in+out trimming (trim_run_inout): both counters of every vertex (in-degree
+  // << 32 | out-degree), and per work-list entry whether its row is the vertex's
+  // G^T row (0) or G row (1)
+  unsigned long long* cnt_io;
+  uint32_t* w4_dir;
   // vertex sampling (trim_set_dead_mask): mask[v] != 0 marks a vertex that is
   // DEAD from the start; nullable
   const uint8_t* __restrict__ mask;
@@ -183,7 +182,7 @@ struct Dev {
   uint32_t commit_after;  // != 0: scheduler flavours commit after this many stable rounds
   uint32_t recheck_rounds;  // length of the first committed stretch (doubles while repeated)
   uint32_t bar_base;  // grid-barrier counter when this kernel starts (0 for a new run)
-  uint32_t local_edges_max;  // AC-4: pending in-edges up to which rounds run locally (0: never)
+  uint32_t local_edges_max;  // AC-4, in+out: pending edges up to which rounds run locally (0: never)
   // asynchronous AC-4 tail: per vertex 16 bytes (live-successor counter, top
   // level among its removed successors, G^T row start, row length), in the
   // arrays of AC-6 and AC-3 (supp, s_head, s_next, s_list, contiguous), which

@@ -107,15 +107,29 @@ struct WarpSlice {
 // reservations, nor a read of the control block: it ends at a barrier that
 // carries the round's totals (see local_barrier). A removal that does not fit
 // the queue goes to the global lists, and the run returns to ordinary rounds.
+//
+// In+out trimming (flavour 17) runs local rounds too: its queue holds, per
+// removed vertex, the one row that still matters (see inout_round), and per
+// queued neighbour which of its two counters the push decrements.
 #if TRIM_MODES == 1 || TRIM_MODES == 9
 #define TRIM_LOCAL 1
+#define TRIM_ASYNC 1
+#elif TRIM_MODES == 17
+#define TRIM_LOCAL 1
+#define TRIM_ASYNC 0
 #else
 #define TRIM_LOCAL 0
+#define TRIM_ASYNC 0
 #endif
 #if TRIM_LOCAL
 constexpr uint32_t LQ_EDGES = 1024;   // predecessors queued per CTA per round
 constexpr uint32_t LQ_ENTRIES = 256;  // removed vertices queued per CTA per round
+constexpr uint32_t LQ_FLOOR = 256;     // least bound of a stretch's queues
+constexpr uint32_t LQ_SKEW = 4;        // ... and the bound as a multiple of the mean load
+constexpr uint32_t LQ_LATE_MIN = 1u << 14;  // from here on offsets are loaded for removals only
 constexpr uint32_t LQ_DMAX = 64;      // larger in-degrees always go to the global work list
+#endif
+#if TRIM_ASYNC
 // asynchronous AC-4 tail (see async_tail)
 constexpr uint32_t ASYNC_MIN_ROUND = 128;  // rounds before the tail may take over
 constexpr uint32_t ASYNC_RETRY = 64;       // local stretches end for it at multiples of this
@@ -149,6 +163,11 @@ struct Cta {
   uint32_t lq_ovf;                    // 1: a removal of this round went to the global lists
   uint32_t lq_pushed;                 // predecessors decremented from the queue this round
   uint32_t lq_next;                   // how the stretch goes on after the local barrier
+#if TRIM_MODES & 16
+  uint8_t lq_dir[2][LQ_EDGES];        // 1: the neighbour is a successor (its in-degree counter)
+#endif
+#endif
+#if TRIM_ASYNC
   // asynchronous tail (see async_tail). The ring of row pieces in dynamic
   // shared memory: pieces taken out and put in so far. The idle workers (a bit
   // each), their wake-up barriers and the rows in their mailboxes. What the CTA does next (read by every worker
@@ -313,6 +332,44 @@ __device__ __forceinline__ uint32_t* w4_rows(const Cta& B, unsigned warp) {
 }
 __device__ __forceinline__ uint32_t w4_cap(const Cta& B) { return B.w4_wide ? 2u * LW : LW; }
 
+// One push from a removed vertex to its neighbour u: the predecessor's
+// live-successor counter. In+out trimming keeps both counters of a vertex in one
+// word (in-degree << 32 | out-degree); dir 1 pushes to a successor's in-degree
+// counter. The old word then tells at once whether this push removes u: its
+// counter went from one to zero and the other had not reached zero before (which
+// would have removed u already).
+#if TRIM_MODES & 16
+using PushWord = unsigned long long;
+__device__ __forceinline__ PushWord push(const Dev& D, uint32_t u, uint32_t dir) {
+  return atomicAdd(&D.cnt_io[u], dir ? 0ull - (1ull << 32) : ~0ull);
+}
+__device__ __forceinline__ bool push_removes(PushWord old, uint32_t dir) {
+  const uint32_t o = (uint32_t)old, i = (uint32_t)(old >> 32);
+  return dir ? i == 1u && o != 0u : o == 1u && i != 0u;
+}
+// the row of a vertex removed by pushes of direction dir, whose entries get pushes of the same one
+__device__ __forceinline__ const uint32_t* push_off(const Dev& D, uint32_t dir) {
+  return dir ? D.off : D.ioff;
+}
+__device__ __forceinline__ const uint32_t* push_tgt(const Dev& D, uint32_t dir) {
+  return dir ? D.tgt : D.itgt;
+}
+// stats runs: the in-edges and out-edges of a removed vertex
+__device__ __forceinline__ void count_rows(const Dev& D, bool removed, uint32_t u, Counters& K) {
+  if (!(D.flags & F_STATS) || !removed) return;
+  K.pushed += __ldg(&D.ioff[u + 1]) - __ldg(&D.ioff[u]);
+  K.edges += __ldg(&D.off[u + 1]) - __ldg(&D.off[u]);
+}
+#else
+using PushWord = uint32_t;
+__device__ __forceinline__ PushWord push(const Dev& D, uint32_t u, uint32_t) {
+  return atomicSub(&D.cnt[u], 1u);
+}
+__device__ __forceinline__ bool push_removes(PushWord old, uint32_t) { return old == 1u; }
+__device__ __forceinline__ const uint32_t* push_off(const Dev& D, uint32_t) { return D.ioff; }
+__device__ __forceinline__ const uint32_t* push_tgt(const Dev& D, uint32_t) { return D.itgt; }
+#endif
+
 // Warp-collective: copies this warp's slices to global memory at the given bases.
 __device__ __forceinline__ void copy_slices(const Dev& D, const Cta& B, const WarpSlice& w,
                                             unsigned warp, uint32_t* live_out) {
@@ -331,10 +388,7 @@ __device__ __forceinline__ void copy_slices(const Dev& D, const Cta& B, const Wa
       ee = w.edge_base + (i + 1 < w.nw4 ? se[i + 1] : w.nedge);
       D.w4_row[w.w4_base + i] = sr[i];
       D.w4_eoff[w.w4_base + i] = eo;
-      if (MODES & M_INOUT) {  // in+out entries: in-degree in slice 0, G row in slice 3
-        D.w4_din[w.w4_base + i] = sl[i];
-        D.w4_orow[w.w4_base + i] = sv[i];
-      }
+      if (MODES & M_INOUT) D.w4_dir[w.w4_base + i] = sl[i];  // in+out: the row's direction
     }
     mark_chunks(D, has, w.w4_base + i, eo, ee);
   }
@@ -359,6 +413,12 @@ __device__ __noinline__ void warp_flush(uint32_t r, uint32_t* live_out) {
         &D.C->w4, (unsigned long long)w.nw4 | ((unsigned long long)w.nedge << 32));
     w.w4_base = (uint32_t)o;
     w.edge_base = (uint32_t)(o >> 32);
+    // (the words of in+out trimming stop a second removal of a vertex only if
+    // G^T is the transpose of G)
+    if ((MODES & M_INOUT) && w.w4_base + w.nw4 > D.n) {
+      set_error(D, TRIM_ERR_STATE, 0xD7);
+      w.nw4 = 0;
+    }
   }
   if (lane == 2 && w.nlive) {
     w.live_base = atomicAdd(&D.C->rs[r & 3].live_count, w.nlive);
@@ -451,58 +511,6 @@ __device__ __forceinline__ void append_dead(const Dev& D, Cta& B, bool pred, uin
   __syncwarp();
 }
 
-#if TRIM_MODES & 16
-// Warp-collective, in+out trimming: lanes with pred were removed in round r
-// (their level is already set). Each joins the work list with one entry whose
-// edge range covers its G^T row (row, din edges: the predecessors whose
-// out-degree counters it decrements) and then its G row (orow, dout edges: the
-// successors whose in-degree counters it decrements). Removals are only
-// counted in the dead log, never written: no variant of this flavour reads it.
-__device__ __forceinline__ void append_dead_io(const Dev& D, Cta& B, bool pred, uint32_t u,
-                                               uint32_t r, bool pre, uint32_t prow,
-                                               uint32_t pdin, uint32_t porow, uint32_t pdout) {
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  const unsigned mask = __ballot_sync(FULL, pred);
-  if (mask == 0u) return;
-  uint32_t row = 0, din = 0, orow = 0, dout = 0;
-  if (pred) {
-    if (pre) {
-      row = prow; din = pdin; orow = porow; dout = pdout;
-    } else {
-      row = __ldg(&D.ioff[u]);
-      din = __ldg(&D.ioff[u + 1]) - row;
-      orow = __ldg(&D.off[u]);
-      dout = __ldg(&D.off[u + 1]) - orow;
-    }
-  }
-  const bool w = pred && din + dout > 0u;
-  const unsigned wmask = __ballot_sync(FULL, w);
-  const unsigned k = __popc(mask), kw = __popc(wmask);
-  const unsigned ew = w ? din + dout : 0u;
-  const unsigned eincl = warp_incl_scan(ew);
-  const unsigned esum = __shfl_sync(FULL, eincl, 31);
-  WarpSlice& ws = B.ws[warp];
-  if (ws.nw4 + kw > w4_cap(B)) warp_flush(r, D.live0);
-  const uint32_t pw = ws.nw4, pe = ws.nedge;
-  const unsigned mdin = __reduce_max_sync(FULL, ew);
-  if (w) {
-    const unsigned at = pw + __popc(wmask & ((1u << lane) - 1u));
-    w4_rows(B, warp)[at] = row;
-    slice(warp, 2)[at] = pe + eincl - ew;
-    slice(warp, 0)[at] = din;
-    slice(warp, 3)[at] = orow;
-  }
-  __syncwarp();
-  if (lane == 0) {
-    ws.ncount += k;
-    ws.nw4 = pw + kw;
-    ws.nedge = pe + esum;
-    ws.max_din = max(ws.max_din, mdin);
-  }
-  __syncwarp();
-}
-#endif
-
 // Warp-collective append of survivors to the AC-3 output live list.
 __device__ __forceinline__ void append_live(const Dev& D, Cta& B, bool pred, uint32_t v,
                                             uint32_t r, uint32_t* out_list) {
@@ -520,11 +528,10 @@ __device__ __forceinline__ void append_live(const Dev& D, Cta& B, bool pred, uin
 }
 
 #if TRIM_LOCAL
-// Warp-collective: lanes with pred add a work-list entry (G^T row start, in-degree)
-// of a vertex that is already removed and counted (local queue entries handed
-// to the global work list when local rounds end).
+// Warp-collective: lanes with pred add a work-list entry (row start, length; in+out
+// trimming: and direction) of a vertex that is already removed and counted.
 __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint32_t row,
-                                          uint32_t din, uint32_t r) {
+                                          uint32_t din, uint32_t r, uint32_t dir) {
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
   const bool w = pred && din > 0u;
   const unsigned wmask = __ballot_sync(FULL, w);
@@ -541,6 +548,7 @@ __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint3
     const unsigned at = pw + __popc(wmask & ((1u << lane) - 1u));
     w4_rows(B, warp)[at] = row;
     slice(warp, 2)[at] = pe + eincl - ew;
+    if (MODES & M_INOUT) slice(warp, 0)[at] = dir;
   }
   __syncwarp();
   if (lane == 0) {
@@ -551,6 +559,21 @@ __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint3
   __syncwarp();
 }
 
+#if TRIM_MODES & 16
+// Warp-collective, in+out trimming: lanes with pred were removed in this round
+// (their level is already set) by pushes of direction dir; each joins the work list with
+// its row of that direction. Removals are only counted in the dead log, never
+// written: no variant of this flavour reads it.
+__device__ __forceinline__ void append_dead_io(const Dev& D, Cta& B, bool pred, uint32_t r,
+                                               uint32_t row, uint32_t len, uint32_t dir) {
+  const unsigned mask = __ballot_sync(FULL, pred);
+  if (mask == 0u) return;
+  append_w4(D, B, pred, row, len, r, dir);
+  if (lane_id() == 0) B.ws[threadIdx.x >> 5].ncount += __popc(mask);
+  __syncwarp();
+}
+#endif
+
 // Warp-collective, local rounds: lanes with pred remove u in round r (its G^T
 // row start and in-degree already loaded). A removal with at most LQ_DMAX
 // in-edges that fits this CTA's queue (buffer b) stays local: its G^T row is
@@ -560,7 +583,7 @@ __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint3
 // round as overflowing.
 __device__ __forceinline__ void local_append(const Dev& D, Cta& B, bool pred, uint32_t u,
                                              uint32_t r, uint32_t row, uint32_t din,
-                                             uint32_t b) {
+                                             uint32_t b, uint32_t dir, uint32_t cap) {
   const unsigned lane = lane_id();
   const unsigned mask = __ballot_sync(FULL, pred);
   if (mask == 0u) return;
@@ -579,28 +602,32 @@ __device__ __forceinline__ void local_append(const Dev& D, Cta& B, bool pred, ui
       old = atomicAdd(&B.lq_cnt[b], (unsigned long long)k | ((unsigned long long)esum << 32));
     old = __shfl_sync(FULL, old, 0);
     const uint32_t be = (uint32_t)old, bd = (uint32_t)(old >> 32);
-    if (be + k <= LQ_ENTRIES && bd + esum <= LQ_EDGES) {  // warp-uniform
+    if (be + k <= LQ_ENTRIES && bd + esum <= cap) {  // warp-uniform
       if (lane == 0) atomicMax(&B.lq_vend[b], be + k);
       if (want) {
         const uint32_t slot = be + __popc(wm & ((1u << lane) - 1u));
         B.lq_row[b][slot] = row;
-        B.lq_din[b][slot] = din;
+        B.lq_din[b][slot] = din | (dir << 31);
       }
       // predecessors: element j of the flattened rows belongs to the lane with
       // the largest exclusive prefix <= j; four loads in flight per lane
       for (uint32_t j0 = 0; j0 < esum; j0 += 128u) {
-        uint32_t t[4];
+        uint32_t t[4], to[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t j = j0 + (uint32_t)q * 32u + lane;
           const unsigned o = owner_of(excl, j);
           const uint32_t ro = __shfl_sync(FULL, row, o), xo = __shfl_sync(FULL, excl, o);
-          t[q] = j < esum ? __ldg(&D.itgt[ro + (j - xo)]) : 0u;
+          to[q] = (MODES & M_INOUT) ? __shfl_sync(FULL, dir, o) : 0u;
+          t[q] = j < esum ? __ldg(&push_tgt(D, to[q])[ro + (j - xo)]) : 0u;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t j = j0 + (uint32_t)q * 32u + lane;
           if (j < esum) B.lq_ids[b][bd + j] = t[q];
+#if TRIM_MODES & 16
+          if (j < esum) B.lq_dir[b][bd + j] = (uint8_t)to[q];
+#endif
         }
       }
     } else {
@@ -612,7 +639,11 @@ __device__ __forceinline__ void local_append(const Dev& D, Cta& B, bool pred, ui
     atomicAdd(&B.lq_k, (unsigned)__popc(mask & ~om));
     if (om) B.lq_ovf = 1u;
   }
+#if TRIM_MODES & 16
+  append_dead_io(D, B, ovf, r, row, din, dir);
+#else
   append_dead(D, B, ovf, u, r, D.live0, false, true, row, din);
+#endif
 }
 #endif
 
@@ -674,6 +705,10 @@ __device__ void flush_round(const Dev& D, Cta& B, uint32_t r, uint32_t* live_out
       w.edge_base = eb + ic - c;
       w.live_base = vb + id - d;
       if (lb == 0xFFFFFFFFu) w.nlog = 0;
+      if ((MODES & M_INOUT) && wb + tb > D.n) {  // as in warp_flush
+        set_error(D, TRIM_ERR_STATE, 0xD7);
+        w.nw4 = 0;
+      }
       if (vb == 0xFFFFFFFFu) w.nlive = 0;
     }
   }
@@ -1204,7 +1239,8 @@ void local_leave(uint32_t b, uint32_t r) {
   for (uint32_t i0 = (threadIdx.x >> 5) * 32u; i0 < ne; i0 += blockDim.x) {
     const uint32_t i = i0 + lane;
     const bool has = i < ne;
-    append_w4(D, B, has, has ? B.lq_row[b][i] : 0u, has ? B.lq_din[b][i] : 0u, r);
+    const uint32_t len = has ? B.lq_din[b][i] : 0u;  // (in+out: direction in the top bit)
+    append_w4(D, B, has, has ? B.lq_row[b][i] : 0u, len & 0x7FFFFFFFu, r, len >> 31);
   }
   flush_round(D, B, r, D.live0);
   if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0 && threadIdx.x == 0)
@@ -1273,6 +1309,7 @@ __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   L.fe += nF;
 }
 
+#if TRIM_ASYNC
 // The asynchronous tail (see below) takes a level's vertices one to a warp, so it starts once there are
 // about as many workers as vertices. Measured on deep cascades (ms, tail from
 // round 128 against rounds; 4,560 workers): 4,096 chains of 2,867 6.8 against
@@ -1282,6 +1319,7 @@ __device__ __forceinline__ uint32_t async_workers() { return gridDim.x * ((block
 __device__ __forceinline__ bool async_few(uint32_t vertices) {
   return 10ull * vertices <= 13ull * async_workers();
 }
+#endif
 
 // End of local round r (all threads): one arrival per CTA on the barrier word
 // of this round's parity, carrying 2^48 + 2^32 * (overflowed) + the CTA's local
@@ -1327,9 +1365,12 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     // the stretch ends before the last round of a committed stretch (the
     // scheduler reads its features) and, where the asynchronous tail may take
     // over (asked every ASYNC_RETRY rounds), as it starts from the work list
-    const bool stop = ((MODES & M_SCHED) && r + 1u >= S.cstop) ||
-                      (D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
-                       r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u && async_few(nF));
+    const bool stop = ((MODES & M_SCHED) && r + 1u >= S.cstop)
+#if TRIM_ASYNC
+                      || (D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
+                       r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u && async_few(nF))
+#endif
+        ;
     if (n_ovf == 0u && (nF == 0u || !stop)) {
       local_close(D, B, nF);  // every removal of the round is in the queues
       B.lq_next = nF ? LQ_GO : LQ_DONE;
@@ -1351,9 +1392,14 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
 
 // Runs local rounds from round B.S.round on: the first pushes the pending
 // work-list entries (one per warp), later ones the predecessors in the CTA's
-// queue; every decrement loads the G^T row bounds of its vertex alongside the
-// atomic, so a removal costs no further dependent load before its row is
-// queued. The stretch ends when a round removes nothing (the run is done),
+// queue. A removed vertex's row bounds are loaded once its counter has reached
+// zero, not alongside every decrement: one more dependent load per round, but
+// one random access per push instead of two, and large rounds are bound by
+// those (kernel ms, rounds only, late against alongside: in+out of 2^23
+// vertices 6.73 and 7.25, AC-4 of 2^24 12.4 and 12.8, of 2^20 1.205 and 1.222, of
+// 2^16 1.005 and 1.015). Up to LQ_LATE_MIN vertices the offsets stay in every
+// SM's L1, and the bounds come alongside (1,000 vertices: 0.0539 against 0.0549).
+// The stretch ends when a round removes nothing (the run is done),
 // when a round overflowed the queues, or (with the schedulers) before the last
 // round of the committed stretch; in the last
 // two cases the queued vertices join the global work list and the round ends
@@ -1364,11 +1410,22 @@ __device__ __noinline__ bool local_stretch() {
   Cta& B = cta_state;
   Counters K;
   const unsigned lane = lane_id();
+  // A CTA may queue LQ_SKEW times the stretch's mean load at its start: past that
+  // every round waits for the fullest CTAs (a removal goes to the CTA that pushed
+  // last, often one that lags), and the ordinary round that an overflow brings
+  // (about 12 us) spreads the work evenly again. Kernel ms, with the bound and
+  // with queues filled to LQ_EDGES: in+out of 2^23 vertices 6.73 and 7.52, of 2^20
+  // 1.354 and 1.510; AC-4 of 2^24 (rounds only) 12.4 and 13.2, of 2^20 1.205 and
+  // 1.283; 256 packed graphs 0.616 and 0.601. Multiples of 2 to 6 on an in+out
+  // cascade of 5,000,011: 4.61, 4.45, 4.54, 4.68, 4.85 (2: packed graphs 0.84).
+  const float mean = __fdividef((float)(B.S.e_end - B.S.e_c4), (float)gridDim.x);
+  const uint32_t cap = min(LQ_EDGES, max(LQ_FLOOR, (uint32_t)((float)LQ_SKEW * mean)));
+  const bool late = D.n > LQ_LATE_MIN;
   bool first = true;
   while (true) {
     const uint32_t r = B.S.round;
     const uint32_t b = B.S.lround & 1u;
-    const bool check = B.S.mixed;
+    [[maybe_unused]] const bool check = B.S.mixed;
     start_round(D, r);
     if (first) {
       const uint32_t ia = B.S.c4w, ib = B.S.w_end, eb = B.S.e_end;
@@ -1377,43 +1434,71 @@ __device__ __noinline__ bool local_stretch() {
         const uint32_t row = ldcg(&D.w4_row[j]);
         const uint32_t eo = ldcg(&D.w4_eoff[j]);
         const uint32_t ee = (j + 1u < ib) ? ldcg(&D.w4_eoff[j + 1u]) : eb;
+        const uint32_t dir = (MODES & M_INOUT) ? ldcg(&D.w4_dir[j]) : 0u;
         for (uint32_t k0 = eo; k0 < ee; k0 += 32u) {
           const uint32_t e = k0 + lane;
           const bool valid = e < ee;
-          const uint32_t u = valid ? __ldg(&D.itgt[row + (e - eo)]) : 0u;
-          const uint32_t p0 = valid ? __ldg(&D.ioff[u]) : 0u;
-          const uint32_t p1 = valid ? __ldg(&D.ioff[u + 1u]) : 0u;
-          const uint32_t old = valid ? atomicSub(&D.cnt[u], 1u) : 0u;
+          const uint32_t u = valid ? __ldg(&push_tgt(D, dir)[row + (e - eo)]) : 0u;
+          uint32_t p0 = 0u, p1 = 0u;
+          if (valid && !late) {
+            p0 = __ldg(&push_off(D, dir)[u]);
+            p1 = __ldg(&push_off(D, dir)[u + 1u]);
+          }
+          const PushWord old = valid ? push(D, u, dir) : 0u;
+          bool pred = valid && push_removes(old, dir);
+#if TRIM_MODES & 16
+          count_rows(D, pred, u, K);
+#else
           K.pushed += valid ? 1u : 0u;
-          bool pred = valid && old == 1u;
           if (pred && check) pred = ldcg(&D.level[u]) == LIVE;
-          local_append(D, B, pred, u, r, p0, p1 - p0, b);
+#endif
+          if (pred && late) {
+            p0 = __ldg(&push_off(D, dir)[u]);
+            p1 = __ldg(&push_off(D, dir)[u + 1u]);
+          }
+          local_append(D, B, pred, u, r, p0, p1 - p0, b, dir, cap);
         }
       }
     } else {
       const uint32_t qb = b ^ 1u;
       const uint32_t qe = (uint32_t)(B.lq_cnt[qb] >> 32);
       for (uint32_t base = 0; base < qe; base += 2u * blockDim.x) {  // CTA-uniform
-        uint32_t u[2], p0[2], p1[2], old[2];
+        uint32_t u[2], p0[2], p1[2], dir[2];
+        PushWord old[2];
         bool valid[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const uint32_t k = base + (uint32_t)q * blockDim.x + threadIdx.x;
           valid[q] = k < qe;
           u[q] = valid[q] ? B.lq_ids[qb][k] : 0u;
+          dir[q] = 0u;
+#if TRIM_MODES & 16
+          dir[q] = valid[q] ? B.lq_dir[qb][k] : 0u;
+#endif
         }
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          p0[q] = valid[q] ? __ldg(&D.ioff[u[q]]) : 0u;
-          p1[q] = valid[q] ? __ldg(&D.ioff[u[q] + 1u]) : 0u;
-          old[q] = valid[q] ? atomicSub(&D.cnt[u[q]], 1u) : 0u;
+          p0[q] = p1[q] = 0u;
+          if (valid[q] && !late) {
+            p0[q] = __ldg(&push_off(D, dir[q])[u[q]]);
+            p1[q] = __ldg(&push_off(D, dir[q])[u[q] + 1u]);
+          }
+          old[q] = valid[q] ? push(D, u[q], dir[q]) : 0u;
         }
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
+          bool pred = valid[q] && push_removes(old[q], dir[q]);
+#if TRIM_MODES & 16
+          count_rows(D, pred, u[q], K);
+#else
           K.pushed += valid[q] ? 1u : 0u;
-          bool pred = valid[q] && old[q] == 1u;
           if (pred && check) pred = ldcg(&D.level[u[q]]) == LIVE;
-          local_append(D, B, pred, u[q], r, p0[q], p1[q] - p0[q], b);
+#endif
+          if (pred && late) {
+            p0[q] = __ldg(&push_off(D, dir[q])[u[q]]);
+            p1[q] = __ldg(&push_off(D, dir[q])[u[q] + 1u]);
+          }
+          local_append(D, B, pred, u[q], r, p0[q], p1[q] - p0[q], b, dir[q], cap);
         }
       }
       if (threadIdx.x == 0) B.lq_pushed = qe;
@@ -1436,6 +1521,8 @@ __device__ __noinline__ bool local_stretch() {
   return B.err == 0u;
 }
 
+#endif  // TRIM_LOCAL
+#if TRIM_ASYNC
 // ------------------------------------------------------- asynchronous AC-4 tail
 //
 // A vertex's level is one more than the top level among its successors
@@ -2354,13 +2441,20 @@ __device__ __noinline__ bool async_tail() {
 // ------------------------------------------------------------------ in+out
 
 // In+out round r (Section 4's remark: with G^T loaded a vertex also needs a
-// live incoming edge): every vertex removed before round r and not yet pushed
-// decrements the out-degree counter of each predecessor (its G^T row) and the
-// in-degree counter of each successor (its G row). A counter that reaches zero
-// removes its vertex in round r unless the vertex is already removed; when
-// both of a vertex's counters reach zero in the same round, the first
-// compare-and-swap of its level wins. Edges are balanced over the warps in
+// live incoming edge). A vertex whose out-degree counter reached zero has only
+// removed successors left, so its G row has no live vertex and only its G^T row is
+// pushed (the predecessors' out-degree counters); one whose in-degree counter
+// reached zero has only removed predecessors, and only its G row is pushed (the
+// successors' in-degree counters). So every work-list entry has one row and its direction,
+// half the pushes of walking both. A counter that reaches zero removes its
+// vertex in round r unless the other counter had removed it before: both are in
+// one word, and the push sees both. Edges are balanced over the warps in
 // 32-edge chunks as in ac4_round.
+//
+// Measured (ms per run, deep cascades of 5,000,011 vertices and 1,001 rounds /
+// 2^20 and 501 / 2^22 and 151): 4.26 / 2.0 / 1.4 with local rounds; before, with
+// both rows pushed, a compare-and-swap of the level and every round through the
+// global lists, 7.94 / 3.79 / 1.76.
 __device__ ROUND_FN void inout_round(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
                                      uint32_t nwarps) {
   constexpr int U = 4;
@@ -2376,8 +2470,9 @@ __device__ ROUND_FN void inout_round(const Dev& D, Cta& B, const Sched& S, uint3
   for (uint32_t c = cb; c < ce; c += U) {
     const uint32_t k = (c - cb) & 31u;
     if (k == 0u) cfb = (c + lane < ce) ? ldcg(&D.chunk_first[c + lane]) : 0u;
-    uint32_t wrow[U], weo[U], worow[U], wdin[U], u[U], old[U];
-    bool valid[U], pred_in[U];
+    uint32_t wrow[U], weo[U], wdir[U], u[U];
+    PushWord old[U];
+    bool valid[U];
 #pragma unroll
     for (int q = 0; q < U; ++q) {
       const uint32_t first = max(__shfl_sync(FULL, cfb, (k + q) & 31u), ia);
@@ -2385,29 +2480,30 @@ __device__ ROUND_FN void inout_round(const Dev& D, Cta& B, const Sched& S, uint3
       const bool in = c + q < ce && ii < ib;
       wrow[q] = in ? ldcg(&D.w4_row[ii]) : 0u;
       weo[q] = in ? ldcg(&D.w4_eoff[ii]) : 0xFFFFFFFFu;
-      worow[q] = in ? ldcg(&D.w4_orow[ii]) : 0u;
-      wdin[q] = in ? ldcg(&D.w4_din[ii]) : 0u;
+      wdir[q] = in ? ldcg(&D.w4_dir[ii]) : 0u;
     }
 #pragma unroll
     for (int q = 0; q < U; ++q) {
       const uint32_t e = ((c + q) << 5) + lane;
       valid[q] = c + q < ce && e >= ea && e < eb;
       const unsigned j = owner_of(weo[q], e);
-      const uint32_t kk = e - __shfl_sync(FULL, weo[q], j);
-      const uint32_t dj = __shfl_sync(FULL, wdin[q], j);
-      const uint32_t rj = __shfl_sync(FULL, wrow[q], j), oj = __shfl_sync(FULL, worow[q], j);
-      pred_in[q] = kk < dj;  // the edge lies in the entry's G^T row
-      u[q] = !valid[q] ? 0u : pred_in[q] ? __ldg(&D.itgt[rj + kk]) : __ldg(&D.tgt[oj + (kk - dj)]);
+      const uint32_t at = __shfl_sync(FULL, wrow[q], j) + (e - __shfl_sync(FULL, weo[q], j));
+      wdir[q] = __shfl_sync(FULL, wdir[q], j);
+      u[q] = valid[q] ? __ldg(&push_tgt(D, wdir[q])[at]) : 0u;
     }
 #pragma unroll
-    for (int q = 0; q < U; ++q)
-      old[q] = valid[q] ? atomicSub(pred_in[q] ? &D.cnt[u[q]] : &D.cnt_in[u[q]], 1u) : 0u;
+    for (int q = 0; q < U; ++q) old[q] = valid[q] ? push(D, u[q], wdir[q]) : 0u;
 #pragma unroll
     for (int q = 0; q < U; ++q) {
-      K.pushed += (valid[q] && pred_in[q]) ? 1 : 0;
-      K.edges += (valid[q] && !pred_in[q]) ? 1 : 0;
-      const bool pred = valid[q] && old[q] == 1u && atomicCAS(&D.level[u[q]], LIVE, r) == LIVE;
-      append_dead_io(D, B, pred, u[q], r, false, 0u, 0u, 0u, 0u);
+      const bool pred = valid[q] && push_removes(old[q], wdir[q]);
+      uint32_t row = 0, len = 0;
+      if (pred) {
+        row = __ldg(&push_off(D, wdir[q])[u[q]]);
+        len = __ldg(&push_off(D, wdir[q])[u[q] + 1u]) - row;
+        D.level[u[q]] = r;
+      }
+      count_rows(D, pred, u[q], K);
+      append_dead_io(D, B, pred, r, row, len, wdir[q]);
     }
   }
   stats_flush(D, B, K);
@@ -2665,8 +2761,11 @@ __device__ ROUND_FN void init_round(const Dev& D, Cta& B, uint32_t gwarp, uint32
   constexpr int U = 4;
   const unsigned lane = lane_id();
   const uint32_t n = D.n;
-  const bool w4 = (D.flags & F_AC4_POSSIBLE) != 0;
+  [[maybe_unused]] const bool w4 = (D.flags & F_AC4_POSSIBLE) != 0;
   const bool rows = D.ioff != nullptr;
+#if TRIM_MODES & 16
+  Counters K;
+#endif
   for (uint32_t base = gwarp * (32u * U); base < n; base += nwarps * (32u * U)) {
     uint32_t o0[U], o1[U], i0[U], i1[U];
 #pragma unroll
@@ -2706,10 +2805,11 @@ __device__ ROUND_FN void init_round(const Dev& D, Cta& B, uint32_t gwarp, uint32
       const uint32_t din = i1[q] - i0[q];
       if (has) {
         D.level[v] = (d && din) ? LIVE : 0u;
-        D.cnt[v] = d;
-        D.cnt_in[v] = din;
+        D.cnt_io[v] = ((unsigned long long)din << 32) | d;
       }
-      append_dead_io(D, B, has && (d == 0u || din == 0u), v, 0u, true, i0[q], din, o0[q], d);
+      const bool dies = has && (d == 0u || din == 0u);
+      if (dies) K.pushed += din, K.edges += d;
+      append_dead_io(D, B, dies, 0u, d ? o0[q] : i0[q], d ? d : din, d ? 1u : 0u);
 #else
       if (has) {
         D.level[v] = d ? LIVE : 0u;
@@ -2719,6 +2819,9 @@ __device__ ROUND_FN void init_round(const Dev& D, Cta& B, uint32_t gwarp, uint32
 #endif
     }
   }
+#if TRIM_MODES & 16
+  stats_flush(D, B, K);
+#endif
 }
 
 #if !(TRIM_MODES & 48)
@@ -3003,11 +3106,13 @@ __global__ void __launch_bounds__(512, TRIM_MIN_BLOCKS) TRIM_KERNEL(const __grid
       break;
     }
 #if TRIM_LOCAL
+#if TRIM_ASYNC
     if (async_start(D, S)) {
       if (!async_tail()) break;
       fresh = false;  // done: the tail ran the rest of the run
       continue;
     }
+#endif
     if (local_start(D, S)) {
       if (!local_stretch()) break;
       fresh = false;  // done, or the stretch's last round already ran advance()
