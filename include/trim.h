@@ -118,11 +118,12 @@ typedef struct {
                                  with TRIM_ERR_TIMEOUT                                       */
   float heur_push_ratio;      /* heuristic: push while sum(indeg F) < ratio * n_live        */
   float heur_ac6_ratio;       /* heuristic (no G^T): AC-6 while |F| < ratio * n_live        */
-  uint32_t local_round_edges; /* AC-4 and in+out kernels: once the in-edges still to push fit a
+  uint32_t local_round_edges; /* AC-4, AC-6 and in+out kernels: once the edges still to push fit a
                                  small round (at most this many, one work-list entry per
                                  warp), rounds run CTA-locally: each CTA queues the vertices
                                  it removes in shared memory and pushes them itself in the
-                                 next round, and a round ends at one barrier that carries
+                                 next round (AC-6: re-scans their sets; at most one to a warp
+                                 to start with), and a round ends at one barrier that carries
                                  its totals; a round whose removals overflow the queues
                                  returns to ordinary rounds (0 = never local)            */
   float sched_commit_confidence; /* LEARNED: a choice whose softmax probability (among the
@@ -164,8 +165,8 @@ typedef struct {
   uint32_t n_dead;          /* vertices removed                                          */
   float device_ms;          /* trim time between events around the device work          */
   uint64_t edges_inspected; /* TRIM_FLAG_STATS: out-edge targets read by AC-6/AC-3 scans.
-                               Scans read targets in groups (4 per thread step, up to 32
-                               per warp step) and a scan that resumes after its support
+                               Scans read targets in groups (one for the first successor, 4
+                               per thread step, up to 32 per warp step) and a scan that resumes after its support
                                reads again the targets its last group loaded past it, so
                                the count can exceed m for AC-6, whose logical inspections
                                are at most m (Section 8)                                */
@@ -175,7 +176,7 @@ typedef struct {
   uint32_t rounds_by_variant[3]; /* rounds run by AC-4, AC-6, AC-3                         */
   uint32_t segments;        /* persistent-kernel launches of the run (1 unless a scheduled
                                trim_run switched between variant kernels)               */
-  uint32_t local_rounds;    /* AC-4 rounds that ran CTA-locally (see local_round_edges)   */
+  uint32_t local_rounds;    /* rounds that ran CTA-locally (see local_round_edges)        */
   uint32_t launches;        /* kernel launches of the run: the control-block reset, every
                                segment, a continuation launch, a dead-mask pass          */
   uint32_t async_round;     /* round from which the run was asynchronous (0: never; see

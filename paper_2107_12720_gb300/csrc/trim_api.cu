@@ -47,6 +47,7 @@ struct trim_ctx {
   uint4* aw = nullptr;
   uint32_t *oq_row = nullptr, *oq_len = nullptr, *oq_lev = nullptr;
   uint32_t oq_cap = 0;
+  uint4* s_rec = nullptr;
   uint32_t *ae_id = nullptr, *ae_lev = nullptr;
   uint32_t ae_cap = 0;
   uint32_t *er_row = nullptr, *er_len = nullptr, *er_lev = nullptr;
@@ -612,15 +613,19 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   const bool in_host = gi && gi->on_device == TRIM_MEM_HOST;
   const size_t a_ioff = in_host ? A.add<uint32_t>(n + 1) : 0;
   const size_t a_itgt = in_host ? A.add<uint32_t>(c->m) : 0;
-  const size_t a_level = A.add<uint32_t>(n), a_cnt = A.add<uint32_t>(n);
-  // (next to each other: together they hold the asynchronous tail's 16 bytes per vertex)
+  const size_t a_level = A.add<uint32_t>(n);
+  // (next to each other: cnt to s_next hold the 16-byte records of a run of AC-6
+  // alone, supp to s_list the asynchronous tail's)
+  const size_t a_cnt = A.add<uint32_t>(n);
   const size_t a_supp = A.add<uint32_t>(n), a_shead = A.add<uint32_t>(n);
   const size_t a_snext = A.add<uint32_t>(n), a_slist = A.add<uint32_t>(n);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_log = A.add<uint32_t>(n);
-  const size_t a_roff = A.add<uint32_t>(n + 2), a_live0 = A.add<uint32_t>(n);
-  const size_t a_live1 = A.add<uint32_t>(n), a_bsum = A.add<uint32_t>(8192);
+  const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
   const size_t a_ctrl = A.add<Ctrl>(1);
+  // (next to each other: together they hold the four list heads per vertex of a
+  // run of AC-6 alone)
+  const size_t a_live0 = A.add<uint32_t>(n), a_live1 = A.add<uint32_t>(n);
   const size_t a_w4r = A.add<uint32_t>(n), a_w4e = A.add<uint32_t>(n);
   const size_t a_chunk = A.add<uint32_t>((c->m >> 5) + 2);
   const size_t a_rlog = c->rlog_cap ? A.add<trim_round_rec_t>(c->rlog_cap) : 0;
@@ -661,6 +666,7 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   c->live0 = at(a_live0); c->live1 = at(a_live1); c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
   c->aw = reinterpret_cast<uint4*>(c->supp);
+  c->s_rec = reinterpret_cast<uint4*>(c->cnt);
   c->w4_row = at(a_w4r); c->w4_eoff = at(a_w4e); c->chunk_first = at(a_chunk);
   if (c->rlog_cap) c->rlog = reinterpret_cast<trim_round_rec_t*>(base + a_rlog);
   if (flags & TRIM_FLAG_VALIDATE) TRY(validate(c, gi ? c->ioff : nullptr));
@@ -699,21 +705,23 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   const size_t n = c->n;
   if (flags & TRIM_FLAG_ROUND_LOG) c->rlog_cap = (uint32_t)std::min<uint64_t>(n + 1, 1u << 20);
   ArenaPlan A;
-  const size_t a_level = A.add<uint32_t>(n), a_supp = A.add<uint32_t>(n);
-  const size_t a_shead = A.add<uint32_t>(n), a_snext = A.add<uint32_t>(n);
+  // records of 16 bytes (AC-3: its support positions), AC-6's sets, and four list
+  // heads per vertex (AC-3: its live lists)
+  const size_t a_level = A.add<uint32_t>(n), a_rec = A.add<uint4>(n);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_slist = A.add<uint32_t>(n), a_log = A.add<uint32_t>(n);
-  const size_t a_roff = A.add<uint32_t>(n + 2), a_live0 = A.add<uint32_t>(n);
-  const size_t a_live1 = A.add<uint32_t>(n), a_bsum = A.add<uint32_t>(8192);
+  const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
+  const size_t a_heads = A.add<uint4>(n);
   const size_t a_ctrl = A.add<Ctrl>(1), a_m = A.add<unsigned long long>(1);
   const size_t a_rlog = c->rlog_cap ? A.add<trim_round_rec_t>(c->rlog_cap) : 0;
   char* base = nullptr;
   TRY(dalloc(c, &base, A.bytes));
   auto at = [&](size_t o) { return reinterpret_cast<uint32_t*>(base + o); };
-  c->level = at(a_level); c->supp = at(a_supp); c->cnt = nullptr;
-  c->s_head = at(a_shead); c->s_next = at(a_snext); c->s_cnt = at(a_scnt);
+  c->level = at(a_level); c->supp = at(a_rec); c->cnt = nullptr;
+  c->s_rec = reinterpret_cast<uint4*>(c->supp);
+  c->s_cnt = at(a_scnt);
   c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->roff = at(a_roff);
-  c->live0 = at(a_live0); c->live1 = at(a_live1); c->bsum = at(a_bsum);
+  c->live0 = at(a_heads); c->live1 = c->live0 + n; c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
   if (c->rlog_cap) c->rlog = reinterpret_cast<trim_round_rec_t*>(base + a_rlog);
   CK(cudaMemsetAsync(c->s_cnt, 0, n * 4, c->stream));
@@ -865,6 +873,10 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   else if (inout) flavour = kFlavourInout;
   else if (variant <= TRIM_AC3_PULL) flavour = (int)variant;
   else if (seg_flavour >= 0) flavour = seg_flavour;
+  if (variant == TRIM_AC6_SUPPORT) {  // AC-6 throughout
+    D.s_rec = c->s_rec;
+    D.s_heads = reinterpret_cast<uint4*>(c->live0);
+  }
   c->last_dev = D;
   const int grid = c->grids[flavour];
   if ((uint32_t)grid > 8192) return fail(c, TRIM_ERR_INVALID_ARG, "grid too large");

@@ -152,6 +152,11 @@ struct Dev {
   uint32_t* level;
   uint32_t* cnt;      // AC-4 out-degree counters
   uint32_t* supp;     // edge_index of AC-3 / AC-6: position of the current support
+  // runs of AC-6 alone: per vertex its record (next member of its list, next
+  // successor to try, its position, row end) and four list heads, in the arrays from
+  // cnt to s_next and from live0 to w4_eoff
+  uint4* s_rec;
+  uint4* s_heads;
   uint32_t* s_head;   // AC-6 supporting sets added during the epoch (intrusive lists)
   uint32_t* s_next;
   uint32_t* s_cnt;    // AC-6 bulk build: member counts per support (zero between builds)

@@ -111,16 +111,20 @@ struct WarpSlice {
 // In+out trimming (flavour 17) runs local rounds too: its queue holds, per
 // removed vertex, the one row that still matters (see inout_round), and per
 // queued neighbour which of its two counters the push decrements.
+// So does AC-6 (flavours 2 and 34, the ones that run nothing else): its queue
+// holds the removed vertices, whose supporting sets the CTA re-scans in the next
+// round.
 #if TRIM_MODES == 1 || TRIM_MODES == 9
 #define TRIM_LOCAL 1
 #define TRIM_ASYNC 1
-#elif TRIM_MODES == 17
+#elif TRIM_MODES == 17 || TRIM_MODES == 2 || TRIM_MODES == 34
 #define TRIM_LOCAL 1
 #define TRIM_ASYNC 0
 #else
 #define TRIM_LOCAL 0
 #define TRIM_ASYNC 0
 #endif
+#define TRIM_AC6_ONLY (TRIM_MODES == 2 || TRIM_MODES == 34)
 #if TRIM_LOCAL
 constexpr uint32_t LQ_EDGES = 1024;   // predecessors queued per CTA per round
 constexpr uint32_t LQ_ENTRIES = 256;  // removed vertices queued per CTA per round
@@ -152,11 +156,16 @@ struct Cta {
   unsigned long long kstat[4];  // TRIM_FLAG_STATS totals of this CTA (see stats_flush)
   uint32_t wbuf[MAX_WARPS][WBUF];
 #if TRIM_LOCAL
+#if TRIM_AC6_ONLY
+  // local AC-6 rounds: the vertices this CTA removed, by local-round parity
+  uint32_t lq_ids[2][LQ_ENTRIES];
+#else
   // local queues, double-buffered by local-round parity: buffer b is filled in
   // the round whose lround parity is b and read in the next one
   uint32_t lq_ids[2][LQ_EDGES];       // predecessors to decrement
   uint32_t lq_row[2][LQ_ENTRIES];     // the queued vertices' G^T rows ...
   uint32_t lq_din[2][LQ_ENTRIES];     // ... and in-degrees
+#endif
   unsigned long long lq_cnt[2];       // reserved: entries (low 32) | predecessors (high 32)
   uint32_t lq_vend[2];                // end of the reservations that fit (entries)
   uint32_t lq_k;                      // this round's removals kept local
@@ -527,7 +536,7 @@ __device__ __forceinline__ void append_live(const Dev& D, Cta& B, bool pred, uin
   __syncwarp();
 }
 
-#if TRIM_LOCAL
+#if TRIM_LOCAL && !TRIM_AC6_ONLY
 // Warp-collective: lanes with pred add a work-list entry (row start, length; in+out
 // trimming: and direction) of a vertex that is already removed and counted.
 __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint32_t row,
@@ -1221,6 +1230,7 @@ __device__ ROUND_FN void ac4_round(const Dev& D, Cta& B, const Sched& S, uint32_
 #if TRIM_LOCAL
 // ------------------------------------------------------------------ local AC-4 rounds
 
+#if !TRIM_AC6_ONLY
 // End of a local stretch that returns to ordinary rounds (all threads): the
 // queued vertices of round r (buffer b) become work-list entries, and the round
 // ends like an ordinary one (flush, grid barrier, advance). A rare path, out of
@@ -1249,17 +1259,24 @@ void local_leave(uint32_t b, uint32_t r) {
   if (threadIdx.x < 32) advance(D, B);
   __syncthreads();
 }
+#endif
 
 // Does round S.round start a stretch of local rounds? Its pending work-list
 // entries (the stretch's first round gives each warp whole entries) must have
 // at most local_edges_max in-edges in all, none more than 256.
 __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
+#if TRIM_AC6_ONLY
+  // AC-6: the sets were built, and the last round's removals are at most one to a warp
+  return S.prev_variant == TRIM_AC6_SUPPORT && S.variant == TRIM_AC6_SUPPORT &&
+         S.fe - S.fb <= min(D.local_edges_max, gridDim.x * (blockDim.x >> 5));
+#else
   if (D.local_edges_max == 0u || S.variant != TRIM_AC4_PUSH) return false;
   // with the schedulers: inside a committed stretch only, whose last round
   // (the one the scheduler reads features of) runs as an ordinary round
   if ((MODES & M_SCHED) && !(S.cstop != 0u && S.round + 1u < S.cstop)) return false;
   const uint32_t edges = S.e_end - S.e_c4;
   return edges <= D.local_edges_max && S.bmax <= 256u;
+#endif
 }
 
 // Thread 0: closes local round L.round, in which nF vertices were removed, all
@@ -1268,21 +1285,22 @@ __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
 __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   Sched& L = B.S;
   const uint32_t r = L.round;
-  L.vcount[TRIM_AC4_PUSH] += 1u;
+  constexpr uint32_t variant = TRIM_AC6_ONLY ? TRIM_AC6_SUPPORT : TRIM_AC4_PUSH;
+  L.vcount[variant] += 1u;
   L.c4w = L.w_end;  // the stretch's first round pushed every pending entry
   L.e_c4 = L.e_end;
   L.bmax = 0u;
   L.skew += nF;
   if (blockIdx.x == 0) {
     Ctrl* C = D.C;
-    C->vcount[TRIM_AC4_PUSH] = L.vcount[TRIM_AC4_PUSH];
+    C->vcount[variant] = L.vcount[variant];
     C->rounds = nF ? r + 1u : r;
     C->n_dead = L.fe + nF;
     C->local_rounds = L.lround;
     if ((D.flags & F_ROUND_LOG) && D.rlog != nullptr && r >= 1u && r - 1u < D.rlog_cap) {
       trim_round_rec_t* rec = &D.rlog[r - 1u];
       rec->round = r;
-      rec->variant = TRIM_AC4_PUSH;
+      rec->variant = variant;
       rec->frontier = L.fe - L.fb;
       rec->removed = nF;
       rec->t_start_ns = C->t_round[r & 3];
@@ -1302,7 +1320,7 @@ __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
     return;
   }
   L.stable = D.commit_after ? D.commit_after - 1u : 0u;  // as advance() in this flavour
-  L.prev_variant = TRIM_AC4_PUSH;
+  L.prev_variant = variant;
   L.fprev = L.fe - L.fb;
   L.round = r + 1u;
   L.fb = L.fe;
@@ -1340,7 +1358,9 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     const unsigned long long add =
         (1ull << 48) | ((unsigned long long)B.lq_ovf << 32) | (unsigned long long)B.lq_k;
     const unsigned long long base = S.lbase[slot];
-    // No fence before the arrival: across a local barrier CTAs exchange nothing
+    // AC-6 rounds hand levels, records and list heads to other CTAs.
+    if (TRIM_AC6_ONLY) fence_acq_rel();
+    // Otherwise no fence before the arrival: across a local barrier CTAs exchange nothing
     // through plain memory, only counter decrements, and every decrement of
     // this round has returned its value (it is performed at L2) before this
     // arrival is issued. Levels written here are read after the kernel or
@@ -1358,6 +1378,7 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       }
       cur = ld_relaxed64(&D.C->lbar[slot]);
     }
+    if (TRIM_AC6_ONLY) fence_acq_rel();
     const unsigned long long d = cur - base;
     S.lbase[slot] = cur;
     S.lround += 1u;
@@ -1375,7 +1396,9 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       local_close(D, B, nF);  // every removal of the round is in the queues
       B.lq_next = nF ? LQ_GO : LQ_DONE;
     } else {
-      S.skew += nF;  // advance() closes the round after the work-list handover
+      // advance() closes the round after the handover (AC-6: the queued removals
+      // join the dead log and are counted there)
+      if (!TRIM_AC6_ONLY) S.skew += nF;
       if (blockIdx.x == 0) D.C->local_rounds = S.lround;
       B.lq_next = LQ_LEAVE;
     }
@@ -1390,6 +1413,7 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
   return B.err == 0u;
 }
 
+#if !TRIM_AC6_ONLY
 // Runs local rounds from round B.S.round on: the first pushes the pending
 // work-list entries (one per warp), later ones the predecessors in the CTA's
 // queue. A removed vertex's row bounds are loaded once its counter has reached
@@ -1520,6 +1544,7 @@ __device__ __noinline__ bool local_stretch() {
   stats_flush(D, B, K);
   return B.err == 0u;
 }
+#endif
 
 #endif  // TRIM_LOCAL
 #if TRIM_ASYNC
@@ -2546,6 +2571,7 @@ __device__ ROUND_FN void ac3_round(const Dev& D, Cta& B, const Sched& S, uint32_
 
 // ------------------------------------------------------------------ AC-6
 
+#if !TRIM_AC6_ONLY
 // Warp-collective re-scan of members of a supporting set whose owner was
 // removed in round r-1: scan forward from the position after the lost support;
 // on success join the new support's set (intrusive list), else remove.
@@ -2568,6 +2594,8 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
   K.cand += valid ? 1 : 0;
   append_dead(D, B, dies, v, r, D.live0, false, false, 0, 0, d);
 }
+
+#endif
 
 // Block-wide exclusive scan of one value per thread (blockDim.x <= 1024).
 __device__ unsigned block_excl_scan(unsigned x, unsigned* total) {
@@ -2607,12 +2635,137 @@ __device__ unsigned block_sum(unsigned x) {
   return t;
 }
 
-// AC-6 entry (the first AC-6 round, or the first after another variant ran):
-// every live vertex re-checks its support position, joins the bulk supporting
-// set of the support it keeps (a counting sort by support: count, grid-wide
-// scan, scatter), or is removed. Three internal grid barriers.
-__device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
-                                   uint32_t nwarps) {
+#if TRIM_AC6_ONLY
+// The counters of the entry's counting sort are contended: on skewed graphs with
+// sorted rows the first successors of most vertices are a few hubs, and the atomics on
+// the hottest line alone took most of the pass. So each CTA counts in a table in
+// shared memory first (a slot belongs to the first support that hashes there;
+// others go to the global counter) and adds its totals to the global counters at
+// the end. A vertex keeps its rank (in its CTA's table, or globally), so the
+// scatter needs no atomics. The table lies in append slices that AC-6 does not use:
+// keys, counts, and the CTA's first rank of each support.
+constexpr uint32_t AC6_HEADS = 4;
+__device__ __forceinline__ uint32_t* set_head(const Dev& D, uint32_t w, uint32_t q) {
+  return reinterpret_cast<uint32_t*>(&D.s_heads[w]) + q;
+}
+__device__ __forceinline__ uint32_t sort_slots() { return (blockDim.x >> 5) * LW; }
+__device__ __forceinline__ uint32_t sort_slot(uint32_t t) {
+  return __umulhi(t * 0x9E3779B1u, sort_slots());
+}
+__device__ __forceinline__ uint32_t* sort_word(uint32_t slot, int which) {
+  return &slice(slot / LW, which)[slot % LW];
+}
+
+// First pass of the entry in the flavours that run AC-6 alone: every live vertex
+// looks for its support, is counted there and gets its record, or is removed. Each
+// lane has four vertices in flight, and checks their rows' first successors; the
+// vertices that must scan on (about one in eight) wait in a list until they
+// fill a warp.
+__device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, uint32_t gwarp,
+                                             uint32_t nwarps) {
+  constexpr int U = 4;
+  Counters K;
+  const unsigned lane = lane_id();
+  const uint32_t n = D.n;
+  for (uint32_t e = threadIdx.x; e < sort_slots(); e += blockDim.x) {
+    *sort_word(e, 1) = NIL;
+    *sort_word(e, 2) = 0u;
+  }
+  __syncthreads();
+  // counts v's support t: v's rank in the CTA's table or globally
+  auto count = [&](uint32_t t) -> uint32_t {
+    const uint32_t e = sort_slot(t);
+    uint32_t key = *const_cast<volatile uint32_t*>(sort_word(e, 1));
+    if (key == NIL) key = atomicCAS(sort_word(e, 1), NIL, t);
+    return atomicAdd(key == NIL || key == t ? sort_word(e, 2) : &D.s_cnt[t], 1u);
+  };
+  // (support and rank are parked in the link and, as the frontier offsets are read
+  // by nothing on the device, in roff until the scatter)
+  auto store = [&](uint32_t v, uint32_t t, uint32_t rank, uint32_t after, uint32_t pos,
+                   uint32_t end) {
+    D.s_rec[v] = make_uint4(t, after, pos, end);
+    D.roff[v] = rank;
+  };
+  uint32_t* list = slice(threadIdx.x >> 5, 3);  // at most 31 + 32 * U entries
+  uint32_t nl = 0;
+  for (uint32_t base = gwarp * (32u * U);; base += nwarps * (32u * U)) {
+    const bool last = base >= n;
+    if (!last) {
+      uint32_t s[U], d[U], t[U], after[U], x[U];
+      bool alive[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const uint32_t v = base + q * 32u + lane;
+        alive[q] = v < n && ldcg(&D.level[v]) == LIVE;
+        s[q] = d[q] = 0u;
+#if !(TRIM_MODES & 32)
+        if (v < n) row_bounds(D, v, s[q], d[q]);
+#endif
+        K.swept += v < n ? 1 : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {  // (a live vertex has a successor)
+        const uint32_t v = base + q * 32u + lane;
+#if TRIM_MODES & 32
+        if (alive[q]) row_bounds(D, v, s[q], d[q]);
+#endif
+        t[q] = alive[q] ? row_target(D, v, s[q], 0u) : 0u;
+        after[q] = alive[q] && d[q] > 1u ? row_target(D, v, s[q], 1u) : NIL;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        x[q] = alive[q] ? ldcg(&D.level[t[q]]) : 0u;
+        K.edges += alive[q] ? 1 : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const bool slow = alive[q] && x[q] < r;
+        const unsigned mask = __ballot_sync(FULL, slow);
+        if (slow) list[nl + __popc(mask & ((1u << lane) - 1u))] = base + q * 32u + lane;
+        nl += __popc(mask);
+        alive[q] = alive[q] && !slow;
+        x[q] = alive[q] ? count(t[q]) : 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (alive[q])
+          store(base + q * 32u + lane, t[q], x[q], after[q], s[q] + 1u, s[q] + d[q]);
+      __syncwarp();
+    }
+    while (nl >= 32u || (last && nl)) {
+      const uint32_t take = min(32u, nl);
+      const bool has = lane < take;
+      const uint32_t v = has ? list[nl - take + lane] : 0u;
+      __syncwarp();
+      nl -= take;
+      uint32_t s = 0, d = 0, i = 0;
+      bool resolved = true;
+      if (has) {
+        row_bounds(D, v, s, d);
+        i = scan_thread(D, v, s, d, 1u, r, 2, resolved, K);
+      }
+      scan_warp_finish(D, resolved, v, s, d, i, r, K);
+      const bool found = has && i < d;
+      if (found) {
+        const uint32_t t = row_target(D, v, s, i);
+        store(v, t, count(t), i + 1u < d ? row_target(D, v, s, i + 1u) : NIL, s + i + 1u, s + d);
+      } else if (has) {
+        D.s_heads[v] = make_uint4(NIL, NIL, NIL, NIL);
+      }
+      append_dead(D, B, has && !found, v, r, D.live0);
+    }
+    if (last) break;
+  }
+  __syncthreads();
+  for (uint32_t e = threadIdx.x; e < sort_slots(); e += blockDim.x) {
+    const uint32_t k = *sort_word(e, 2);
+    *sort_word(e, 3) = k ? atomicAdd(&D.s_cnt[*sort_word(e, 1)], k) : 0u;
+  }
+  stats_flush(D, B, K);
+}
+#else
+__device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
+                                             uint32_t nwarps) {
   Counters K;
   const unsigned lane = lane_id();
   const uint32_t r = S.round, n = D.n;
@@ -2640,13 +2793,45 @@ __device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_
     append_dead(D, B, dies, v, r, D.live0, false, false, 0, 0, d);
   }
   stats_flush(D, B, K);
+}
+#endif
+
+// AC-6 entry (the first AC-6 round, or the first after another variant ran):
+// every live vertex re-checks its support position, joins the bulk supporting
+// set of the support it keeps (a counting sort by support: count, grid-wide
+// scan, scatter), or is removed. Three internal grid barriers.
+//
+// Measured (R-MAT of 2^22 vertices, 1.8 million of them live, kernel us with AC-6
+// alone): 168 before, with every count and rank an atomic on the global counter and
+// one vertex per lane in flight; 124 now (four in flight alone 197 with the records,
+// the counting table 164, scans on in full warps 160, list heads written once 130).
+__device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
+                                   uint32_t nwarps) {
+  const unsigned lane = lane_id();
+  const uint32_t n = D.n;
+#if TRIM_AC6_ONLY
+  ac6_supports(D, B, S.round, gwarp, nwarps);
+#else
+  ac6_supports(D, B, S, gwarp, nwarps);
+#endif
   if (!grid_barrier(D, B)) return false;
-  // grid-wide exclusive scan of s_cnt into s_off
+  // grid-wide exclusive scan of s_cnt into s_off, four entries per thread and step
   const uint32_t chunk = ((n + gridDim.x - 1) / gridDim.x + 31) & ~31u;
   const uint32_t c0 = min(n, blockIdx.x * chunk), c1 = min(n, c0 + chunk);
+  auto counts = [&](uint32_t i) -> uint4 {  // entries i .. i+3, i a multiple of 4
+    if (i + 3u < c1) return __ldcg(reinterpret_cast<const uint4*>(&D.s_cnt[i]));
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (i < c1) x.x = ldcg(&D.s_cnt[i]);
+    if (i + 1u < c1) x.y = ldcg(&D.s_cnt[i + 1u]);
+    if (i + 2u < c1) x.z = ldcg(&D.s_cnt[i + 2u]);
+    return x;
+  };
   {
     unsigned acc = 0;
-    for (uint32_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) acc += ldcg(&D.s_cnt[i]);
+    for (uint32_t i = c0 + 4u * threadIdx.x; i < c1; i += 4u * blockDim.x) {
+      const uint4 x = counts(i);
+      acc += x.x + x.y + x.z + x.w;
+    }
     acc = block_sum(acc);
     if (threadIdx.x == 0) D.bsum[blockIdx.x] = acc;
   }
@@ -2655,34 +2840,359 @@ __device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_
     unsigned pre = 0;
     for (uint32_t j = threadIdx.x; j < blockIdx.x; j += blockDim.x) pre += ldcg(&D.bsum[j]);
     pre = block_sum(pre);
-    for (uint32_t t0 = c0; t0 < c1; t0 += blockDim.x) {
-      const uint32_t i = t0 + threadIdx.x;
-      const unsigned x = i < c1 ? ldcg(&D.s_cnt[i]) : 0u;
+    for (uint32_t t0 = c0; t0 < c1; t0 += 4u * blockDim.x) {
+      const uint32_t i = t0 + 4u * threadIdx.x;
+      const uint4 x = i < c1 ? counts(i) : make_uint4(0u, 0u, 0u, 0u);
       unsigned tot;
-      const unsigned ex = block_excl_scan(x, &tot);
-      if (i < c1) D.s_off[i] = pre + ex;
+      const unsigned ex = pre + block_excl_scan(x.x + x.y + x.z + x.w, &tot);
+      const uint4 o = make_uint4(ex, ex + x.x, ex + x.x + x.y, ex + x.x + x.y + x.z);
+      if (i + 3u < c1) {
+        *reinterpret_cast<uint4*>(&D.s_off[i]) = o;
+      } else {
+        if (i < c1) D.s_off[i] = o.x;
+        if (i + 1u < c1) D.s_off[i + 1u] = o.y;
+        if (i + 2u < c1) D.s_off[i + 2u] = o.z;
+      }
+#if TRIM_AC6_ONLY
+      // (the counters are zero between builds)
+      if (i + 3u < c1) {
+        *reinterpret_cast<uint4*>(&D.s_cnt[i]) = make_uint4(0u, 0u, 0u, 0u);
+      } else {
+        for (uint32_t j = i; j < c1; ++j) D.s_cnt[j] = 0u;
+      }
+#endif
       pre += tot;
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-      unsigned all = 0;
-      for (uint32_t j = 0; j < gridDim.x; ++j) all += ldcg(&D.bsum[j]);
-      D.s_off[n] = all;
-    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) D.s_off[n] = pre;
   }
   if (!grid_barrier(D, B)) return false;
-  for (uint32_t base = gwarp * 32; base < n; base += nwarps * 32) {
-    const uint32_t v = base + lane;
-    if (v < n && ldcg(&D.level[v]) == LIVE) {
-      const uint32_t t = ldcg(&D.s_next[v]);
-      const uint32_t left = atomicSub(&D.s_cnt[t], 1u);
-      const uint32_t pos = ldcg(&D.s_off[t]) + left - 1u;
-      if (left == 0u || pos >= n) set_error(D, TRIM_ERR_STATE, 0xD2);  // counts out of step
-      else D.s_list[pos] = v;
+  constexpr int U = 4;
+  for (uint32_t base = gwarp * (32u * U); base < n; base += nwarps * (32u * U)) {
+    uint32_t t[U], off[U], pos[U];
+    bool alive[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const uint32_t v = base + q * 32u + lane;
+      alive[q] = v < n && ldcg(&D.level[v]) == LIVE;
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const uint32_t v = base + q * 32u + lane;
+#if TRIM_AC6_ONLY
+      t[q] = alive[q] ? ldcg(&D.s_rec[v].x) : 0u;
+      pos[q] = alive[q] ? ldcg(&D.roff[v]) : 0u;
+#else
+      t[q] = alive[q] ? ldcg(&D.s_next[v]) : 0u;
+#endif
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      off[q] = alive[q] ? ldcg(&D.s_off[t[q]]) : 0u;
+#if !TRIM_AC6_ONLY
+      pos[q] = alive[q] ? atomicSub(&D.s_cnt[t[q]], 1u) - 1u : 0u;  // (back to zero)
+#endif
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      if (!alive[q]) continue;
+      const uint32_t v = base + q * 32u + lane;
+#if TRIM_AC6_ONLY
+      const uint32_t e = sort_slot(t[q]);
+      if (*sort_word(e, 1) == t[q]) pos[q] += *sort_word(e, 3);
+      D.s_heads[v] = make_uint4(NIL, NIL, NIL, NIL);
+#endif
+      pos[q] += off[q];
+      if (pos[q] >= n) set_error(D, TRIM_ERR_STATE, 0xD2);  // counts out of step
+      else D.s_list[pos[q]] = v;
     }
   }
   return true;
 }
 
+#if TRIM_AC6_ONLY
+// AC-6 rounds of the flavours that run nothing else. What bounds a deep run is the
+// chain of dependent random accesses in each round, so every vertex with a support
+// has a record of 16 bytes: the next member of its list, the successor to try when
+// its support goes (already read from the row, NIL at the row's end), that successor's
+// position and the row's end. A walk of a set finds all a re-scan needs in one
+// access per hop, and the vertex that dies (no successor left) needs no other. A
+// member that moves checks the successor's level, and reads its row's next entry
+// for the new record meanwhile. A vertex has four list heads, and members go to the
+// one that a hash of their id gives: the hops down a set run side by side (sets
+// of some tens of members in the first rounds of a deep graph).
+//
+// Measured (kernel ms per run, before: one list head, members' level, position and row
+// loaded one after the other, every round through the global lists): deep
+// cascades of 1,000,003 vertices and 1,503 rounds 16.7 and now 10.6, of 2^20 and 2,802
+// rounds 33.2 and 19.6, of 2^16 and 302 rounds 3.4 and 2.13. Without the records 13.7
+// (one head 17.3, two 14.6, sixteen 12.3); records and one general walk for all
+// rounds 13.1. A round is now 6.7 us: about 3.5 of it a walk and a move (a warp alone
+// on its scheduler takes 5 cycles an instruction, an access 400, an atomic 800), 0.65
+// the fence, 1.1 the barrier.
+
+// Warp-collective, local rounds: lanes with pred remove u in round r. The CTA
+// queues up to cap of them in buffer b; the others go to the dead log and mark
+// the round as overflowing.
+__device__ __forceinline__ void local_remove(const Dev& D, Cta& B, bool pred, uint32_t u,
+                                             uint32_t r, uint32_t b, uint32_t cap) {
+  const unsigned lane = lane_id();
+  const unsigned mask = __ballot_sync(FULL, pred);
+  if (mask == 0u) return;
+  const uint32_t k = __popc(mask);
+  uint32_t at = 0;
+  if (lane == 0) {
+    at = (uint32_t)atomicAdd(&B.lq_cnt[b], (unsigned long long)k);
+    if (at + k <= cap) {
+      atomicMax(&B.lq_vend[b], at + k);
+      atomicAdd(&B.lq_k, k);
+    } else {
+      B.lq_ovf = 1u;
+    }
+  }
+  at = __shfl_sync(FULL, at, 0);
+  if (at + k <= cap) {
+    if (pred) {
+      B.lq_ids[b][at + __popc(mask & ((1u << lane) - 1u))] = u;
+      D.level[u] = r;
+    }
+  } else {
+    append_dead(D, B, pred, u, r, D.live0);
+  }
+}
+
+// Warp-collective re-scan of members v of sets whose owner was removed in round
+// r - 1, from their records (next successor t at position pos of a row that
+// ends at end): the first live successor from there on takes them into its set,
+// without one they are removed.
+template <bool LOCAL>
+__device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uint32_t v, uint32_t t,
+                                           uint32_t pos, uint32_t end, uint32_t r, Counters& K,
+                                           uint32_t b, uint32_t cap) {
+  const bool cand = valid && t != NIL;
+  uint32_t lv = 0, after = NIL;
+  if (cand) {
+    lv = ldcg(&D.level[t]);
+    if (pos + 1u < end) after = row_target(D, v, 0u, pos + 1u);
+    K.edges += 1;
+  }
+  bool found = cand && lv >= r;
+  if (__any_sync(FULL, cand && !found)) {  // the rare case: scan on
+    uint32_t i = pos + 1u;
+    bool resolved = true;
+    if (cand && !found) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
+    scan_warp_finish(D, resolved, v, 0u, end, i, r, K);
+    if (cand && !found && i < end) {
+      found = true;
+      pos = i;
+      t = row_target(D, v, 0u, i);
+      after = i + 1u < end ? row_target(D, v, 0u, i + 1u) : NIL;
+    }
+  }
+  if (found) {
+    const uint32_t next = atomicExch(set_head(D, t, (v * 0x9E3779B1u) >> 30), v);
+    D.s_rec[v] = make_uint4(next, after, pos + 1u, end);
+  }
+  K.cand += valid ? 1 : 0;
+  const bool dies = valid && !found;
+  if (LOCAL) local_remove(D, B, dies, v, r, b, cap);
+  else append_dead(D, B, dies, v, r, D.live0);
+}
+
+// Warp-collective: re-scans the supporting sets of up to 32 removed vertices,
+// the w of lanes < G with has. Members are staged with their records, up to 64, in
+// an append slice that AC-6 does not use.
+__device__ __forceinline__ void ac6_sets(const Dev& D, Cta& B, bool has, uint32_t w, uint32_t G,
+                                         uint32_t r, Counters& K) {
+  const unsigned lane = lane_id();
+  uint4* st = reinterpret_cast<uint4*>(slice(threadIdx.x >> 5, 1));
+  // bulk members of S(w): contiguous, spread over the lanes
+  uint32_t ss = 0, sd = 0;
+  if (has) {
+    ss = ldcg(&D.s_off[w]);
+    sd = ldcg(&D.s_off[w + 1]) - ss;
+  }
+  uint32_t kb = 0, total = 0, excl = 0;
+  unsigned nbuf = 0;
+  for (unsigned q0 = 0; q0 < G * AC6_HEADS; q0 += 32) {
+    // members that joined S(w) during the epoch: 32 lists at a time
+    const unsigned j = (q0 + lane) / AC6_HEADS;  // below 32, as G is at most 32
+    const uint32_t wj = __shfl_sync(FULL, w, j);
+    const bool hj = __shfl_sync(FULL, has ? 1 : 0, j) != 0 && j < G;
+    uint32_t cur = hj ? ldcg(set_head(D, wj, lane % AC6_HEADS)) : NIL;
+    if (q0 == 0) {
+      const unsigned incl = warp_incl_scan(sd);
+      total = __shfl_sync(FULL, incl, 31);
+      excl = incl - sd;
+    }
+    unsigned steps = 0;
+    // bulk members, then the lists' (all walkers hop in step), are staged; re-scans
+    // run 32 at a time. A member's record is read before it can be re-scanned
+    // (and move to another set).
+    while (true) {
+      const unsigned wm = __ballot_sync(FULL, cur != NIL);
+      bool stage = false, hop = false;
+      uint32_t v = 0, at = nbuf + lane;
+      if (kb < total) {
+        const uint32_t k = kb + lane;
+        const unsigned o = G == 1 ? 0u : owner_of(excl, k);
+        const unsigned so = __shfl_sync(FULL, ss, o), eo = __shfl_sync(FULL, excl, o);
+        stage = k < total;
+        if (stage) v = ldcg(&D.s_list[so + (k - eo)]);
+        nbuf += min(32u, total - kb);
+        kb += 32u;
+      } else if (wm) {
+        if (++steps > D.n) {  // a set holds at most n members: longer means a broken list
+          if (lane == 0) set_error(D, TRIM_ERR_STATE, 0xD4);
+          return;
+        }
+        stage = hop = cur != NIL;
+        v = cur;
+        at = nbuf + __popc(wm & ((1u << lane) - 1u));
+        nbuf += __popc(wm);
+      } else if (nbuf == 0u) {
+        break;
+      }
+      if (stage) {
+        const uint4 x = __ldcg(&D.s_rec[v]);
+        if (hop) cur = x.x;
+        st[at] = make_uint4(v, x.y, x.z, x.w);
+      }
+      __syncwarp();
+      const bool more = __any_sync(FULL, cur != NIL) || kb < total;
+      while (nbuf >= 32u || (!more && nbuf > 0u)) {
+        const unsigned take = min(32u, nbuf);
+        const bool valid = lane < take;
+        const uint4 m = st[valid ? nbuf - take + lane : 0u];
+        __syncwarp();
+        nbuf -= take;
+        ac6_rescan<false>(D, B, valid, m.x, m.y, m.z, m.w, r, K, 0u, 0u);
+      }
+    }
+  }
+}
+
+// The same for the set of one removed vertex w in a local round. A warp that runs
+// alone on its scheduler pays for every instruction as well: this is the short form.
+__device__ __forceinline__ void ac6_set(const Dev& D, Cta& B, uint32_t w, uint32_t r, Counters& K,
+                                        uint32_t b, uint32_t cap) {
+  const unsigned lane = lane_id();
+  uint4* st = reinterpret_cast<uint4*>(slice(threadIdx.x >> 5, 1));
+  uint32_t cur = lane < AC6_HEADS ? ldcg(set_head(D, w, lane)) : NIL;
+  const uint32_t ss = ldcg(&D.s_off[w]), total = ldcg(&D.s_off[w + 1]) - ss;
+  uint32_t kb = 0, steps = 0;
+  unsigned nbuf = 0, wm = __ballot_sync(FULL, cur != NIL);
+  while (wm || kb < total) {
+    if (kb < total) {
+      if (kb + lane < total) {
+        const uint32_t v = ldcg(&D.s_list[ss + kb + lane]);
+        const uint4 x = __ldcg(&D.s_rec[v]);
+        st[nbuf + lane] = make_uint4(v, x.y, x.z, x.w);
+      }
+      nbuf += min(32u, total - kb);
+      kb += 32u;
+    } else {
+      if (cur != NIL) {
+        const uint4 x = __ldcg(&D.s_rec[cur]);
+        st[nbuf + __popc(wm & ((1u << lane) - 1u))] = make_uint4(cur, x.y, x.z, x.w);
+        cur = x.x;
+      }
+      nbuf += __popc(wm);
+      wm = __ballot_sync(FULL, cur != NIL);
+      if (++steps > D.n) {  // a set holds at most n members: longer means a broken list
+        if (lane == 0) set_error(D, TRIM_ERR_STATE, 0xD4);
+        return;
+      }
+    }
+    __syncwarp();
+    while (nbuf >= 32u || (nbuf && !wm && kb >= total)) {
+      const unsigned take = min(32u, nbuf);
+      const bool valid = lane < take;
+      const uint4 m = st[valid ? nbuf - take + lane : 0u];
+      __syncwarp();
+      nbuf -= take;
+      ac6_rescan<true>(D, B, valid, m.x, m.y, m.z, m.w, r, K, b, cap);
+    }
+  }
+}
+
+__device__ ROUND_FN bool ac6_round(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
+                                   uint32_t nwarps) {
+  if (S.prev_variant != TRIM_AC6_SUPPORT) return ac6_entry(D, B, S, gwarp, nwarps);
+  Counters K;
+  const unsigned lane = lane_id();
+  const uint32_t r = S.round;
+  const uint32_t N = S.fe - S.fb;
+  const uint32_t G = min(32u, max(1u, (N + nwarps - 1) / nwarps));
+  for (uint32_t base = S.fb + gwarp * G; base < S.fe; base += nwarps * G) {
+    const uint32_t item = base + lane;
+    const bool has = lane < G && item < S.fe;
+    const uint32_t w = has ? ldcg(&D.log[item - S.skew]) : 0u;  // (as in the other ac6_round)
+    ac6_sets(D, B, has, w, G, r, K);
+  }
+  stats_flush(D, B, K);
+  return true;
+}
+
+// Local AC-6 rounds, from round B.S.round on: the first takes the removals of the
+// last round from the dead log, one to a warp, later ones the CTA's own queue. A
+// round needs no log, no space reservation and no read of the control block; it
+// ends at a fenced local barrier that carries its totals (the fence covers
+// levels, records and heads). The stretch ends when nothing was removed (the run
+// is done) or a queue overflowed; then the queued vertices join the dead log and
+// the round ends like an ordinary one. The queues are bounded by a few times the
+// mean load, at least LQ_SETS: a CTA has a warp for each of 16 sets, but removals drift
+// to few CTAs (a vertex stays with the set it leaves last). Bounds of 32, 8 and 4, ms: 11.8,
+// 10.7 and 11.1 (1,000,003 vertices), 24.3, 19.6 and 19.8 (2^20, 2,802 rounds). Returns
+// false on a timeout.
+constexpr uint32_t LQ_SETS = 8;  // least bound of the queues
+__device__ __noinline__ bool local_stretch() {
+  const Dev& D = cta_dev;
+  Cta& B = cta_state;
+  Counters K;
+  const unsigned lane = lane_id();
+  const uint32_t cap = min(LQ_ENTRIES, max(LQ_SETS, LQ_SKEW * ((B.S.fe - B.S.fb) / gridDim.x)));
+  bool first = true;
+  while (true) {
+    const uint32_t r = B.S.round;
+    const uint32_t b = B.S.lround & 1u;
+    start_round(D, r);
+    const uint32_t step = first ? gridDim.x * (blockDim.x >> 5) : blockDim.x >> 5;
+    const uint32_t end = first ? B.S.fe - B.S.fb : B.lq_vend[b ^ 1u];
+    const uint32_t from = B.S.fb - B.S.skew;
+    uint32_t k = threadIdx.x >> 5;
+    if (first) k = k * gridDim.x + blockIdx.x;
+    for (; k < end; k += step) {
+      const uint32_t w = first ? ldcg(&D.log[from + k]) : B.lq_ids[b ^ 1u][k];
+      ac6_set(D, B, w, r, K, b, cap);
+    }
+    if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0) {
+      __syncthreads();
+      if (threadIdx.x == 0) D.C->t_work[r & 3] = globaltimer();
+    }
+    if (!local_barrier(D, B, b, r)) break;
+    const uint32_t next = B.lq_next;
+    if (next == LQ_DONE) break;
+    if (next == LQ_GO) {
+      first = false;
+      continue;
+    }
+    const uint32_t ne = B.lq_vend[b];
+    for (uint32_t i0 = (threadIdx.x >> 5) * 32u; i0 < ne; i0 += blockDim.x) {
+      const uint32_t i = i0 + lane;
+      append_dead(D, B, i < ne, i < ne ? B.lq_ids[b][i] : 0u, r, D.live0);
+    }
+    flush_round(D, B, r, D.live0);
+    if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0 && threadIdx.x == 0)
+      D.C->t_flush[r & 3] = globaltimer();
+    if (!grid_barrier(D, B, false)) break;
+    if (threadIdx.x < 32) advance(D, B);
+    __syncthreads();
+    break;
+  }
+  stats_flush(D, B, K);
+  return B.err == 0u;
+}
+#else
 __device__ ROUND_FN bool ac6_round(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
                                    uint32_t nwarps) {
   if (S.prev_variant != TRIM_AC6_SUPPORT) return ac6_entry(D, B, S, gwarp, nwarps);
@@ -2751,6 +3261,7 @@ __device__ ROUND_FN bool ac6_round(const Dev& D, Cta& B, const Sched& S, uint32_
   stats_flush(D, B, K);
   return true;
 }
+#endif
 
 // ------------------------------------------------------------------ init (round 0)
 
