@@ -424,49 +424,54 @@ trim_err_t build_transpose(trim_ctx* c) {
   if (m == 0) {
     CK(cudaMemsetAsync(ioff, 0, ((size_t)n + 1) * 4, c->stream));
   } else if (lg <= 27) {
-    // buckets of 2^shift targets, at most 32,768 each (128 KB of counters in
-    // pass 4): up to 2^26 vertices 2,048 buckets and two CTAs per SM in passes
-    // 1 and 3 (96 KB of shared memory each in pass 3), above that 4,096
-    // buckets and one CTA per SM; either way the open sectors of all (bucket,
-    // CTA) ranges, 32 B each, stay in the L2
-    const bool wide = lg > 26;
-    const uint32_t keep = wide ? 12u : 11u;
-    const uint32_t shift = lg > keep ? lg - keep : 0;
+    // 256 to 4,096 buckets of 2^shift targets (at most 32,768: 128 KB of counters in
+    // pass 4), of 16,384 to 32,768 edges on average in between: every tile of pass 3
+    // and every bucket of pass 4 costs some microseconds whatever its size, and past
+    // 4,096 a tile's runs of pairs per bucket get too short to write. Build in ms with
+    // half / a quarter of the edges per bucket: R-MAT 2^20 (14.5 million edges) 0.300
+    // against 0.321 / 0.364, deep 2^20 (8.4 million) 0.208 against 0.238 / 0.280; with
+    // 32 buckets instead of 256 for 290,000 edges 0.123 against 0.106.
+    uint32_t keep = 8u;
+    while (keep < 12u && (m >> 14) >> keep) ++keep;
+    keep = std::max(keep, lg > 15u ? lg - 15u : 0u);
+    const uint32_t shift = lg > keep ? lg - keep : 0u;
     const uint32_t nb = (uint32_t)(((uint64_t)n + (1u << shift) - 1) >> shift);
-    const uint32_t C = (uint32_t)c->sm_count * (wide ? 1u : 2u);
-    const uint32_t rows = (n + C - 1) / C;
-    // (bucket, CTA) ranges hold whole sectors: up to 3 unused slots each
-    const size_t cap = (size_t)m + 3 * (size_t)nb * C;
-    uint32_t *counts = nullptr, *slots = nullptr, *real = nullptr, *rstart = nullptr;
+    const uint32_t sms = (uint32_t)c->sm_count;
+    const uint32_t piece = (m + sms - 1) / sms;
+    uint32_t *counts = nullptr, *start = nullptr, *cursor = nullptr;
     unsigned long long* pairs = nullptr;
-    TRY(dalloc(c, &counts, (size_t)nb * C));
-    TRY(dalloc(c, &slots, (size_t)nb * C + 1));
-    TRY(dalloc(c, &real, nb));
-    TRY(dalloc(c, &rstart, (size_t)nb + 1));
-    TRY(dalloc(c, &pairs, cap));
-    CK(cudaMemsetAsync(real, 0, (size_t)nb * 4, c->stream));
-    const size_t hist_bytes = (size_t)nb * 4, scatter_bytes = (size_t)nb * 48;
-    const size_t place_bytes = ((size_t)1 << shift) * 4;
+    TRY(dalloc(c, &counts, (size_t)nb + 1));  // and pass 4's ticket
+    TRY(dalloc(c, &start, (size_t)nb + 1));
+    TRY(dalloc(c, &cursor, nb));
+    TRY(dalloc(c, &pairs, (size_t)m));
+    CK(cudaMemsetAsync(counts, 0, ((size_t)nb + 1) * 4, c->stream));
+    const size_t scatter_bytes = (size_t)trimk::kGtTile * 12 + (size_t)nb * 8;
+    // pass 4: two CTAs per SM if buckets a quarter larger than the mean still fit half
+    // its shared memory
+    const size_t place_cnt = ((size_t)1 << shift) * 4, half = 112u << 10, whole = 224u << 10;
+    const bool two = place_cnt + ((size_t)m / nb) * 5 <= half;
+    const size_t place_bytes = two ? half : whole;
+    const uint32_t cap = (uint32_t)((place_bytes - place_cnt) / 4);
     CK(cudaFuncSetAttribute(trim_gt_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)scatter_bytes));
     CK(cudaFuncSetAttribute(trim_gt_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)place_bytes));
-    trim_gt_hist_kernel<<<C, 1024, hist_bytes, c->stream>>>(c->off, c->tgt, n, rows, shift, nb,
-                                                            counts, real);
+    trim_gt_hist_kernel<<<sms * 2, 1024, (size_t)nb * 4, c->stream>>>(c->tgt, n, m, shift, nb,
+                                                                      counts);
     CK(cudaGetLastError());
-    TRY(device_scan(c, counts, nb * C, slots));
-    TRY(device_scan(c, real, nb, rstart));
-    trim_gt_scatter_kernel<<<C, 1024, scatter_bytes, c->stream>>>(c->off, c->tgt, n, rows, shift,
-                                                                  nb, slots, pairs);
+    TRY(device_scan(c, counts, nb, start));
+    CK(cudaMemcpyAsync(cursor, start, (size_t)nb * 4, cudaMemcpyDeviceToDevice, c->stream));
+    trim_gt_scatter_kernel<<<sms, trimk::kGtThreads, scatter_bytes, c->stream>>>(
+        c->off, c->tgt, n, m, piece, shift, nb, cursor, pairs);
     CK(cudaGetLastError());
-    trim_gt_place_kernel<<<std::min<uint32_t>(nb, (uint32_t)c->sm_count * 4), 512, place_bytes,
-                           c->stream>>>(pairs, slots, rstart, C, n, m, shift, nb, ioff, itgt);
+    trim_gt_place_kernel<<<std::min<uint32_t>(nb, two ? sms * 2 : sms), 1024, place_bytes,
+                           c->stream>>>(pairs, start, n, m, shift, nb, cap, counts + nb, ioff,
+                                        itgt);
     CK(cudaGetLastError());
-    dfree(c, pairs, cap);
-    dfree(c, rstart, (size_t)nb + 1);
-    dfree(c, real, nb);
-    dfree(c, slots, (size_t)nb * C + 1);
-    dfree(c, counts, (size_t)nb * C);
+    dfree(c, pairs, (size_t)m);
+    dfree(c, cursor, nb);
+    dfree(c, start, (size_t)nb + 1);
+    dfree(c, counts, (size_t)nb + 1);
   } else {
     uint32_t *fill = nullptr, *bad = nullptr;
     TRY(dalloc(c, &fill, (size_t)n + 1));

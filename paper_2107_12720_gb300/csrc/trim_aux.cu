@@ -129,164 +129,159 @@ __global__ void trim_transpose_fill_kernel(const uint32_t* off, const uint32_t* 
 // Same-address atomics on the in-degree counters of hub targets serialise at
 // the L2, so the global counting sort above is slow on skewed graphs. Here
 // every count and every placement is a shared-memory atomic:
-//   1. each CTA counts, for its rows, the edges per target bucket b = t >> shift
-//      (counts[b * C + c], bucket-major, rounded up to whole 32-byte sectors of
-//      8-byte pairs; the exact totals per bucket go to real[b]);
-//   2. exclusive scans give every (bucket, CTA) its sector-aligned slot range
-//      and every bucket its start in itgt;
-//   3. the same traversal writes each edge's (t, u) into its range: pairs wait
-//      in shared memory in groups of four per bucket and leave as one full
-//      32-byte sector (a partial sector written to DRAM costs a read first);
-//      pairs that find their bucket's group taken go out one by one from the
-//      range's other end; slots left over get the fill value ~0;
+//   1. every CTA counts a part of the edges per target bucket b = t >> shift;
+//   2. an exclusive scan gives the buckets their ranges of pairs;
+//   3. each CTA sorts tiles of its equal piece of the edges by bucket in shared
+//      memory and writes every bucket's run of (t, u) pairs to the bucket's next
+//      free range (one atomic per tile and bucket);
 //   4. one CTA per bucket counts the bucket's targets in shared memory, scans
-//      them into ioff, and places every u at its target's next slot in itgt.
+//      them into ioff, and places every u at its target's next slot in itgt (in
+//      shared memory first, if the bucket fits: writes of single words cost a
+//      sector each at the L2).
 // Targets >= n are skipped (only TRIM_FLAG_VALIDATE reports them).
+//
+// What bounds it: pass 3 the shared-memory pipe (35 wavefronts per 32 edges) and the
+// latencies between its phases, pass 4 the same; DRAM is a fifth busy. R-MAT of 2^22
+// vertices and 58.4 million edges, us per pass: 51, 9, 466 and 346; before, with
+// equal rows per CTA (the fullest had 1.6 times the mean edges), a group of four pairs
+// per bucket guarded by atomics and fences, and itgt written word by word: 172, 16,
+// 622 and 447. Whole builds in ms: R-MAT 2^20 0.411 and 0.300, 2^24 5.48 and 3.41, deep 2^24
+// 3.54 and 2.05. Tried: tiles of 8,192 with two CTAs per SM and 2,048 buckets 450
+// (pass 4 then 301 to 545), of 4,096 with three 838; ranges per (bucket, CTA) instead
+// of one cursor per bucket 571; two passes of 64 buckets each 346 + 277.
 
-// Rows with more out-edges than kHeavyRow are walked by the whole CTA (one
-// warp would take a skewed graph's longest rows alone, one dependent load per
-// 32 edges); up to kHeavyCap of them per CTA, any further ones by their warp.
-constexpr uint32_t kHeavyRow = 256;
-constexpr uint32_t kHeavyCap = 1024;
-
-// All threads of the CTA: f(u, t) for every out-edge of rows [r0, r1).
-// Light rows: each warp takes 32 rows at a time and walks their edges laid end
-// to end, 32 per step, four steps' loads in flight. Heavy rows: afterwards,
-// one at a time, the whole CTA strides over the row. `heavy` and `nheavy` are
-// shared scratch (*nheavy = 0 on entry).
-template <class F>
-__device__ __forceinline__ void cta_row_edges(const uint32_t* off, const uint32_t* tgt,
-                                              uint32_t r0, uint32_t r1, uint32_t* heavy,
-                                              uint32_t* nheavy, F f) {
-  const unsigned lane = lane_id();
-  const uint32_t nw = blockDim.x >> 5;
-  for (uint32_t r = r0 + (threadIdx.x >> 5) * 32u; r < r1; r += nw * 32u) {  // warp-uniform
-    const uint32_t v = r + lane;
-    const bool has = v < r1;
-    const uint32_t s = has ? off[v] : 0u;
-    uint32_t d = has ? off[v + 1] - s : 0u;
-    if (d > kHeavyRow) {
-      const uint32_t at = atomicAdd(nheavy, 1u);
-      if (at < kHeavyCap) {
-        heavy[at] = v;
-        d = 0u;
-      }
-    }
-    const uint32_t incl = warp_incl_scan(d);
-    const uint32_t excl = incl - d;
-    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    for (uint32_t k0 = 0; k0 < total; k0 += 128u) {  // warp-uniform
-      uint32_t u[4], t[4];
-      bool ok[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t k = k0 + (uint32_t)q * 32u + lane;
-        const unsigned o = owner_of(excl, k);
-        const uint32_t so = __shfl_sync(0xFFFFFFFFu, s, o);
-        const uint32_t xo = __shfl_sync(0xFFFFFFFFu, excl, o);
-        ok[q] = k < total;
-        u[q] = r + o;
-        t[q] = ok[q] ? __ldg(&tgt[so + (k - xo)]) : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (ok[q]) f(u[q], t[q]);
-    }
-  }
-  __syncthreads();
-  const uint32_t nh = min(*nheavy, kHeavyCap);
-  for (uint32_t h = 0; h < nh; ++h) {  // block-uniform
-    const uint32_t v = heavy[h];
-    const uint32_t s = off[v], e = off[v + 1];
-    for (uint32_t k0 = s; k0 < e; k0 += 4u * blockDim.x) {
-      uint32_t t[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t k = k0 + (uint32_t)q * blockDim.x + threadIdx.x;
-        t[q] = k < e ? __ldg(&tgt[k]) : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (k0 + (uint32_t)q * blockDim.x + threadIdx.x < e) f(v, t[q]);
-    }
-  }
+__device__ __forceinline__ uint32_t gt_piece(uint64_t c, uint32_t piece, uint32_t m) {
+  const uint64_t e = c * piece;
+  return e < m ? (uint32_t)e : m;
 }
 
-// Pass 1: per-CTA histogram of target buckets over rows [c * rows, (c+1) * rows).
-__global__ void trim_gt_hist_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n,
-                                    uint32_t rows, uint32_t shift, uint32_t nb,
-                                    uint32_t* counts, uint32_t* real) {
+// Pass 1: histogram of the target buckets.
+__global__ void __launch_bounds__(1024)
+trim_gt_hist_kernel(const uint32_t* tgt, uint32_t n, uint32_t m, uint32_t shift, uint32_t nb,
+                    uint32_t* counts) {
   extern __shared__ uint32_t hist[];
-  __shared__ uint32_t heavy[kHeavyCap];
-  __shared__ uint32_t nheavy;
   for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) hist[i] = 0u;
-  if (threadIdx.x == 0) nheavy = 0u;
   __syncthreads();
-  const uint32_t r0 = min(n, blockIdx.x * rows), r1 = min(n, r0 + rows);
-  cta_row_edges(off, tgt, r0, r1, heavy, &nheavy, [&](uint32_t, uint32_t t) {
-    if (t < n) atomicAdd(&hist[t >> shift], 1u);
-  });
-  __syncthreads();
-  for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) {
-    counts[(size_t)i * gridDim.x + blockIdx.x] = (hist[i] + 3u) & ~3u;
-    if (hist[i]) atomicAdd(&real[i], hist[i]);
+  constexpr int U = 8;
+  const uint64_t step = (uint64_t)U * blockDim.x;
+  for (uint64_t k0 = blockIdx.x * step; k0 < m; k0 += gridDim.x * step) {
+    uint32_t t[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const uint64_t k = k0 + (uint64_t)q * blockDim.x + threadIdx.x;
+      t[q] = k < m ? __ldg(&tgt[k]) : 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (t[q] < n) atomicAdd(&hist[t[q] >> shift], 1u);
   }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x)
+    if (hist[i]) atomicAdd(&counts[i], hist[i]);
 }
 
-// Pass 3: the edges of the same rows go to their (bucket, CTA) slot ranges.
-// Shared memory per bucket: a group of four pairs, its slot requests and
-// completed writes, and the range's two cursors (groups from the start,
-// single pairs from the end).
-__global__ void trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n,
-                                       uint32_t rows, uint32_t shift, uint32_t nb,
-                                       const uint32_t* slots, unsigned long long* pairs) {
-  extern __shared__ unsigned long long gbuf[];  // nb x 4 pairs, then the counters
-  uint32_t* req = reinterpret_cast<uint32_t*>(gbuf + (size_t)nb * 4u);
-  uint32_t* done = req + nb;
-  uint32_t* lo = done + nb;
-  uint32_t* hi = lo + nb;
-  __shared__ uint32_t heavy[kHeavyCap];
-  __shared__ uint32_t nheavy;
-  for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) {
-    const size_t at = (size_t)i * gridDim.x + blockIdx.x;
-    req[i] = 0u;
-    done[i] = 0u;
-    lo[i] = slots[at];
-    hi[i] = slots[at + 1];
+// Pass 3. A tile's edges get their rows from marks at the rows' first edges and a
+// running maximum; an atomic on the bucket's counter ranks an edge in its bucket,
+// a scan of the counters places the buckets, and the sorted pairs leave in order,
+// each bucket's run contiguous. Shared memory: the tile's pairs and marks, and per
+// bucket its counter (then first position in the tile) and the distance of its
+// range in `pairs` from that position. Each warp has a contiguous part of the tile.
+__global__ void __launch_bounds__(kGtThreads)
+trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n, uint32_t m,
+                       uint32_t piece, uint32_t shift, uint32_t nb, uint32_t* cursor,
+                       unsigned long long* pairs) {
+  constexpr int U = kGtTile / kGtThreads;
+  extern __shared__ unsigned long long sorted[];
+  uint32_t* mark = reinterpret_cast<uint32_t*>(sorted + kGtTile);
+  uint32_t* first = mark + kGtTile;
+  uint32_t* dist = first + nb;
+  __shared__ uint32_t wmax[kGtThreads / 32];
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint32_t e0 = gt_piece(blockIdx.x, piece, m), e1 = gt_piece(blockIdx.x + 1ull, piece, m);
+  // a row that starts at or before the piece: the last of those tried, narrowed down
+  uint32_t ra = 0;
+  for (uint32_t len = n; len > 1u;) {  // block-uniform
+    const uint32_t step = (len + kGtThreads - 1u) / kGtThreads;
+    const uint64_t r = (uint64_t)threadIdx.x * step;
+    const int k = __syncthreads_count(r < len && __ldg(&off[ra + r]) <= e0);
+    const uint32_t skip = (uint32_t)max(k - 1, 0) * step;
+    ra += skip;
+    len = min(step, len - skip);
   }
-  if (threadIdx.x == 0) nheavy = 0u;
-  __syncthreads();
-  volatile unsigned long long* vbuf = gbuf;
-  const uint32_t r0 = min(n, blockIdx.x * rows), r1 = min(n, r0 + rows);
-  cta_row_edges(off, tgt, r0, r1, heavy, &nheavy, [&](uint32_t u, uint32_t t) {
-    if (t >= n) return;
-    const uint32_t b = t >> shift;
-    const unsigned long long pr = ((unsigned long long)t << 32) | u;
-    const uint32_t slot = atomicAdd(&req[b], 1u);
-    if (slot >= 4u) {  // the group is taken: this pair goes out alone
-      pairs[atomicSub(&hi[b], 1u) - 1u] = pr;
-      return;
+  const uint32_t part = warp * (U * 32) + lane;
+  for (uint64_t t0 = e0; t0 < e1; t0 += kGtTile) {  // block-uniform
+    const uint32_t tile = (uint32_t)t0, size = min((uint32_t)kGtTile, e1 - tile);
+    for (uint32_t i = threadIdx.x; i < kGtTile; i += kGtThreads) mark[i] = i ? 0u : ra;
+    for (uint32_t b = threadIdx.x; b < nb; b += kGtThreads) first[b] = 0u;
+    uint32_t t[U], rank[U], row[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      t[q] = part + q * 32u < size ? __ldg(&tgt[tile + part + q * 32u]) : 0xFFFFFFFFu;
+    __syncthreads();
+    // (of rows with the same first edge only the last has edges)
+    for (uint64_t r = (uint64_t)ra + 1u + threadIdx.x; r < n; r += kGtThreads) {
+      const uint32_t o = __ldg(&off[r]);
+      if (o >= tile + size) break;
+      atomicMax(&mark[o > tile ? o - tile : 0u], (uint32_t)r);
     }
-    vbuf[b * 4u + slot] = pr;
-    __threadfence_block();
-    if (atomicAdd(&done[b], 1u) != 3u) return;
-    // the fourth write of the group: send it as one sector and open the next
-    __threadfence_block();
-    const uint32_t at = atomicAdd(&lo[b], 4u);
-    ulonglong2* dst = reinterpret_cast<ulonglong2*>(pairs + at);
-    dst[0] = make_ulonglong2(vbuf[b * 4u], vbuf[b * 4u + 1u]);
-    dst[1] = make_ulonglong2(vbuf[b * 4u + 2u], vbuf[b * 4u + 3u]);
-    __threadfence_block();
-    atomicExch(&done[b], 0u);
-    __threadfence_block();
-    atomicExch(&req[b], 0u);
-  });
-  __syncthreads();
-  // groups that never filled: their pairs go out one by one; the range's
-  // unused slots (at most 3) get the fill value
-  for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) {
-    for (uint32_t k = 0; k < done[i]; ++k) pairs[--hi[i]] = vbuf[i * 4u + k];
-    for (uint32_t k = lo[i]; k < hi[i]; ++k) pairs[k] = ~0ull;
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      rank[q] = t[q] < n ? atomicAdd(&first[t[q] >> shift], 1u) : 0u;
+    __syncthreads();
+    // running maximum of the marks
+    uint32_t carry = 0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      uint32_t x = mark[part + q * 32u];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (unsigned)o) x = max(x, y);
+      }
+      row[q] = max(x, carry);
+      carry = __shfl_sync(0xFFFFFFFFu, row[q], 31);
+    }
+    if (lane == 0) wmax[warp] = carry;
+    // exclusive scan of the bucket counts, and the buckets' next free ranges
+    uint32_t pre = 0;
+    for (uint32_t b0 = 0; b0 < nb; b0 += 4u * kGtThreads) {  // block-uniform
+      uint32_t c[4], sum = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t b = b0 + 4u * threadIdx.x + q;
+        c[q] = b < nb ? first[b] : 0u;
+        sum += c[q];
+      }
+      unsigned all;
+      uint32_t at = pre + block_excl_scan(sum, &all);  // (syncs: wmax is complete)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t b = b0 + 4u * threadIdx.x + q;
+        if (b < nb) {
+          first[b] = at;
+          if (c[q]) dist[b] = atomicAdd(&cursor[b], c[q]) - at;
+        }
+        at += c[q];
+      }
+      pre += all;
+    }
+    uint32_t before = 0;  // rows that began in an earlier warp's part
+    for (unsigned w = 0; w < kGtThreads / 32; ++w) {
+      if (w < warp) before = max(before, wmax[w]);
+      ra = max(ra, wmax[w]);  // the tile's last row
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (t[q] < n)
+        sorted[first[t[q] >> shift] + rank[q]] =
+            ((unsigned long long)t[q] << 32) | max(row[q], before);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < pre; i += kGtThreads) {
+      const unsigned long long pr = sorted[i];
+      pairs[dist[(uint32_t)(pr >> 32) >> shift] + i] = pr;
+    }
+    __syncthreads();
   }
 }
 
@@ -299,29 +294,35 @@ __device__ __forceinline__ unsigned hub_lanes(uint32_t t) {
   return __popc(same) >= 8 ? same : 0u;
 }
 
-// Pass 4: CTA per bucket (grid-stride).
-__global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint32_t* slots,
-                                     const uint32_t* rstart, uint32_t C, uint32_t n, uint32_t m,
-                                     uint32_t shift, uint32_t nb, uint32_t* ioff,
-                                     uint32_t* itgt) {
+// Pass 4: a CTA takes the next bucket until there is none (skewed graphs have
+// buckets of very different sizes). A bucket's pairs and its part of itgt are the
+// same range; a bucket of at most `cap` pairs is put together in shared memory.
+__global__ void __launch_bounds__(1024)
+trim_gt_place_kernel(const unsigned long long* pairs, const uint32_t* start, uint32_t n,
+                     uint32_t m, uint32_t shift, uint32_t nb, uint32_t cap, uint32_t* ticket,
+                     uint32_t* ioff, uint32_t* itgt) {
   extern __shared__ uint32_t cnt[];
+  uint32_t* stage = cnt + (1u << shift);
+  __shared__ uint32_t next;
   const unsigned lane = lane_id();
-  const uint32_t nw = blockDim.x >> 5;
-  for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
+  while (true) {
+    if (threadIdx.x == 0) next = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t b = next;
+    if (b >= nb) break;
     const uint32_t base = b << shift;
     const uint32_t nt = min(1u << shift, n - base);
-    const uint32_t p0 = slots[(size_t)b * C];
-    const uint32_t p1 = slots[(size_t)(b + 1u) * C];  // slots[nb * C] = all slots
+    const uint32_t p0 = start[b], np = start[b + 1u] - p0;
+    const unsigned long long* in = pairs + p0;
     for (uint32_t i = threadIdx.x; i < nt; i += blockDim.x) cnt[i] = 0u;
     __syncthreads();
     // four loads in flight per lane, then the combined atomics
-    for (uint32_t q = p0 + (threadIdx.x >> 5) * 32u; q < p1; q += 4u * nw * 32u) {  // warp-uniform
+    for (uint64_t q = threadIdx.x - lane; q < np; q += 4u * blockDim.x) {  // warp-uniform
       uint32_t t[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const uint32_t p = q + (uint32_t)k * nw * 32u + lane;
-        const unsigned long long pr = p < p1 ? pairs[p] : ~0ull;  // ~0: an unused slot
-        t[k] = pr != ~0ull ? (uint32_t)(pr >> 32) - base : 0xFFFFFFFFu;
+        const uint64_t p = q + (uint64_t)k * blockDim.x + lane;
+        t[k] = p < np ? (uint32_t)(in[p] >> 32) - base : 0xFFFFFFFFu;
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -334,7 +335,7 @@ __global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint
       }
     }
     __syncthreads();
-    uint32_t carry = rstart[b];  // edges of the buckets before b
+    uint32_t carry = 0;
     for (uint32_t j0 = 0; j0 < nt; j0 += blockDim.x) {  // block-uniform
       const uint32_t j = j0 + threadIdx.x;
       const uint32_t x = j < nt ? cnt[j] : 0u;
@@ -342,17 +343,19 @@ __global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint
       const uint32_t ex = block_excl_scan(x, &tot);
       if (j < nt) {
         cnt[j] = carry + ex;
-        ioff[base + j] = carry + ex;
+        ioff[base + j] = p0 + carry + ex;
       }
       carry += tot;
     }
     __syncthreads();
-    for (uint32_t q = p0 + (threadIdx.x >> 5) * 32u; q < p1; q += 4u * nw * 32u) {
+    const bool staged = np <= cap;
+    uint32_t* out = staged ? stage : itgt + p0;
+    for (uint64_t q = threadIdx.x - lane; q < np; q += 4u * blockDim.x) {
       unsigned long long pr[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const uint32_t p = q + (uint32_t)k * nw * 32u + lane;
-        pr[k] = p < p1 ? pairs[p] : ~0ull;
+        const uint64_t p = q + (uint64_t)k * blockDim.x + lane;
+        pr[k] = p < np ? in[p] : ~0ull;
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -363,9 +366,12 @@ __global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint
         if (lane == 0 && same) at = atomicAdd(&cnt[t], (uint32_t)__popc(same));
         at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(same & ((1u << lane) - 1u));
         if (valid && !(same >> lane & 1u)) at = atomicAdd(&cnt[t], 1u);
-        if (valid) itgt[at] = (uint32_t)pr[k];
+        if (valid) out[at] = (uint32_t)pr[k];
       }
     }
+    __syncthreads();
+    if (staged)
+      for (uint32_t i = threadIdx.x; i < np; i += blockDim.x) itgt[p0 + i] = stage[i];
     __syncthreads();
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) ioff[n] = m;

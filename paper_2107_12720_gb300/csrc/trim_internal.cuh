@@ -15,6 +15,10 @@
 
 namespace trimk {
 
+// edges a CTA sorts at a time when G^T is built, and its threads
+constexpr uint32_t kGtTile = 16384;
+constexpr uint32_t kGtThreads = 1024;
+
 constexpr uint32_t LIVE = 0xFFFFFFFFu;
 constexpr uint32_t NIL = 0xFFFFFFFFu;
 constexpr int NFEAT = 12;
@@ -357,15 +361,14 @@ __global__ void trim_scan_blocks_kernel(const uint32_t* in, uint32_t n, uint32_t
                                         uint32_t* block_sums, uint32_t chunk);
 __global__ void trim_scan_apply_kernel(uint32_t* out, uint32_t n, const uint32_t* block_sums,
                                        uint32_t nblocks, uint32_t chunk);
-__global__ void trim_gt_hist_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n,
-                                    uint32_t rows, uint32_t shift, uint32_t nb, uint32_t* counts,
-                                    uint32_t* real);
+__global__ void trim_gt_hist_kernel(const uint32_t* tgt, uint32_t n, uint32_t m, uint32_t shift,
+                                    uint32_t nb, uint32_t* counts);
 __global__ void trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n,
-                                       uint32_t rows, uint32_t shift, uint32_t nb,
-                                       const uint32_t* slots, unsigned long long* pairs);
-__global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint32_t* slots,
-                                     const uint32_t* rstart, uint32_t C, uint32_t n, uint32_t m,
-                                     uint32_t shift, uint32_t nb, uint32_t* ioff,
+                                       uint32_t m, uint32_t piece, uint32_t shift, uint32_t nb,
+                                       uint32_t* cursor, unsigned long long* pairs);
+__global__ void trim_gt_place_kernel(const unsigned long long* pairs, const uint32_t* start,
+                                     uint32_t n, uint32_t m, uint32_t shift, uint32_t nb,
+                                     uint32_t cap, uint32_t* ticket, uint32_t* ioff,
                                      uint32_t* itgt);
 __global__ void trim_transpose_fill_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n,
                                            const uint32_t* ioff, uint32_t* fill, uint32_t* itgt);
