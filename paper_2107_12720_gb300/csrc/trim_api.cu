@@ -58,7 +58,8 @@ struct trim_ctx {
   // the chunk-owner index of its edge space (both rows: up to 2m edges)
   unsigned long long* cnt_io = nullptr;
   uint32_t *w4_dir = nullptr, *chunk_io = nullptr;
-  uint8_t* mask = nullptr;  // trim_set_dead_mask: device copy of the dead mask
+  uint8_t* mask = nullptr;  // trim_set_dead_mask: device copy of the dead mask ...
+  uint32_t* mask_bits = nullptr;  // ... and the same as one bit per vertex
   bool has_mask = false;
   bool implicit = false;      // trim_create_implicit: successors computed, no CSR
   trim_implicit_graph_t ig{};
@@ -849,7 +850,7 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   D.live1 = c->live1; D.w4_row = c->w4_row; D.w4_eoff = c->w4_eoff;
   D.chunk_first = c->chunk_first; D.bsum = c->bsum; D.C = c->ctrl;
   D.cnt_io = c->cnt_io; D.w4_dir = c->w4_dir;
-  D.mask = c->has_mask ? c->mask : nullptr;
+  D.mask = c->has_mask ? c->mask_bits : nullptr;
   D.ig = c->ig;
   if (inout) D.chunk_first = c->chunk_io;
   D.rlog = c->rlog; D.rlog_cap = c->rlog_cap;
@@ -1455,9 +1456,13 @@ trim_err_t trim_set_dead_mask(trim_ctx* c, const uint8_t* mask, int on_device) {
     return TRIM_OK;
   }
   if (c->n && !c->mask) TRY(dalloc(c, &c->mask, c->n));
-  if (c->n)
+  if (c->n && !c->mask_bits) TRY(dalloc(c, &c->mask_bits, ((size_t)c->n + 31) / 32));
+  if (c->n) {
     CK(cudaMemcpyAsync(c->mask, mask, c->n,
                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    trim_mask_bits_kernel<<<c->sm_count * 4, 512, 0, c->stream>>>(c->mask, c->n, c->mask_bits);
+    CK(cudaGetLastError());
+  }
   TRY(sync_check(c));
   c->has_mask = true;
   return TRIM_OK;

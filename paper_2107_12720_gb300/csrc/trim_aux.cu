@@ -60,6 +60,16 @@ __global__ void trim_status_kernel(const uint32_t* level, uint32_t n, uint8_t* s
     status[v] = level[v] == LIVE ? 1 : 0;
 }
 
+// A dead mask as one bit per vertex, for the runs' initial pass (a warp per word).
+__global__ void trim_mask_bits_kernel(const uint8_t* mask, uint32_t n, uint32_t* bits) {
+  const uint32_t words = (n + 31u) / 32u, nw = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < words; w += nw) {
+    const uint32_t v = w * 32u + lane_id();
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, v < n && mask[v] != 0);
+    if (lane_id() == 0) bits[w] = b;
+  }
+}
+
 // After a run with a dead mask: masked vertices carry level 0 inside the run
 // (removed before round 1, so every variant's "level[u] < r" test skips them);
 // their reported level is TRIM_MASKED.

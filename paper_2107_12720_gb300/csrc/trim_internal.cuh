@@ -180,9 +180,9 @@ struct Dev {
   // G^T row (0) or G row (1)
   unsigned long long* cnt_io;
   uint32_t* w4_dir;
-  // vertex sampling (trim_set_dead_mask): mask[v] != 0 marks a vertex that is
-  // DEAD from the start; nullable
-  const uint8_t* __restrict__ mask;
+  // vertex sampling (trim_set_dead_mask): bit v & 31 of mask[v >> 5] marks a vertex
+  // that is DEAD from the start; nullable
+  const uint32_t* __restrict__ mask;
   // implicit graph (trim_create_implicit): successors computed on the fly by
   // the implicit flavours; off/tgt are null then
   trim_implicit_graph_t ig;
@@ -354,6 +354,7 @@ __global__ void trim_implicit_degree_sum_kernel(trimk::Dev D, unsigned long long
 __global__ void trim_reset_ctrl_kernel(trimk::Ctrl* C);
 __global__ void trim_status_kernel(const uint32_t* level, uint32_t n, uint8_t* status);
 __global__ void trim_scc_kernel(trimk::SccArgs A);  // SCC decomposition (trim_scc.cu)
+__global__ void trim_mask_bits_kernel(const uint8_t* mask, uint32_t n, uint32_t* bits);
 __global__ void trim_mask_levels_kernel(uint32_t* level, const uint8_t* mask, uint32_t n);
 __global__ void trim_indeg_kernel(const uint32_t* tgt, uint64_t m, uint32_t n, uint32_t* cnt,
                                   uint32_t* bad);

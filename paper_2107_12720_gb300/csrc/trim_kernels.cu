@@ -3357,8 +3357,8 @@ __device__ ROUND_FN void init_round(const Dev& D, Cta& B, uint32_t gwarp, uint32
 // vertices and walks their edges laid end to end, 32 per step with four
 // steps' loads in flight; a vertex's count in a step is the popcount of the
 // step's unmasked-target ballot over the lanes that hold its edges. Rows with
-// more than kMaskHeavy edges are left to the whole CTA afterwards (one warp
-// would walk a skewed graph's longest row alone). A run
+// more than kMaskHeavy edges wait until the end, when a warp takes each of them
+// or, with more than kMaskGiant, the whole CTA. A run
 // without AC-4 needs only whether one unmasked successor exists, so each lane
 // scans its own row and stops at the first one (rows longer than 32: the
 // whole warp).
@@ -3368,8 +3368,26 @@ __device__ __forceinline__ uint32_t lane_range(uint32_t a, uint32_t b) {  // bit
   return hi & ~lo;
 }
 
-constexpr uint32_t kMaskHeavy = 1024;
+constexpr uint32_t kMaskHeavy = 512;
+constexpr uint32_t kMaskGiant = 4096;
 constexpr uint32_t kMaskHeavyCap = LW - MAX_WARPS;  // list + per-warp sums in one slice
+
+// The mask comes as one bit per vertex: the pass is bound by the look-ups of the
+// targets' marks (random accesses), and the bits of the targets that skewed graphs
+// keep asking for stay in the L1, which the streamed targets pass by. R-MAT of
+// 3,000,017 vertices, half of them masked, 21 million look-ups, initial pass in us: 213
+// with a byte per vertex, one 32-vertex block after the other and heavy rows (over
+// 1,024) by the CTA; 191 with bits, 178 with heavy rows by warps, 159 with the next block's loads
+// (and its G^T rows) ahead. Bounds of 128 / 256 / 512 for the heavy rows: 217, 207, 178;
+// of 2,048 / 4,096 / 8,192 / 16,384 for the giant ones (at 256): 201, 207, 205, 242.
+__device__ __forceinline__ bool is_masked(const Dev& D, uint32_t v) {
+  return __ldg(&D.mask[v >> 5]) >> (v & 31u) & 1u;
+}
+__device__ __forceinline__ uint32_t ld_once(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
 
 __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
                                            uint32_t nwarps) {
@@ -3383,12 +3401,24 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
   uint32_t* wsum = heavy + kMaskHeavyCap;
   if (threadIdx.x == 0) B.lq_scratch = 0u;
   __syncthreads();
+  // the next 32 vertices' mark, row and G^T row are loaded while the last are counted
+  uint32_t next[5];
+  auto load = [&](uint32_t v) {
+    const bool in = v < n;
+    next[0] = in && is_masked(D, v) ? 1u : 0u;
+    next[1] = in ? __ldg(&D.off[v]) : 0u;
+    next[2] = in ? __ldg(&D.off[v + 1]) : 0u;
+    next[3] = in && w4 ? __ldg(&D.ioff[v]) : 0u;
+    next[4] = in && w4 ? __ldg(&D.ioff[v + 1]) : 0u;
+  };
+  load(gwarp * 32u + lane);
   for (uint32_t base = gwarp * 32u; base < n; base += nwarps * 32u) {
     const uint32_t v = base + lane;
     const bool has = v < n;
-    const bool masked = has && D.mask[v] != 0;
-    const uint32_t s = has ? __ldg(&D.off[v]) : 0u;
-    const uint32_t d = has ? __ldg(&D.off[v + 1]) - s : 0u;
+    const bool masked = next[0] != 0u;
+    const uint32_t s = next[1], d = next[2] - next[1];
+    const uint32_t irow = next[3], din = next[4] - next[3];
+    load(min(base + nwarps * 32u, n) + lane);
     uint32_t c = 0;
     bool deferred = false;
     if (w4 && !masked && d > kMaskHeavy) {
@@ -3409,12 +3439,12 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
           const uint32_t k = k0 + (uint32_t)q * 32u + lane;
           const unsigned o = owner_of(excl, k);
           const uint32_t so = __shfl_sync(FULL, s, o), xo = __shfl_sync(FULL, excl, o);
-          t[q] = k < total ? __ldg(&D.tgt[so + (k - xo)]) : 0u;
+          t[q] = k < total ? ld_once(&D.tgt[so + (k - xo)]) : 0u;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t cs = k0 + (uint32_t)q * 32u;  // flattened index of lane 0
-          const bool live = cs + lane < total && D.mask[t[q]] == 0;
+          const bool live = cs + lane < total && !is_masked(D, t[q]);
           const uint32_t bal = __ballot_sync(FULL, live);
           const uint32_t a = excl <= cs ? 0u : min(excl - cs, 32u);
           const uint32_t e = excl + dd;
@@ -3429,7 +3459,7 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
 #pragma unroll
         for (int q = 0; q < 4; ++q) tq[q] = (k0 + q < d) ? __ldg(&D.tgt[s + k0 + q]) : 0u;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) c += (k0 + q < d && D.mask[tq[q]] == 0) ? 1u : 0u;
+        for (int q = 0; q < 4; ++q) c += (k0 + q < d && !is_masked(D, tq[q])) ? 1u : 0u;
       }
       unsigned big = __ballot_sync(FULL, has && !masked && d > 32u);
       while (big) {
@@ -3447,7 +3477,7 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const uint32_t k = k0 + (uint32_t)q * 32u + lane;
-            part += (k < dj && D.mask[tq[q]] == 0) ? 1u : 0u;
+            part += (k < dj && !is_masked(D, tq[q])) ? 1u : 0u;
           }
           if (__any_sync(FULL, part != 0u)) break;
         }
@@ -3461,14 +3491,37 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
       D.level[v] = (masked || c == 0u) ? 0u : LIVE;
       if (w4) D.cnt[v] = masked ? 0u : c;
     }
-    append_dead(D, B, has && !masked && !deferred && c == 0u, v, 0u, D.live0, true);
+    append_dead(D, B, has && !masked && !deferred && c == 0u, v, 0u, D.live0, true, w4, irow, din);
   }
   __syncthreads();
   const uint32_t nh = min(B.lq_scratch, kMaskHeavyCap);
   const unsigned warp = threadIdx.x >> 5;
+  for (uint32_t h = warp; h < nh; h += blockDim.x >> 5) {  // a warp to a row
+    const uint32_t v = heavy[h];
+    const uint32_t s = __ldg(&D.off[v]), e = __ldg(&D.off[v + 1]);
+    if (e - s > kMaskGiant) continue;
+    uint32_t part = 0;
+    const uint32_t d = e - s;
+    for (uint32_t k0 = lane; k0 < d; k0 += 256u) {
+      uint32_t tq[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        tq[q] = k0 + q * 32u < d ? ld_once(&D.tgt[s + k0 + q * 32u]) : 0u;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        part += (k0 + q * 32u < d && !is_masked(D, tq[q])) ? 1u : 0u;
+    }
+    part = __reduce_add_sync(FULL, part);
+    if (lane == 0) {
+      D.level[v] = part ? LIVE : 0u;
+      D.cnt[v] = part;
+    }
+    append_dead(D, B, lane == 0 && part == 0u, v, 0u, D.live0, true);
+  }
   for (uint32_t h = 0; h < nh; ++h) {  // block-uniform
     const uint32_t v = heavy[h];
     const uint32_t s = __ldg(&D.off[v]), e = __ldg(&D.off[v + 1]);
+    if (e - s <= kMaskGiant) continue;
     uint32_t part = 0;
     for (uint32_t k0 = s; k0 < e; k0 += 4u * blockDim.x) {
       uint32_t tq[4];
@@ -3480,7 +3533,7 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const uint32_t k = k0 + (uint32_t)q * blockDim.x + threadIdx.x;
-        part += (k < e && D.mask[tq[q]] == 0) ? 1u : 0u;
+        part += (k < e && !is_masked(D, tq[q])) ? 1u : 0u;
       }
     }
     part = __reduce_add_sync(FULL, part);
