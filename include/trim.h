@@ -123,8 +123,9 @@ typedef struct {
                                  warp), rounds run CTA-locally: each CTA queues the vertices
                                  it removes in shared memory and pushes them itself in the
                                  next round (AC-6: re-scans their sets; at most one to a warp
-                                 to start with), and a round ends at one barrier that carries
-                                 its totals; a round whose removals overflow the queues
+                                 to start with; AC-3 alone: every round, each CTA on a live
+                                 list of its own vertices), and a round ends at one
+                                 barrier that carries its totals; a round whose removals overflow the queues
                                  returns to ordinary rounds (0 = never local)            */
   float sched_commit_confidence; /* LEARNED: a choice whose softmax probability (among the
                                  variants the run can use) is at least this commits the

@@ -717,7 +717,7 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_slist = A.add<uint32_t>(n), a_log = A.add<uint32_t>(n);
   const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
-  const size_t a_heads = A.add<uint4>(n);
+  const size_t a_heads = A.add<uint4>(n + 32);
   const size_t a_ctrl = A.add<Ctrl>(1), a_m = A.add<unsigned long long>(1);
   const size_t a_rlog = c->rlog_cap ? A.add<trim_round_rec_t>(c->rlog_cap) : 0;
   char* base = nullptr;
@@ -727,7 +727,7 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   c->s_rec = reinterpret_cast<uint4*>(c->supp);
   c->s_cnt = at(a_scnt);
   c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->roff = at(a_roff);
-  c->live0 = at(a_heads); c->live1 = c->live0 + n; c->bsum = at(a_bsum);
+  c->live0 = at(a_heads); c->live1 = c->live0 + ((n + 63) & ~(size_t)63); c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
   if (c->rlog_cap) c->rlog = reinterpret_cast<trim_round_rec_t*>(base + a_rlog);
   CK(cudaMemsetAsync(c->s_cnt, 0, n * 4, c->stream));

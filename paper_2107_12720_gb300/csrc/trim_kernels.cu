@@ -113,11 +113,11 @@ struct WarpSlice {
 // queued neighbour which of its two counters the push decrements.
 // So does AC-6 (flavours 2 and 34, the ones that run nothing else): its queue
 // holds the removed vertices, whose supporting sets the CTA re-scans in the next
-// round.
+// round. And so does AC-3 (flavours 4 and 36), with a live list per CTA.
 #if TRIM_MODES == 1 || TRIM_MODES == 9
 #define TRIM_LOCAL 1
 #define TRIM_ASYNC 1
-#elif TRIM_MODES == 17 || TRIM_MODES == 2 || TRIM_MODES == 34
+#elif TRIM_MODES == 17 || TRIM_MODES == 2 || TRIM_MODES == 34 || TRIM_MODES == 4 || TRIM_MODES == 36
 #define TRIM_LOCAL 1
 #define TRIM_ASYNC 0
 #else
@@ -125,6 +125,7 @@ struct WarpSlice {
 #define TRIM_ASYNC 0
 #endif
 #define TRIM_AC6_ONLY (TRIM_MODES == 2 || TRIM_MODES == 34)
+#define TRIM_AC3_ONLY (TRIM_MODES == 4 || TRIM_MODES == 36)
 #if TRIM_LOCAL
 constexpr uint32_t LQ_EDGES = 1024;   // predecessors queued per CTA per round
 constexpr uint32_t LQ_ENTRIES = 256;  // removed vertices queued per CTA per round
@@ -156,7 +157,9 @@ struct Cta {
   unsigned long long kstat[4];  // TRIM_FLAG_STATS totals of this CTA (see stats_flush)
   uint32_t wbuf[MAX_WARPS][WBUF];
 #if TRIM_LOCAL
-#if TRIM_AC6_ONLY
+#if TRIM_AC3_ONLY
+  uint32_t live_n[2];  // local AC-3 rounds: the CTA's live list, by local-round parity
+#elif TRIM_AC6_ONLY
   // local AC-6 rounds: the vertices this CTA removed, by local-round parity
   uint32_t lq_ids[2][LQ_ENTRIES];
 #else
@@ -536,7 +539,7 @@ __device__ __forceinline__ void append_live(const Dev& D, Cta& B, bool pred, uin
   __syncwarp();
 }
 
-#if TRIM_LOCAL && !TRIM_AC6_ONLY
+#if TRIM_LOCAL && !TRIM_AC6_ONLY && !TRIM_AC3_ONLY
 // Warp-collective: lanes with pred add a work-list entry (row start, length; in+out
 // trimming: and direction) of a vertex that is already removed and counted.
 __device__ __forceinline__ void append_w4(const Dev& D, Cta& B, bool pred, uint32_t row,
@@ -1230,7 +1233,7 @@ __device__ ROUND_FN void ac4_round(const Dev& D, Cta& B, const Sched& S, uint32_
 #if TRIM_LOCAL
 // ------------------------------------------------------------------ local AC-4 rounds
 
-#if !TRIM_AC6_ONLY
+#if !TRIM_AC6_ONLY && !TRIM_AC3_ONLY
 // End of a local stretch that returns to ordinary rounds (all threads): the
 // queued vertices of round r (buffer b) become work-list entries, and the round
 // ends like an ordinary one (flush, grid barrier, advance). A rare path, out of
@@ -1265,7 +1268,9 @@ void local_leave(uint32_t b, uint32_t r) {
 // entries (the stretch's first round gives each warp whole entries) must have
 // at most local_edges_max in-edges in all, none more than 256.
 __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
-#if TRIM_AC6_ONLY
+#if TRIM_AC3_ONLY
+  return D.local_edges_max != 0u;  // from the first round to the last
+#elif TRIM_AC6_ONLY
   // AC-6: the sets were built, and the last round's removals are at most one to a warp
   return S.prev_variant == TRIM_AC6_SUPPORT && S.variant == TRIM_AC6_SUPPORT &&
          S.fe - S.fb <= min(D.local_edges_max, gridDim.x * (blockDim.x >> 5));
@@ -1285,7 +1290,9 @@ __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
 __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   Sched& L = B.S;
   const uint32_t r = L.round;
-  constexpr uint32_t variant = TRIM_AC6_ONLY ? TRIM_AC6_SUPPORT : TRIM_AC4_PUSH;
+  constexpr uint32_t variant = TRIM_AC6_ONLY   ? TRIM_AC6_SUPPORT
+                               : TRIM_AC3_ONLY ? TRIM_AC3_PULL
+                                               : TRIM_AC4_PUSH;
   L.vcount[variant] += 1u;
   L.c4w = L.w_end;  // the stretch's first round pushed every pending entry
   L.e_c4 = L.e_end;
@@ -1358,8 +1365,8 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     const unsigned long long add =
         (1ull << 48) | ((unsigned long long)B.lq_ovf << 32) | (unsigned long long)B.lq_k;
     const unsigned long long base = S.lbase[slot];
-    // AC-6 rounds hand levels, records and list heads to other CTAs.
-    if (TRIM_AC6_ONLY) fence_acq_rel();
+    // AC-6 rounds hand levels, records and list heads to other CTAs, AC-3 rounds levels.
+    if (TRIM_AC6_ONLY || TRIM_AC3_ONLY) fence_acq_rel();
     // Otherwise no fence before the arrival: across a local barrier CTAs exchange nothing
     // through plain memory, only counter decrements, and every decrement of
     // this round has returned its value (it is performed at L2) before this
@@ -1378,7 +1385,7 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       }
       cur = ld_relaxed64(&D.C->lbar[slot]);
     }
-    if (TRIM_AC6_ONLY) fence_acq_rel();
+    if (TRIM_AC6_ONLY || TRIM_AC3_ONLY) fence_acq_rel();
     const unsigned long long d = cur - base;
     S.lbase[slot] = cur;
     S.lround += 1u;
@@ -1403,6 +1410,9 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       B.lq_next = LQ_LEAVE;
     }
     // the next round fills the buffer this round read
+#if TRIM_AC3_ONLY
+    B.live_n[b ^ 1u] = 0u;
+#endif
     B.lq_cnt[b ^ 1u] = 0ull;
     B.lq_vend[b ^ 1u] = 0u;
     B.lq_k = 0u;
@@ -1413,7 +1423,7 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
   return B.err == 0u;
 }
 
-#if !TRIM_AC6_ONLY
+#if !TRIM_AC6_ONLY && !TRIM_AC3_ONLY
 // Runs local rounds from round B.S.round on: the first pushes the pending
 // work-list entries (one per warp), later ones the predecessors in the CTA's
 // queue. A removed vertex's row bounds are loaded once its counter has reached
@@ -2581,6 +2591,84 @@ __device__ ROUND_FN void ac3_round(const Dev& D, Cta& B, const Sched& S, uint32_
   stats_flush(D, B, K);
 }
 
+#if TRIM_LOCAL && TRIM_AC3_ONLY
+// A run of AC-3 alone, from round 1 to the end: each CTA sweeps its own vertices
+// (every nwarps-th block of 32 per warp) and keeps its survivors in its own part of
+// the live lists, in the part's order of blocks. A round needs no shared list, no space
+// reservation, no dead log and no read of the control block; it ends at a fenced
+// local barrier that carries the removals. A survivor is live: no level is
+// loaded for it. Returns false on a timeout.
+//
+// Small rounds are bound by their fixed parts (flush and reservations 1.1 us,
+// barrier and schedule step 3, the level of every live vertex one more
+// dependent load), large ones by the rows. Kernel us per run, through the shared
+// lists / as here: planted graphs of 1,000 vertices (17 rounds) 95 / 59, 100,000 (22)
+// 164 / 120, 1,000,000 (31) 582 / 446; deep cascade of 2^20 (301) 7,663 / 4,224; R-MAT
+// of 2^22 (4) 231 / 207.
+__device__ __noinline__ bool local_stretch() {
+  const Dev& D = cta_dev;
+  Cta& B = cta_state;
+  Counters K;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+  const uint32_t n = D.n, blocks = (n + 31u) / 32u, nwarps = gridDim.x * wpb;
+  // first entry of the CTA's part, and its blocks
+  const uint32_t turns = blocks / nwarps, left = blocks % nwarps;
+  const uint32_t part = 32u * (turns * wpb * blockIdx.x + min(left, blockIdx.x * wpb));
+  const uint32_t own = turns * wpb + min(wpb, left - min(left, blockIdx.x * wpb));
+  bool first = true;
+  while (true) {
+    const uint32_t r = B.S.round;
+    const uint32_t b = B.S.lround & 1u;
+    const uint32_t* in = (b ? D.live0 : D.live1) + part;  // written in the last round
+    uint32_t* out = (b ? D.live1 : D.live0) + part;
+    start_round(D, r);
+    const uint32_t N = first ? own * 32u : B.live_n[b ^ 1u];
+    for (uint32_t base = warp * 32u; base < N; base += blockDim.x) {
+      const uint32_t k = base + lane;
+      bool alive = k < N;
+      uint32_t v = 0u, s = 0, d = 0, i0 = 0;
+      if (first) {  // block q of the CTA is its warp q % wpb's, in turn q / wpb
+        const uint32_t q = base / 32u;
+        v = 32u * ((q / wpb) * nwarps + blockIdx.x * wpb + q % wpb) + lane;
+        alive = v < n;
+        K.swept += alive ? 1 : 0;
+        alive = alive && ldcg(&D.level[v]) == LIVE;
+        if (alive) row_bounds(D, v, s, d);
+      } else if (alive) {
+        v = ldcg(&in[k]);
+        i0 = ldcg(&D.supp[v]);
+        row_bounds(D, v, s, d);
+        K.swept += 1;
+      }
+      uint32_t i = 0;
+      bool resolved = true;
+      if (alive) i = scan_thread(D, v, s, d, i0, r, 2, resolved, K);
+      scan_warp_finish(D, resolved, v, s, d, i, r, K);
+      const bool dies = alive && i >= d, stays = alive && !dies;
+      if (dies) D.level[v] = r;
+      if (stays && (i != i0 || first)) D.supp[v] = i;
+      const unsigned gone = __ballot_sync(FULL, dies), kept = __ballot_sync(FULL, stays);
+      uint32_t at = 0;
+      if (lane == 0) {
+        if (gone) atomicAdd(&B.lq_k, (uint32_t)__popc(gone));
+        if (kept) at = atomicAdd(&B.live_n[b], (uint32_t)__popc(kept));
+      }
+      at = __shfl_sync(FULL, at, 0);
+      if (stays) out[at + __popc(kept & ((1u << lane) - 1u))] = v;
+    }
+    if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0) {
+      __syncthreads();
+      if (threadIdx.x == 0) D.C->t_work[r & 3] = globaltimer();
+    }
+    if (!local_barrier(D, B, b, r)) break;
+    if (B.lq_next != LQ_GO) break;  // done (a round cannot overflow)
+    first = false;
+  }
+  stats_flush(D, B, K);
+  return B.err == 0u;
+}
+#endif
+
 // ------------------------------------------------------------------ AC-6
 
 #if !TRIM_AC6_ONLY
@@ -3620,6 +3708,9 @@ __global__ void __launch_bounds__(512, TRIM_MIN_BLOCKS) TRIM_KERNEL(const __grid
     B.lq_cnt[0] = B.lq_cnt[1] = 0;
     B.lq_vend[0] = B.lq_vend[1] = 0;
     B.lq_k = B.lq_ovf = B.lq_pushed = 0;
+#if TRIM_AC3_ONLY
+    B.live_n[0] = B.live_n[1] = 0;
+#endif
 #endif
   }
   if (threadIdx.x == 0 && B.resume) {
