@@ -1300,10 +1300,12 @@ __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   L.skew += nF;
   if (blockIdx.x == 0) {
     Ctrl* C = D.C;
-    C->vcount[variant] = L.vcount[variant];
-    C->rounds = nF ? r + 1u : r;
-    C->n_dead = L.fe + nF;
-    C->local_rounds = L.lround;
+    if (nF == 0u) {  // (a stretch that goes on or leaves publishes later)
+      C->vcount[variant] = L.vcount[variant];
+      C->rounds = r;
+      C->n_dead = L.fe;
+      C->local_rounds = L.lround;
+    }
     if ((D.flags & F_ROUND_LOG) && D.rlog != nullptr && r >= 1u && r - 1u < D.rlog_cap) {
       trim_round_rec_t* rec = &D.rlog[r - 1u];
       rec->round = r;
@@ -1373,6 +1375,23 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     // arrival is issued. Levels written here are read after the kernel or
     // after an ordinary (fenced) barrier.
     red_relaxed_add64(&D.C->lbar[slot], add);
+    // the next round fills the buffer this round read
+#if TRIM_AC3_ONLY
+    B.live_n[b ^ 1u] = 0u;
+#endif
+    B.lq_cnt[b ^ 1u] = 0ull;
+    B.lq_vend[b ^ 1u] = 0u;
+    B.lq_k = 0u;
+    B.lq_ovf = 0u;
+    B.lq_pushed = 0u;
+    // the stretch ends before the last round of a committed stretch (the
+    // scheduler reads its features) and, where the asynchronous tail may take
+    // over (asked every ASYNC_RETRY rounds), as it starts from the work list
+    const bool last = (MODES & M_SCHED) && r + 1u >= S.cstop;
+#if TRIM_ASYNC
+    const bool ask = D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
+                     r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u;
+#endif
     const uint64_t t0 = globaltimer();
     // relaxed polls: an acquiring load would also invalidate this SM's L1 on
     // every iteration, and nothing read after this barrier needs it
@@ -1390,15 +1409,11 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     S.lbase[slot] = cur;
     S.lround += 1u;
     const uint32_t nF = (uint32_t)d, n_ovf = (uint32_t)(d >> 32) & 0xFFFFu;
-    // the stretch ends before the last round of a committed stretch (the
-    // scheduler reads its features) and, where the asynchronous tail may take
-    // over (asked every ASYNC_RETRY rounds), as it starts from the work list
-    const bool stop = ((MODES & M_SCHED) && r + 1u >= S.cstop)
 #if TRIM_ASYNC
-                      || (D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
-                       r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u && async_few(nF))
+    const bool stop = last || (ask && async_few(nF));
+#else
+    const bool stop = last;
 #endif
-        ;
     if (n_ovf == 0u && (nF == 0u || !stop)) {
       local_close(D, B, nF);  // every removal of the round is in the queues
       B.lq_next = nF ? LQ_GO : LQ_DONE;
@@ -1409,15 +1424,6 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       if (blockIdx.x == 0) D.C->local_rounds = S.lround;
       B.lq_next = LQ_LEAVE;
     }
-    // the next round fills the buffer this round read
-#if TRIM_AC3_ONLY
-    B.live_n[b ^ 1u] = 0u;
-#endif
-    B.lq_cnt[b ^ 1u] = 0ull;
-    B.lq_vend[b ^ 1u] = 0u;
-    B.lq_k = 0u;
-    B.lq_ovf = 0u;
-    B.lq_pushed = 0u;
   }
   __syncthreads();
   return B.err == 0u;
@@ -1533,6 +1539,7 @@ __device__ __noinline__ bool local_stretch() {
         }
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
+          if (q && base + blockDim.x >= qe) break;  // CTA-uniform
           bool pred = valid[q] && push_removes(old[q], dir[q]);
 #if TRIM_MODES & 16
           count_rows(D, pred, u[q], K);
