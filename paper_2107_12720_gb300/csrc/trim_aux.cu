@@ -47,12 +47,10 @@ __device__ unsigned block_sum(unsigned x) {
 
 }  // namespace
 
-// Control block reset before every run (one thread).
+// Control block reset before every run (one warp).
 __global__ void trim_reset_ctrl_kernel(Ctrl* C) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    unsigned* w = reinterpret_cast<unsigned*>(C);
-    for (size_t i = 0; i < sizeof(Ctrl) / 4; ++i) w[i] = 0u;
-  }
+  unsigned* w = reinterpret_cast<unsigned*>(C);
+  for (unsigned i = threadIdx.x; i < sizeof(Ctrl) / 4; i += blockDim.x) w[i] = 0u;
 }
 
 __global__ void trim_status_kernel(const uint32_t* level, uint32_t n, uint8_t* status) {
