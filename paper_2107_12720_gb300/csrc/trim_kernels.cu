@@ -111,9 +111,8 @@ struct WarpSlice {
 // In+out trimming (flavour 17) runs local rounds too: its queue holds, per
 // removed vertex, the one row that still matters (see inout_round), and per
 // queued neighbour which of its two counters the push decrements.
-// So does AC-6 (flavours 2 and 34, the ones that run nothing else): its queue
-// holds the removed vertices, whose supporting sets the CTA re-scans in the next
-// round. And so does AC-3 (flavours 4 and 36), with a live list per CTA.
+// So does AC-6 (flavours 2 and 34, the ones that run nothing else), with the dead log
+// as the queue of all CTAs (see its local_stretch). And so does AC-3 (flavours 4 and 36), with a live list per CTA.
 #if TRIM_MODES == 1 || TRIM_MODES == 9
 #define TRIM_LOCAL 1
 #define TRIM_ASYNC 1
@@ -159,10 +158,7 @@ struct Cta {
 #if TRIM_LOCAL
 #if TRIM_AC3_ONLY
   uint32_t live_n[2];  // local AC-3 rounds: the CTA's live list, by local-round parity
-#elif TRIM_AC6_ONLY
-  // local AC-6 rounds: the vertices this CTA removed, by local-round parity
-  uint32_t lq_ids[2][LQ_ENTRIES];
-#else
+#elif !TRIM_AC6_ONLY
   // local queues, double-buffered by local-round parity: buffer b is filled in
   // the round whose lround parity is b and read in the next one
   uint32_t lq_ids[2][LQ_EDGES];       // predecessors to decrement
@@ -1287,7 +1283,11 @@ __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
 #if TRIM_AC3_ONLY
   return D.local_edges_max != 0u;  // from the first round to the last
 #elif TRIM_AC6_ONLY
-  // AC-6: the sets were built, and the last round's removals are at most one to a warp
+  // AC-6: the sets were built, and the last round's removals are at most one to a
+  // warp (kernel ms, with up to one / two / four / eight: deep cascades of 2^20 vertices
+  // with 7,340 to a level 1.387 / 1.428 / 1.428 / 1.429, with 14,680 0.826 / 0.826 /
+  // 1.046 / 1.043; planted graphs of 300,000 vertices 0.229 / 0.246 / 0.247 / 0.247, of
+  // 1,000,000 0.287 / 0.288 / 0.292 / 0.461)
   return S.prev_variant == TRIM_AC6_SUPPORT && S.variant == TRIM_AC6_SUPPORT &&
          S.fe - S.fb <= min(D.local_edges_max, gridDim.x * (blockDim.x >> 5));
 #else
@@ -1313,7 +1313,7 @@ __device__ void local_close(const Dev& D, Cta& B, uint32_t nF) {
   L.c4w = L.w_end;  // the stretch's first round pushed every pending entry
   L.e_c4 = L.e_end;
   L.bmax = 0u;
-  L.skew += nF;
+  if (!TRIM_AC6_ONLY) L.skew += nF;  // (those are in the log)
   if (blockIdx.x == 0) {
     Ctrl* C = D.C;
     if (nF == 0u) {  // (a stretch that goes on or leaves publishes later)
@@ -1434,9 +1434,7 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
       local_close(D, B, nF);  // every removal of the round is in the queues
       B.lq_next = nF ? LQ_GO : LQ_DONE;
     } else {
-      // advance() closes the round after the handover (AC-6: the queued removals
-      // join the dead log and are counted there)
-      if (!TRIM_AC6_ONLY) S.skew += nF;
+      S.skew += nF;  // advance() closes the round after the work-list handover
       if (blockIdx.x == 0) D.C->local_rounds = S.lround;
       B.lq_next = LQ_LEAVE;
     }
@@ -3046,40 +3044,33 @@ __device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_
 //
 // Measured (kernel ms per run, before: one list head, members' level, position and row
 // loaded one after the other, every round through the global lists): deep
-// cascades of 1,000,003 vertices and 1,503 rounds 16.7 and now 10.6, of 2^20 and 2,802
-// rounds 33.2 and 19.6, of 2^16 and 302 rounds 3.4 and 2.13. Without the records 13.7
-// (one head 17.3, two 14.6, sixteen 12.3); records and one general walk for all
-// rounds 13.1. A round is now 6.7 us: about 3.5 of it a walk and a move (a warp alone
+// cascades of 1,000,003 vertices and 1,503 rounds 16.7 and now 10.2, of 2^20 and 2,802
+// rounds 33.2 and 19.1, of 2^16 and 302 rounds 3.4 and 2.08. On the way: local rounds
+// without the records 13.7 (one head 17.3, two 14.6, sixteen 12.3), with records and
+// one general walk for all rounds 13.1, with the short walk and queues per CTA 10.6. A
+// round is now 6.4 us: about 3.5 of it a walk and a move (a warp alone
 // on its scheduler takes 5 cycles an instruction, an access 400, an atomic 800), 0.65
 // the fence, 1.1 the barrier.
 
-// Warp-collective, local rounds: lanes with pred remove u in round r. The CTA
-// queues up to cap of them in buffer b; the others go to the dead log and mark
-// the round as overflowing.
-__device__ __forceinline__ void local_remove(const Dev& D, Cta& B, bool pred, uint32_t u,
-                                             uint32_t r, uint32_t b, uint32_t cap) {
-  const unsigned lane = lane_id();
-  const unsigned mask = __ballot_sync(FULL, pred);
-  if (mask == 0u) return;
-  const uint32_t k = __popc(mask);
+// Warp-collective, local rounds: space in the dead log for the lanes of mask (lane 0's
+// atomic, under way until log_removed).
+__device__ __forceinline__ uint32_t log_space(const Dev& D, Cta& B, unsigned mask) {
   uint32_t at = 0;
-  if (lane == 0) {
-    at = (uint32_t)atomicAdd(&B.lq_cnt[b], (unsigned long long)k);
-    if (at + k <= cap) {
-      atomicMax(&B.lq_vend[b], at + k);
-      atomicAdd(&B.lq_k, k);
-    } else {
-      B.lq_ovf = 1u;
-    }
+  if (mask && lane_id() == 0) {
+    at = atomicAdd(&D.C->log_len, (uint32_t)__popc(mask));
+    atomicAdd(&B.lq_k, (uint32_t)__popc(mask));
   }
+  return at;
+}
+__device__ __forceinline__ void log_removed(const Dev& D, unsigned mask, uint32_t at, uint32_t u,
+                                            uint32_t r) {
+  if (mask == 0u) return;
   at = __shfl_sync(FULL, at, 0);
-  if (at + k <= cap) {
-    if (pred) {
-      B.lq_ids[b][at + __popc(mask & ((1u << lane) - 1u))] = u;
-      D.level[u] = r;
-    }
-  } else {
-    append_dead(D, B, pred, u, r, D.live0);
+  if (at + __popc(mask) > D.n) {
+    if (lane_id() == 0) set_error(D, TRIM_ERR_STATE, 0xD8);
+  } else if (mask >> lane_id() & 1u) {
+    D.log[at + __popc(mask & ((1u << lane_id()) - 1u))] = u;
+    D.level[u] = r;
   }
 }
 
@@ -3089,9 +3080,11 @@ __device__ __forceinline__ void local_remove(const Dev& D, Cta& B, bool pred, ui
 // without one they are removed.
 template <bool LOCAL>
 __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uint32_t v, uint32_t t,
-                                           uint32_t pos, uint32_t end, uint32_t r, Counters& K,
-                                           uint32_t b, uint32_t cap) {
+                                           uint32_t pos, uint32_t end, uint32_t r, Counters& K) {
   const bool cand = valid && t != NIL;
+  // members without a successor left die: their log space is asked for first
+  const unsigned now = __ballot_sync(FULL, valid && !cand);
+  const uint32_t at = LOCAL ? log_space(D, B, now) : 0u;
   uint32_t lv = 0, after = NIL;
   if (cand) {
     lv = ldcg(&D.level[t]);
@@ -3099,10 +3092,13 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
     K.edges += 1;
   }
   bool found = cand && lv >= r;
-  if (__any_sync(FULL, cand && !found)) {  // the rare case: scan on
+  const unsigned scan = __ballot_sync(FULL, cand && !found);
+  if (scan) {  // the rare case: scan on
     uint32_t i = pos + 1u;
-    bool resolved = true;
-    if (cand && !found) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
+    bool resolved = !(cand && !found);
+    // one or two rows: the whole warp scans each, 32 successors in one step; more of
+    // them: each lane its own first, four successors in a step
+    if (__popc(scan) > 2 && !resolved) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
     scan_warp_finish(D, resolved, v, 0u, end, i, r, K);
     if (cand && !found && i < end) {
       found = true;
@@ -3116,9 +3112,13 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
     D.s_rec[v] = make_uint4(next, after, pos + 1u, end);
   }
   K.cand += valid ? 1 : 0;
-  const bool dies = valid && !found;
-  if (LOCAL) local_remove(D, B, dies, v, r, b, cap);
-  else append_dead(D, B, dies, v, r, D.live0);
+  if (LOCAL) {
+    log_removed(D, now, at, v, r);
+    const unsigned late = __ballot_sync(FULL, cand && !found);  // after a scan
+    if (late) log_removed(D, late, log_space(D, B, late), v, r);
+  } else {
+    append_dead(D, B, valid && !found, v, r, D.live0);
+  }
 }
 
 // Warp-collective: re-scans the supporting sets of up to 32 removed vertices,
@@ -3188,7 +3188,7 @@ __device__ __forceinline__ void ac6_sets(const Dev& D, Cta& B, bool has, uint32_
         const uint4 m = st[valid ? nbuf - take + lane : 0u];
         __syncwarp();
         nbuf -= take;
-        ac6_rescan<false>(D, B, valid, m.x, m.y, m.z, m.w, r, K, 0u, 0u);
+        ac6_rescan<false>(D, B, valid, m.x, m.y, m.z, m.w, r, K);
       }
     }
   }
@@ -3196,8 +3196,7 @@ __device__ __forceinline__ void ac6_sets(const Dev& D, Cta& B, bool has, uint32_
 
 // The same for the set of one removed vertex w in a local round. A warp that runs
 // alone on its scheduler pays for every instruction as well: this is the short form.
-__device__ __forceinline__ void ac6_set(const Dev& D, Cta& B, uint32_t w, uint32_t r, Counters& K,
-                                        uint32_t b, uint32_t cap) {
+__device__ __forceinline__ void ac6_set(const Dev& D, Cta& B, uint32_t w, uint32_t r, Counters& K) {
   const unsigned lane = lane_id();
   uint4* st = reinterpret_cast<uint4*>(slice(threadIdx.x >> 5, 1));
   uint32_t cur = lane < AC6_HEADS ? ldcg(set_head(D, w, lane)) : NIL;
@@ -3233,7 +3232,7 @@ __device__ __forceinline__ void ac6_set(const Dev& D, Cta& B, uint32_t w, uint32
       const uint4 m = st[valid ? nbuf - take + lane : 0u];
       __syncwarp();
       nbuf -= take;
-      ac6_rescan<true>(D, B, valid, m.x, m.y, m.z, m.w, r, K, b, cap);
+      ac6_rescan<true>(D, B, valid, m.x, m.y, m.z, m.w, r, K);
     }
   }
 }
@@ -3256,62 +3255,38 @@ __device__ ROUND_FN bool ac6_round(const Dev& D, Cta& B, const Sched& S, uint32_
   return true;
 }
 
-// Local AC-6 rounds, from round B.S.round on: the first takes the removals of the
-// last round from the dead log, one to a warp, later ones the CTA's own queue. A
-// round needs no log, no space reservation and no read of the control block; it
-// ends at a fenced local barrier that carries its totals (the fence covers
-// levels, records and heads). The stretch ends when nothing was removed (the run
-// is done) or a queue overflowed; then the queued vertices join the dead log and
-// the round ends like an ordinary one. The queues are bounded by a few times the
-// mean load, at least LQ_SETS: a CTA has a warp for each of 16 sets, but removals drift
-// to few CTAs (a vertex stays with the set it leaves last). Bounds of 32, 8 and 4, ms: 11.8,
-// 10.7 and 11.1 (1,000,003 vertices), 24.3, 19.6 and 19.8 (2^20, 2,802 rounds). Returns
-// false on a timeout.
-constexpr uint32_t LQ_SETS = 8;  // least bound of the queues
+// Local AC-6 rounds, from round B.S.round on: the removals of the last round, in the
+// dead log, are spread over all warps, and a warp writes what its set removes to the
+// log at once. A round needs no slices, no flush and no read of the control block; it
+// ends at a fenced local barrier that carries its totals (the fence covers the
+// log, levels, records and heads). The stretch ends when nothing was removed (the
+// run is done), or with more removals than warps, for ordinary rounds.
+// Returns false on a timeout.
+//
+// One log for all CTAs, an atomic and a load more per round than a queue in each:
+// a vertex stays with the set it leaves last, so the queues of few CTAs filled up
+// (175 to 229 of 304 CTAs had none) and had to be spread again by ordinary rounds. Kernel
+// ms with those queues / with the log: 1,000,003 vertices in 1,503 rounds 10.6 / 10.2, 2^20 in
+// 301 3.09 / 2.49, planted 100,000 0.187 / 0.158.
 __device__ __noinline__ bool local_stretch() {
   const Dev& D = cta_dev;
   Cta& B = cta_state;
   Counters K;
-  const unsigned lane = lane_id();
-  const uint32_t cap = min(LQ_ENTRIES, max(LQ_SETS, LQ_SKEW * ((B.S.fe - B.S.fb) / gridDim.x)));
-  bool first = true;
+  const uint32_t nw = gridDim.x * (blockDim.x >> 5);
   while (true) {
     const uint32_t r = B.S.round;
-    const uint32_t b = B.S.lround & 1u;
     start_round(D, r);
-    const uint32_t step = first ? gridDim.x * (blockDim.x >> 5) : blockDim.x >> 5;
-    const uint32_t end = first ? B.S.fe - B.S.fb : B.lq_vend[b ^ 1u];
-    const uint32_t from = B.S.fb - B.S.skew;
-    uint32_t k = threadIdx.x >> 5;
-    if (first) k = k * gridDim.x + blockIdx.x;
-    for (; k < end; k += step) {
-      const uint32_t w = first ? ldcg(&D.log[from + k]) : B.lq_ids[b ^ 1u][k];
-      ac6_set(D, B, w, r, K, b, cap);
-    }
+    const uint32_t from = B.S.fb - B.S.skew, N = B.S.fe - B.S.fb;
+    for (uint32_t k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; k < N; k += nw)
+      ac6_set(D, B, ldcg(&D.log[from + k]), r, K);
     if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0) {
       __syncthreads();
       if (threadIdx.x == 0) D.C->t_work[r & 3] = globaltimer();
     }
-    if (!local_barrier(D, B, b, r)) break;
-    const uint32_t next = B.lq_next;
-    if (next == LQ_DONE) break;
-    if (next == LQ_GO) {
-      first = false;
-      continue;
-    }
-    const uint32_t ne = B.lq_vend[b];
-    for (uint32_t i0 = (threadIdx.x >> 5) * 32u; i0 < ne; i0 += blockDim.x) {
-      const uint32_t i = i0 + lane;
-      append_dead(D, B, i < ne, i < ne ? B.lq_ids[b][i] : 0u, r, D.live0);
-    }
-    flush_round(D, B, r, D.live0);
-    if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0 && threadIdx.x == 0)
-      D.C->t_flush[r & 3] = globaltimer();
-    if (!grid_barrier(D, B, false)) break;
-    if (threadIdx.x < 32) advance(D, B);
-    __syncthreads();
-    break;
+    if (!local_barrier(D, B, B.S.lround & 1u, r)) break;
+    if (B.lq_next != LQ_GO || B.S.fe - B.S.fb > nw) break;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) D.C->local_rounds = B.S.lround;
   stats_flush(D, B, K);
   return B.err == 0u;
 }
