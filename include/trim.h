@@ -167,7 +167,8 @@ typedef struct {
   float device_ms;          /* trim time between events around the device work          */
   uint64_t edges_inspected; /* TRIM_FLAG_STATS: out-edge targets read by AC-6/AC-3 scans.
                                Scans read targets in groups (one for the first successor, 4
-                               per thread step, up to 32 per warp step) and a scan that resumes after its support
+                               per thread step, up to 32 per warp step) and a scan that
+                               resumes after its support
                                reads again the targets its last group loaded past it, so
                                the count can exceed m for AC-6, whose logical inspections
                                are at most m (Section 8)                                */
@@ -285,13 +286,15 @@ trim_err_t trim_create_implicit(const trim_implicit_graph_t* g, void* cuda_strea
 /* ---- SCC decomposition (Section 1: the use trimming is made for) ----
  * trim_run_scc labels every vertex with its strongly connected component:
  * comp[v] = the smallest vertex id of v's component (the same labels whatever
- * the order of the work). Steps, all on the device, driven from the host:
+ * the order of the work). Steps, all on the device, step 1 in one launch and
+ * the others in a second (one host read at the end):
  *  1. in+out trimming (trim_run_inout): every removed vertex is a size-1
  *     component (it has no in-edge or no out-edge among the others);
  *  2. size-2 trimming: two open vertices that are each other's only open
  *     successor (or each other's only open predecessor) form a component;
- *  3. forward-backward steps (Section 1's FW-BW, from every vertex at once):
- *     forward, every open vertex learns the smallest open vertex that reaches
+ *  3. forward-backward steps (Section 1's FW-BW): the first from one pivot
+ *     (the open vertex with the largest min(in-degree, out-degree)), the
+ *     others from every vertex at once: forward, every open vertex learns the smallest open vertex that reaches
  *     it (label propagation along G); a vertex r that keeps its own label is
  *     reached by no smaller vertex, and the backward search from r through
  *     G^T among the vertices labelled r collects exactly r's component, whose

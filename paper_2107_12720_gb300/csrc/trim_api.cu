@@ -438,7 +438,7 @@ trim_err_t build_transpose(trim_ctx* c) {
     const uint32_t shift = lg > keep ? lg - keep : 0u;
     const uint32_t nb = (uint32_t)(((uint64_t)n + (1u << shift) - 1) >> shift);
     const uint32_t sms = (uint32_t)c->sm_count;
-    const uint32_t piece = (m + sms - 1) / sms;
+    const uint32_t piece = (uint32_t)(((uint64_t)m + sms - 1) / sms);
     uint32_t *counts = nullptr, *start = nullptr, *cursor = nullptr;
     unsigned long long* pairs = nullptr;
     TRY(dalloc(c, &counts, (size_t)nb + 1));  // and pass 4's ticket
