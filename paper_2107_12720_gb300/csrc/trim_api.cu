@@ -711,9 +711,9 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   const size_t n = c->n;
   if (flags & TRIM_FLAG_ROUND_LOG) c->rlog_cap = (uint32_t)std::min<uint64_t>(n + 1, 1u << 20);
   ArenaPlan A;
-  // records of 16 bytes (AC-3: its support positions), AC-6's sets, and four list
-  // heads per vertex (AC-3: its live lists)
-  const size_t a_level = A.add<uint32_t>(n), a_rec = A.add<uint4>(n);
+  // AC-6's records of 16 bytes, its sets, and four list heads per vertex; or AC-3's
+  // live lists of 16 bytes an entry (in parts of whole blocks of 32 vertices)
+  const size_t a_level = A.add<uint32_t>(n), a_rec = A.add<uint4>(n + 32);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_slist = A.add<uint32_t>(n), a_log = A.add<uint32_t>(n);
   const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
@@ -879,7 +879,7 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   else if (inout) flavour = kFlavourInout;
   else if (variant <= TRIM_AC3_PULL) flavour = (int)variant;
   else if (seg_flavour >= 0) flavour = seg_flavour;
-  if (variant == TRIM_AC6_SUPPORT) {  // AC-6 throughout
+  if (variant == TRIM_AC6_SUPPORT || variant == TRIM_AC3_PULL) {  // one of them throughout
     D.s_rec = c->s_rec;
     D.s_heads = reinterpret_cast<uint4*>(c->live0);
   }

@@ -158,7 +158,7 @@ struct Dev {
   uint32_t* supp;     // edge_index of AC-3 / AC-6: position of the current support
   // runs of AC-6 alone: per vertex its record (next member of its list, next
   // successor to try, its position, row end) and four list heads, in the arrays from
-  // cnt to s_next and from live0 to w4_eoff
+  // cnt to s_next and from live0 to w4_eoff; runs of AC-3 alone: the live lists there
   uint4* s_rec;
   uint4* s_heads;
   uint32_t* s_head;   // AC-6 supporting sets added during the epoch (intrusive lists)

@@ -2617,15 +2617,16 @@ __device__ ROUND_FN void ac3_round(const Dev& D, Cta& B, const Sched& S, uint32_
 // (every nwarps-th block of 32 per warp) and keeps its survivors in its own part of
 // the live lists, in the part's order of blocks. A round needs no shared list, no space
 // reservation, no dead log and no read of the control block; it ends at a fenced
-// local barrier that carries the removals. A survivor is live: no level is
-// loaded for it. Returns false on a timeout.
+// local barrier that carries the removals. A list entry has all that a sweep needs:
+// the vertex, its support, the support's position and the row's end; while the
+// support lives, that is the entry and one level. Returns false on a timeout.
 //
 // Small rounds are bound by their fixed parts (flush and reservations 1.1 us,
 // barrier and schedule step 3, the level of every live vertex one more
 // dependent load), large ones by the rows. Kernel us per run, through the shared
-// lists / as here: planted graphs of 1,000 vertices (17 rounds) 95 / 59, 100,000 (22)
-// 164 / 120, 1,000,000 (31) 582 / 446; deep cascade of 2^20 (301) 7,663 / 4,224; R-MAT
-// of 2^22 (4) 231 / 207.
+// lists / with lists per CTA of vertices alone / as here: planted graphs of 1,000
+// vertices (17 rounds) 95 / 59 / 59, 100,000 (22) 164 / 116 / 90, 1,000,000 (31) 582 / 446 /
+// 275; deep cascade of 2^20 (301) 7,663 / 4,224 / 2,640; R-MAT of 2^22 (4) 231 / 207 / 136.
 __device__ __noinline__ bool local_stretch() {
   const Dev& D = cta_dev;
   Cta& B = cta_state;
@@ -2640,42 +2641,55 @@ __device__ __noinline__ bool local_stretch() {
   while (true) {
     const uint32_t r = B.S.round;
     const uint32_t b = B.S.lround & 1u;
-    const uint32_t* in = (b ? D.live0 : D.live1) + part;  // written in the last round
-    uint32_t* out = (b ? D.live1 : D.live0) + part;
+    const uint4* in = (b ? D.s_rec : D.s_heads) + part;  // written in the last round
+    uint4* out = (b ? D.s_heads : D.s_rec) + part;
     start_round(D, r);
     const uint32_t N = first ? own * 32u : B.live_n[b ^ 1u];
     for (uint32_t base = warp * 32u; base < N; base += blockDim.x) {
       const uint32_t k = base + lane;
-      bool alive = k < N;
-      uint32_t v = 0u, s = 0, d = 0, i0 = 0;
+      bool alive = k < N, stays = false;
+      uint4 x = make_uint4(0u, 0u, 0u, 0u);
       if (first) {  // block q of the CTA is its warp q % wpb's, in turn q / wpb
         const uint32_t q = base / 32u;
-        v = 32u * ((q / wpb) * nwarps + blockIdx.x * wpb + q % wpb) + lane;
-        alive = v < n;
+        x.x = 32u * ((q / wpb) * nwarps + blockIdx.x * wpb + q % wpb) + lane;
+        alive = x.x < n;
         K.swept += alive ? 1 : 0;
-        alive = alive && ldcg(&D.level[v]) == LIVE;
-        if (alive) row_bounds(D, v, s, d);
+        alive = alive && ldcg(&D.level[x.x]) == LIVE;
+        if (alive) {
+          uint32_t s, d;
+          row_bounds(D, x.x, s, d);
+          x.z = s;
+          x.w = s + d;
+        }
       } else if (alive) {
-        v = ldcg(&in[k]);
-        i0 = ldcg(&D.supp[v]);
-        row_bounds(D, v, s, d);
+        x = __ldcg(&in[k]);
+        stays = ldcg(&D.level[x.y]) >= r;
         K.swept += 1;
+        K.edges += 1;
       }
-      uint32_t i = 0;
-      bool resolved = true;
-      if (alive) i = scan_thread(D, v, s, d, i0, r, 2, resolved, K);
-      scan_warp_finish(D, resolved, v, s, d, i, r, K);
-      const bool dies = alive && i >= d, stays = alive && !dies;
-      if (dies) D.level[v] = r;
-      if (stays && (i != i0 || first)) D.supp[v] = i;
-      const unsigned gone = __ballot_sync(FULL, dies), kept = __ballot_sync(FULL, stays);
+      if (__any_sync(FULL, alive && !stays)) {
+        const bool scan = alive && !stays;
+        uint32_t i = x.z + (first ? 0u : 1u);
+        bool resolved = true;
+        if (scan) i = scan_thread(D, x.x, 0u, x.w, i, r, 2, resolved, K);
+        scan_warp_finish(D, resolved, x.x, 0u, x.w, i, r, K);
+        if (scan && i < x.w) {
+          stays = true;
+          x.y = row_target(D, x.x, 0u, i);
+          x.z = i;
+        } else if (scan) {
+          D.level[x.x] = r;
+        }
+      }
+      const unsigned gone = __ballot_sync(FULL, alive && !stays);
+      const unsigned kept = __ballot_sync(FULL, stays);
       uint32_t at = 0;
       if (lane == 0) {
         if (gone) atomicAdd(&B.lq_k, (uint32_t)__popc(gone));
         if (kept) at = atomicAdd(&B.live_n[b], (uint32_t)__popc(kept));
       }
       at = __shfl_sync(FULL, at, 0);
-      if (stays) out[at + __popc(kept & ((1u << lane) - 1u))] = v;
+      if (stays) out[at + __popc(kept & ((1u << lane) - 1u))] = x;
     }
     if ((D.flags & F_ROUND_LOG) && blockIdx.x == 0) {
       __syncthreads();
