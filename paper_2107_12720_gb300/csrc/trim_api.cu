@@ -968,13 +968,15 @@ trim_err_t run_scc(trim_ctx* c, uint32_t* out, int out_on_device, trim_scc_stats
   A.fa = c->scc_fa; A.fb = c->scc_fb;
   // lists of one run, in arrays that the in+out run is done with
   A.open0 = c->live0; A.open1 = c->live1; A.heavy = c->log;
+  A.hpos = c->w4_eoff;
   A.C = c->scc_ctl;
   A.spin_limit_ns = c->params.spin_limit_ns;
   CK(cudaMemsetAsync(c->scc_ctl, 0, sizeof(trimk::SccCtl), c->stream));
   CK(cudaMemsetAsync(&c->scc_ctl->least, 0xFF, 4, c->stream));
-  // a small graph takes a small grid: every phase ends at a barrier of its CTAs
-  const uint32_t want = (c->n + kSccThreads - 1) / kSccThreads;
-  const uint32_t grid = std::min<uint32_t>(want, (uint32_t)c->scc_grid);
+  // a small graph takes a small grid (every phase ends at a barrier of its CTAs): a
+  // thread to a vertex, or to 16 edges where rows are dense
+  const uint64_t want = std::max<uint64_t>(c->n, c->m / 16) / kSccThreads + 1;
+  const uint32_t grid = (uint32_t)std::min<uint64_t>(want, (uint64_t)c->scc_grid);
   void* args[] = {&A};
   CK(cudaLaunchCooperativeKernel((const void*)trim_scc_kernel, dim3(grid), dim3(kSccThreads), args,
                                  0, c->stream));

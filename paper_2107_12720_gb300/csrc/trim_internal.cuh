@@ -234,7 +234,8 @@ struct Dev {
 // SCC decomposition (trim_scc.cu): control block, zero before every run but for
 // `least`, and arguments
 struct SccSlot {
-  unsigned int n, heavy, hits, pad;  // a phase's counts (see scc_sync)
+  unsigned int n, hits;      // a phase's counts (see scc_sync)
+  unsigned long long heavy;  // entries of the heavy list, and their pieces << 32
 };
 struct SccCtl {
   unsigned int bar;  unsigned int _p0[31];  // grid-barrier arrivals
@@ -259,7 +260,8 @@ struct SccArgs {
   uint32_t* fb;
   uint32_t* open0;   // open vertices, two lists
   uint32_t* open1;
-  uint32_t* heavy;   // frontier vertices with long rows
+  uint32_t* heavy;   // frontier vertices with long rows ...
+  uint32_t* hpos;    // ... and the first piece of each
   SccCtl* C;
   uint64_t spin_limit_ns;
 };

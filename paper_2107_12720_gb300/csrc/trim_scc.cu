@@ -24,9 +24,9 @@
 //
 // A level of a search is bound by latency when it is small (a grid barrier, not
 // a launch and a host round trip, ends it) and by random accesses when it is
-// large; rows are spread over the warps 32 vertices at a time laid end to end,
-// and rows over kSccHeavy edges over the whole grid (one warp on a hub's row
-// was what a level waited for).
+// large; rows are spread over the warps up to 32 vertices at a time laid end to end,
+// and rows over kSccHeavy edges, cut into pieces and those laid end to end, over the
+// whole grid (one warp on a hub's row was what a level waited for).
 //
 // Measured (ms, in+out trimming included; before: one launch and one host read
 // per level and pass, a warp per row, searches from every vertex in every step):
@@ -81,7 +81,8 @@ __device__ bool scc_sync(const SccArgs& A, Scc& S) {
     S.phase += 1u;
     if (blockIdx.x == 0) {
       SccSlot* z = &A.C->slot[(S.phase + 2u) & 3u];
-      z->n = z->heavy = z->hits = 0u;
+      z->n = z->hits = 0u;
+      z->heavy = 0ull;
     }
   }
   __syncthreads();
@@ -92,6 +93,13 @@ __device__ __forceinline__ SccSlot* now(const SccArgs& A, const Scc& S) {
 }
 __device__ __forceinline__ const SccSlot* before(const SccArgs& A, const Scc& S) {
   return &A.C->slot[(S.phase - 1u) & 3u];
+}
+
+// Vertices that a warp takes at a time out of `count`: few if there are few, as it looks
+// through long rows one after the other (4 parts of 1,500 vertices with 1,300 edges each:
+// 0.98 ms with 32).
+__device__ __forceinline__ uint32_t group(uint32_t count) {
+  return min(32u, max(1u, (count + nwarps() - 1u) / nwarps()));
 }
 
 // Appends to a global list, staged in the warp's buffer: one atomic per flush.
@@ -128,22 +136,33 @@ __device__ __forceinline__ void add(unsigned* c, unsigned x) {
 // All warps: f(u, w, valid) (warp-collective) for the edges u -> w of the rows of
 // list[0..count): a warp takes up to 32 vertices, their rows laid end to end,
 // four loads in flight per lane. Rows over kSccHeavy edges go to the heavy list
-// for heavy_edges, in the next phase.
+// for heavy_edges, in the next phase: one atomic of the warp reserves their entries
+// and their pieces, so that the entries' first pieces rise along the list.
 template <class F>
 __device__ __forceinline__ void list_edges(const SccArgs& A, const Scc& S, const uint32_t* off,
                                            const uint32_t* tgt, const uint32_t* list,
                                            uint32_t count, F f) {
   const unsigned lane = lane_id();
-  const uint32_t nw = nwarps();
-  const uint32_t G = min(32u, max(1u, (count + nw - 1u) / nw));
+  const uint32_t nw = nwarps(), G = group(count);
   for (uint32_t base = gwarp() * G; base < count; base += nw * G) {  // warp-uniform
     const bool has = lane < G && base + lane < count;
     const uint32_t u = has ? ldcg(&list[base + lane]) : 0u;
     const uint32_t s = has ? __ldg(&off[u]) : 0u;
     uint32_t d = has ? __ldg(&off[u + 1u]) - s : 0u;
-    if (d > kSccHeavy) {
-      A.heavy[atomicAdd(&now(A, S)->heavy, 1u)] = u;
-      d = 0u;
+    const bool big = d > kSccHeavy;
+    const unsigned bm = __ballot_sync(FULL, big);
+    if (bm) {
+      const uint32_t np = big ? (d - 1u) / kSccChunk + 1u : 0u, pincl = warp_incl_scan(np);
+      unsigned long long o = 0;
+      if (lane == 31)
+        o = atomicAdd(&now(A, S)->heavy, ((unsigned long long)pincl << 32) | __popc(bm));
+      o = __shfl_sync(FULL, o, 31);
+      if (big) {
+        const uint32_t at = (uint32_t)o + __popc(bm & ((1u << lane) - 1u));
+        A.heavy[at] = u;
+        A.hpos[at] = (uint32_t)(o >> 32) + pincl - np;
+        d = 0u;
+      }
     }
     const uint32_t incl = warp_incl_scan(d), excl = incl - d;
     const uint32_t total = __shfl_sync(FULL, incl, 31);
@@ -162,20 +181,48 @@ __device__ __forceinline__ void list_edges(const SccArgs& A, const Scc& S, const
     }
   }
 }
+// The rows of the heavy list (`heavy`: its entries, and its pieces << 32), their
+// pieces laid end to end: every warp takes an equal run of them, and finds the row
+// of its first one by a search over the entries' first pieces, 32 ways a step.
+// (20 parts of 2,000 vertices with 1,500 edges each, joined by single edges: 697 ms
+// with the rows one after the other, each from the first warp on; a warp per row and
+// launch per level, before that, 42 ms.)
 template <class F>
 __device__ __forceinline__ void heavy_edges(const SccArgs& A, const uint32_t* off,
-                                            const uint32_t* tgt, uint32_t nheavy, F f) {
+                                            const uint32_t* tgt, unsigned long long heavy, F f) {
   const unsigned lane = lane_id();
-  for (uint32_t h = 0; h < nheavy; ++h) {
-    const uint32_t u = ldcg(&A.heavy[h]);
+  const uint32_t rows = (uint32_t)heavy, pieces = (uint32_t)(heavy >> 32), nw = nwarps();
+  const uint32_t per = (pieces + nw - 1u) / nw;
+  // (neighbouring runs on different SMs)
+  uint32_t p = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per;
+  const uint32_t p1 = min(pieces, p + per);
+  if (p >= p1) return;  // warp-uniform
+  uint32_t h = 0;
+  for (uint32_t len = rows; len > 1u;) {
+    const uint32_t step = (len + 31u) / 32u, r = lane * step;
+    const unsigned b = __ballot_sync(FULL, r < len && ldcg(&A.hpos[h + r]) <= p);
+    const uint32_t skip = (31u - __clz(b)) * step;  // (b has lane 0)
+    h += skip;
+    len = min(step, len - skip);
+  }
+  for (; p < p1; ++h) {  // warp-uniform
+    const uint32_t u = ldcg(&A.heavy[h]), first = ldcg(&A.hpos[h]);
     const uint32_t s = __ldg(&off[u]), e = __ldg(&off[u + 1u]);
-    for (uint64_t k0 = (uint64_t)s + (uint64_t)gwarp() * kSccChunk; k0 < e;
-         k0 += (uint64_t)nwarps() * kSccChunk)  // warp-uniform
+    const uint32_t end = min(p1, first + (e - s - 1u) / kSccChunk + 1u);
+    for (; p < end; ++p) {
+      const uint64_t k0 = s + (uint64_t)(p - first) * kSccChunk;
 #pragma unroll
-      for (uint32_t i = 0; i < kSccChunk; i += 32u) {
-        const uint64_t k = k0 + i + lane;
-        f(u, k < e ? __ldg(&tgt[k]) : 0u, k < e);
+      for (uint32_t i = 0; i < kSccChunk; i += 128u) {
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint64_t k = k0 + i + (uint32_t)q * 32u + lane;
+          w[q] = k < e ? __ldg(&tgt[k]) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f(u, w[q], k0 + i + (uint32_t)q * 32u + lane < e);
       }
+    }
   }
 }
 
@@ -313,10 +360,12 @@ __device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint
     ++levels;
     Out o{fb, &now(A, S)->n, 0u};
     if ((uint64_t)k * 16u > left) {
-      for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+      const uint32_t G = group(n_open);
+      for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
         const uint32_t i = base + lane;
-        const uint32_t v = i < n_open ? ldcg(&open[i]) : 0u;
-        const bool want = i < n_open && ldcg(&mark[v]) < stamp &&
+        const bool in = lane < G && i < n_open;
+        const uint32_t v = in ? ldcg(&open[i]) : 0u;
+        const bool want = in && ldcg(&mark[v]) < stamp &&
                           (allow == nullptr || ldcg(&allow[v]) == allowed);
         const uint32_t s = want ? __ldg(&roff[v]) : 0u;
         const uint32_t d = want ? __ldg(&roff[v + 1u]) - s : 0u;
@@ -337,7 +386,7 @@ __device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint
       list_edges(A, S, off, tgt, fa, k, visit);
       flush(S, o);
       if (!scc_sync(A, S)) return false;
-      const uint32_t heavy = ldcg(&before(A, S)->heavy);
+      const unsigned long long heavy = __ldcg(&before(A, S)->heavy);
       k = ldcg(&before(A, S)->n);
       if (heavy) {  // (their finds join the same list, behind those of the phase before)
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&now(A, S)->n, k);
@@ -365,10 +414,12 @@ __device__ bool trim_passes(const SccArgs& A, Scc& S, const uint32_t* open, uint
   const unsigned lane = lane_id();
   for (int pass = 0; pass < 1024; ++pass) {
     unsigned gone = 0;
-    for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+    const uint32_t G = group(n_open);
+    for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
       const uint32_t i = base + lane;
-      const uint32_t v = i < n_open ? ldcg(&open[i]) : 0u;
-      const bool is = i < n_open && ldcg(&A.comp[v]) == SCC_OPEN;
+      const bool in_list = lane < G && i < n_open;
+      const uint32_t v = in_list ? ldcg(&open[i]) : 0u;
+      const bool is = in_list && ldcg(&A.comp[v]) == SCC_OPEN;
       auto hit = [&](uint32_t w) { return ldcg(&A.comp[w]) == SCC_OPEN; };
       const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
       const bool out = row_any(A.tgt, s, d, is, hit);
@@ -423,9 +474,10 @@ __global__ void __launch_bounds__(512, 2) trim_scc_kernel(SccArgs A) {
   // one; a vertex with a self-loop, which is a component of its own, is never
   // paired. `more` is true for a self-loop and for three or more open
   // successors; the second pass over G^T is for the few others.
-  for (uint32_t base = gwarp() * 32u; base < n_open; base += nwarps() * 32u) {
+  const uint32_t G = group(n_open);
+  for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
     const uint32_t i = base + lane;
-    const bool is = i < n_open;
+    const bool is = lane < G && i < n_open;
     const uint32_t v = is ? ldcg(&open[i]) : 0u;
     const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
     uint32_t oth = 0, all = 0, o1 = NONE, ioth = 0, iall = 0, i1 = NONE;
@@ -550,7 +602,7 @@ __global__ void __launch_bounds__(512, 2) trim_scc_kernel(SccArgs A) {
         list_edges(A, S, A.off, A.tgt, fa, k, offer);
         flush(S, o);
         if (!scc_sync(A, S)) return;
-        const uint32_t heavy = ldcg(&before(A, S)->heavy);
+        const unsigned long long heavy = __ldcg(&before(A, S)->heavy);
         k = ldcg(&before(A, S)->n);
         if (heavy) {
           o.count = &now(A, S)->hits;
@@ -590,7 +642,7 @@ __global__ void __launch_bounds__(512, 2) trim_scc_kernel(SccArgs A) {
         list_edges(A, S, A.ioff, A.itgt, fa, k, visit);
         flush(S, o);
         if (!scc_sync(A, S)) return;
-        const uint32_t heavy = ldcg(&before(A, S)->heavy);
+        const unsigned long long heavy = __ldcg(&before(A, S)->heavy);
         k = ldcg(&before(A, S)->n);
         if (heavy) {
           o.count = &now(A, S)->hits;
