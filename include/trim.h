@@ -307,8 +307,9 @@ trim_err_t trim_create_implicit(const trim_implicit_graph_t* g, void* cuda_strea
  * comp: n uint32, on the device if out_on_device else on the host. Needs G^T
  * (csr_in, or built on the device). Overwrites the context's level array (with
  * the in+out trimming of step 1). stats may be NULL. Device memory ~ 24 n
- * bytes is allocated on first use. Not for implicit graphs or with a dead mask
- * (TRIM_ERR_INVALID_ARG). */
+ * bytes is allocated on first use. Steps 2 and 3 end with TRIM_ERR_TIMEOUT only if for
+ * about spin_limit_ns no CTA reaches the end of its part or shows progress, however long
+ * the work takes. Not for implicit graphs or with a dead mask (TRIM_ERR_INVALID_ARG). */
 typedef struct {
   uint32_t components;       /* number of strongly connected components              */
   uint32_t trimmed_size1;    /* size-1 components removed by step 1                  */

@@ -243,6 +243,7 @@ struct SccCtl {
   unsigned long long best;                  // pivot: min(in-degree, out-degree) << 32 | ~vertex
   SccSlot slot[4];
   unsigned int done, components, size2, trimmed, steps, levels;
+  unsigned int beat;  // grows while a warp works through long rows (see scc_sync)
 };
 struct SccArgs {
   uint32_t n;

@@ -59,7 +59,20 @@ __device__ __forceinline__ uint32_t gwarp() {
 }
 __device__ __forceinline__ uint32_t nwarps() { return gridDim.x * (blockDim.x >> 5); }
 
-// Grid-wide barrier (bounded as the trimming kernel's): a phase ends. Phase p
+// A warp in a long phase shows that it goes on: one increment of the heartbeat every
+// kPace steps of its row loops (some 100 us).
+constexpr uint32_t kPace = 256;
+__device__ __forceinline__ void pace(const SccArgs& A, uint32_t& steps, uint32_t k) {
+  steps += k;
+  if (steps >= kPace) {
+    steps = 0u;
+    if (lane_id() == 0) atomicAdd(&A.C->beat, 1u);
+  }
+}
+
+// Grid-wide barrier: a phase ends. The wait is bounded by spin_limit_ns without any
+// progress (an arrival or a heartbeat): how long a phase takes depends on the graph
+// (one warp may have a row of millions of edges to itself). Phase p
 // counts into slot p & 3, which is read in phase p + 1; the slot of phase p + 2
 // was last read in phase p - 1 and is cleared by CTA 0 at the start of phase p.
 // Returns false when the run must stop.
@@ -69,11 +82,19 @@ __device__ bool scc_sync(const SccArgs& A, Scc& S) {
     const unsigned target = (++S.epoch) * gridDim.x;
     __threadfence();
     atomicAdd(&A.C->bar, 1u);
-    const uint64_t t0 = globaltimer();
+    uint64_t t0 = globaltimer();
+    bool looked = false;
+    unsigned seen = 0;
     while ((int)(ld_relaxed(&A.C->bar) - target) < 0) {
       if (globaltimer() - t0 > A.spin_limit_ns) {
-        atomicCAS(&A.C->err, 0u, (unsigned)TRIM_ERR_TIMEOUT);
-        break;
+        const unsigned cur = ld_relaxed(&A.C->bar) + ld_relaxed(&A.C->beat);  // both only grow
+        if (looked && cur == seen) {
+          atomicCAS(&A.C->err, 0u, (unsigned)TRIM_ERR_TIMEOUT);
+          break;
+        }
+        looked = true;
+        seen = cur;
+        t0 = globaltimer();
       }
     }
     (void)ld_acquire(&A.C->bar);
@@ -144,6 +165,7 @@ __device__ __forceinline__ void list_edges(const SccArgs& A, const Scc& S, const
                                            uint32_t count, F f) {
   const unsigned lane = lane_id();
   const uint32_t nw = nwarps(), G = group(count);
+  uint32_t steps = 0;
   for (uint32_t base = gwarp() * G; base < count; base += nw * G) {  // warp-uniform
     const bool has = lane < G && base + lane < count;
     const uint32_t u = has ? ldcg(&list[base + lane]) : 0u;
@@ -166,6 +188,7 @@ __device__ __forceinline__ void list_edges(const SccArgs& A, const Scc& S, const
     }
     const uint32_t incl = warp_incl_scan(d), excl = incl - d;
     const uint32_t total = __shfl_sync(FULL, incl, 31);
+    pace(A, steps, 1u + total / 128u);  // (at most 32 rows of kSccHeavy)
     for (uint32_t k0 = 0; k0 < total; k0 += 128u) {
       uint32_t uu[4], w[4];
 #pragma unroll
@@ -197,7 +220,7 @@ __device__ __forceinline__ void heavy_edges(const SccArgs& A, const uint32_t* of
   uint32_t p = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per;
   const uint32_t p1 = min(pieces, p + per);
   if (p >= p1) return;  // warp-uniform
-  uint32_t h = 0;
+  uint32_t h = 0, steps = 0;
   for (uint32_t len = rows; len > 1u;) {
     const uint32_t step = (len + 31u) / 32u, r = lane * step;
     const unsigned b = __ballot_sync(FULL, r < len && ldcg(&A.hpos[h + r]) <= p);
@@ -210,6 +233,7 @@ __device__ __forceinline__ void heavy_edges(const SccArgs& A, const uint32_t* of
     const uint32_t s = __ldg(&off[u]), e = __ldg(&off[u + 1u]);
     const uint32_t end = min(p1, first + (e - s - 1u) / kSccChunk + 1u);
     for (; p < end; ++p) {
+      pace(A, steps, kSccChunk / 128u);
       const uint64_t k0 = s + (uint64_t)(p - first) * kSccChunk;
 #pragma unroll
       for (uint32_t i = 0; i < kSccChunk; i += 128u) {
@@ -230,8 +254,8 @@ __device__ __forceinline__ void heavy_edges(const SccArgs& A, const uint32_t* of
 // for the lanes with want: four entries per lane at a time, up to 32 of a row;
 // what is left of longer rows is looked through by the whole warp.
 template <class H>
-__device__ __forceinline__ bool row_any(const uint32_t* tgt, uint32_t s, uint32_t d, bool want,
-                                        H hit) {
+__device__ __forceinline__ bool row_any(const SccArgs& A, const uint32_t* tgt, uint32_t s,
+                                        uint32_t d, bool want, uint32_t& steps, H hit) {
   const unsigned lane = lane_id();
   bool found = false;
   uint32_t i = 0;
@@ -253,6 +277,7 @@ __device__ __forceinline__ bool row_any(const uint32_t* tgt, uint32_t s, uint32_
     const uint32_t sj = __shfl_sync(FULL, s, j), dj = __shfl_sync(FULL, d, j);
     bool any = false;
     for (uint32_t k0 = 32u; k0 < dj && !any; k0 += 128u) {  // warp-uniform
+      pace(A, steps, 1u);
       uint32_t w[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -275,8 +300,8 @@ __device__ __forceinline__ bool row_any(const uint32_t* tgt, uint32_t s, uint32_
 // Open entries of the row [s, s + d) for the lanes with want: those other than
 // `self` counted up to 2 (oth, the first one in *first) and all of them up to 3.
 __device__ __forceinline__ void row_count(const SccArgs& A, const uint32_t* tgt, uint32_t s,
-                                          uint32_t d, bool want, uint32_t self, uint32_t& oth,
-                                          uint32_t& all, uint32_t& first) {
+                                          uint32_t d, bool want, uint32_t self, uint32_t& steps,
+                                          uint32_t& oth, uint32_t& all, uint32_t& first) {
   const unsigned lane = lane_id();
   oth = all = 0u;
   first = NONE;
@@ -306,6 +331,7 @@ __device__ __forceinline__ void row_count(const SccArgs& A, const uint32_t* tgt,
     const uint32_t vj = __shfl_sync(FULL, self, j);
     uint32_t o = 0, a = 0, f = NONE;
     for (uint32_t k0 = 0; k0 < dj && (o < 2u || a < 3u); k0 += 32u) {  // warp-uniform
+      pace(A, steps, 1u);
       const uint32_t k = k0 + lane;
       const uint32_t w = k < dj ? __ldg(&tgt[sj + k]) : 0u;
       const bool open = k < dj && ldcg(&A.comp[w]) == SCC_OPEN;
@@ -361,6 +387,7 @@ __device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint
     Out o{fb, &now(A, S)->n, 0u};
     if ((uint64_t)k * 16u > left) {
       const uint32_t G = group(n_open);
+      uint32_t steps = 0;
       for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
         const uint32_t i = base + lane;
         const bool in = lane < G && i < n_open;
@@ -369,7 +396,8 @@ __device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint
                           (allow == nullptr || ldcg(&allow[v]) == allowed);
         const uint32_t s = want ? __ldg(&roff[v]) : 0u;
         const uint32_t d = want ? __ldg(&roff[v + 1u]) - s : 0u;
-        const bool hit = row_any(rtgt, s, d, want, [&](uint32_t w) { return ldcg(&mark[w]) == stamp; });
+        pace(A, steps, 1u);
+        const bool hit = row_any(A, rtgt, s, d, want, steps, [&](uint32_t w) { return ldcg(&mark[w]) == stamp; });
         if (hit) mark[v] = stamp;
         put(S, o, hit, v);
       }
@@ -415,6 +443,7 @@ __device__ bool trim_passes(const SccArgs& A, Scc& S, const uint32_t* open, uint
   for (int pass = 0; pass < 1024; ++pass) {
     unsigned gone = 0;
     const uint32_t G = group(n_open);
+    uint32_t steps = 0;
     for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
       const uint32_t i = base + lane;
       const bool in_list = lane < G && i < n_open;
@@ -422,9 +451,10 @@ __device__ bool trim_passes(const SccArgs& A, Scc& S, const uint32_t* open, uint
       const bool is = in_list && ldcg(&A.comp[v]) == SCC_OPEN;
       auto hit = [&](uint32_t w) { return ldcg(&A.comp[w]) == SCC_OPEN; };
       const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
-      const bool out = row_any(A.tgt, s, d, is, hit);
+      pace(A, steps, 1u);
+      const bool out = row_any(A, A.tgt, s, d, is, steps, hit);
       const uint32_t t = out ? __ldg(&A.ioff[v]) : 0u, e = out ? __ldg(&A.ioff[v + 1u]) - t : 0u;
-      const bool in = row_any(A.itgt, t, e, out, hit);
+      const bool in = row_any(A, A.itgt, t, e, out, steps, hit);
       if (is && !in) {
         close_vertex(A, v, v);
         ++gone;
@@ -475,17 +505,19 @@ __global__ void __launch_bounds__(512, 2) trim_scc_kernel(SccArgs A) {
   // paired. `more` is true for a self-loop and for three or more open
   // successors; the second pass over G^T is for the few others.
   const uint32_t G = group(n_open);
+  uint32_t steps2 = 0;
   for (uint32_t base = gwarp() * G; base < n_open; base += nwarps() * G) {
     const uint32_t i = base + lane;
     const bool is = lane < G && i < n_open;
     const uint32_t v = is ? ldcg(&open[i]) : 0u;
     const uint32_t s = is ? __ldg(&A.off[v]) : 0u, d = is ? __ldg(&A.off[v + 1u]) - s : 0u;
     uint32_t oth = 0, all = 0, o1 = NONE, ioth = 0, iall = 0, i1 = NONE;
-    row_count(A, A.tgt, s, d, is, v, oth, all, o1);
+    pace(A, steps2, 1u);
+    row_count(A, A.tgt, s, d, is, v, steps2, oth, all, o1);
     const bool more = all > oth;
     const bool back = is && !more;
     const uint32_t t = back ? __ldg(&A.ioff[v]) : 0u, e = back ? __ldg(&A.ioff[v + 1u]) - t : 0u;
-    row_count(A, A.itgt, t, e, back, v, ioth, iall, i1);
+    row_count(A, A.itgt, t, e, back, v, steps2, ioth, iall, i1);
     if (is) {
       A.fa[v] = (!more && oth == 1u) ? o1 : NONE;
       A.fb[v] = (!more && ioth == 1u) ? i1 : NONE;

@@ -49,3 +49,25 @@ def test_thousands_of_rows_share_the_grid():
         t.set_params(spin_limit_ns=10_000_000)
         st = check_scc(t, g, "12,000 long rows")
         assert st["components"] == 8 and st["fwbw_steps"] > 1
+
+
+def test_a_long_phase_is_not_a_timeout():
+    """A vertex with four million removed successors and one open one, the other half of its
+    size-2 component: one warp reads that row for some 100 ms, far longer than the limit of a
+    wait without progress (the in+out trimming before it takes about 5 ms)."""
+    import paper_2107_12720_gb300 as P
+    k = 1 << 22
+    off = np.zeros(k + 3, np.uint32)
+    off[k + 1] = k + 1
+    off[k + 2] = k + 2
+    tgt = np.concatenate([np.arange(k), [k + 1, k]]).astype(np.uint32)
+    with P.Trimmer(off, tgt) as t:
+        t.in_csr()
+        assert t.run_inout()["device_ms"] < 15
+        t.set_params(spin_limit_ns=30_000_000)
+        comp, st = t.run_scc()
+        assert st["ms"] > 60  # the phase is longer than the limit
+        want = np.arange(k + 2, dtype=np.uint32)
+        want[k + 1] = k
+        assert np.array_equal(comp, want)
+        assert st["components"] == k + 1 and st["trimmed_size2"] == 1
