@@ -154,7 +154,7 @@ struct Cta {
   unsigned w4_wide;   // initial pass: the work-list slices take all four buffers
   unsigned lq_scratch;  // initial pass with a dead mask: deferred heavy rows
   unsigned long long kstat[4];  // TRIM_FLAG_STATS totals of this CTA (see stats_flush)
-  uint32_t wbuf[MAX_WARPS][WBUF];
+  uint32_t wbuf[(TRIM_MODES & 2) && !TRIM_AC6_ONLY ? MAX_WARPS : 1][WBUF];  // (AC-6 in schedules)
 #if TRIM_LOCAL
 #if TRIM_AC3_ONLY
   uint32_t live_n[2];  // local AC-3 rounds: the CTA's live list, by local-round parity
@@ -212,6 +212,15 @@ struct Cta {
 // 2^24 (2,868 levels) 6,700 and 6,555, 4,096 packed graphs 2,056 and 2,041.
 __shared__ Cta cta_state;
 __shared__ Dev cta_dev;
+// What the two CTAs of an SM take of its 256 KB decides how much is left as L1: with 512
+// threads (64 KB of append slices each) and some 200 bytes of scratch they stay within a
+// carve-out of 164 KB. Past it the next size is 196 KB, and rounds that push millions of
+// edges have a third less L1: in+out of R-MAT 2^23, round 1 in us, 211 with 20 KB of state
+// per CTA and 167 with 9 KB.
+#if TRIM_LOCAL
+static_assert(sizeof(Cta) + sizeof(Dev) + 256 + 1024 + 65536 <= (164 << 10) / 2,
+              "the CTA's state pushes the shared memory past the 164 KB carve-out");
+#endif
 
 // Are scheduler features gathered in round S.round? The learned scheduler (and
 // a round log of a scheduled run) reads them after every round in which it is
