@@ -128,7 +128,7 @@ struct WarpSlice {
 #if TRIM_LOCAL
 constexpr uint32_t LQ_EDGES = 1024;   // predecessors queued per CTA per round
 constexpr uint32_t LQ_ENTRIES = 256;  // removed vertices queued per CTA per round
-constexpr uint32_t LQ_FLOOR = 256;     // least bound of a stretch's queues
+constexpr uint32_t LQ_FLOOR = 512;     // least bound of a stretch's queues
 constexpr uint32_t LQ_SKEW = 4;        // ... and the bound as a multiple of the mean load
 constexpr uint32_t LQ_LATE_MIN = 1u << 14;  // from here on offsets are loaded for removals only
 constexpr uint32_t LQ_DMAX = 64;      // larger in-degrees always go to the global work list
@@ -1480,7 +1480,11 @@ __device__ __noinline__ bool local_stretch() {
   // with queues filled to LQ_EDGES: in+out of 2^23 vertices 6.73 and 7.52, of 2^20
   // 1.354 and 1.510; AC-4 of 2^24 (rounds only) 12.4 and 13.2, of 2^20 1.205 and
   // 1.283; 256 packed graphs 0.616 and 0.601. Multiples of 2 to 6 on an in+out
-  // cascade of 5,000,011: 4.61, 4.45, 4.54, 4.68, 4.85 (2: packed graphs 0.84).
+  // cascade of 5,000,011: 4.61, 4.45, 4.54, 4.68, 4.85 (2: packed graphs 0.84). Where few
+  // edges are pending a full queue is cheaper than leaving, so the bound has a floor:
+  // kernel us with 256 / 512 / 768 / 1,024, packed graphs, 64 402 / 350 / 348 / 356, 80 462 / 405 /
+  // 396 / 400, 256 570 / 556 / 552 / 552; in+out of 2^20 1,055 / 1,049 / 1,145 / 1,202, of
+  // 5,000,011 4,218 / 4,218 / 4,575 / 4,835.
   const float mean = __fdividef((float)(B.S.e_end - B.S.e_c4), (float)gridDim.x);
   const uint32_t cap = min(LQ_EDGES, max(LQ_FLOOR, (uint32_t)((float)LQ_SKEW * mean)));
   const bool late = D.n > LQ_LATE_MIN;
