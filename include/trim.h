@@ -118,15 +118,18 @@ typedef struct {
                                  with TRIM_ERR_TIMEOUT                                       */
   float heur_push_ratio;      /* heuristic: push while sum(indeg F) < ratio * n_live        */
   float heur_ac6_ratio;       /* heuristic (no G^T): AC-6 while |F| < ratio * n_live        */
-  uint32_t local_round_edges; /* AC-4, AC-6 and in+out kernels: once the edges still to push fit a
-                                 small round (at most this many, one work-list entry per
-                                 warp), rounds run CTA-locally: each CTA queues the vertices
-                                 it removes in shared memory and pushes them itself in the
-                                 next round (AC-6: re-scans their sets; at most one to a warp
-                                 to start with; AC-3 alone: every round, each CTA on a live
-                                 list of its own vertices), and a round ends at one
-                                 barrier that carries its totals; a round whose removals overflow the queues
-                                 returns to ordinary rounds (0 = never local)            */
+  uint32_t local_round_edges; /* rounds that run CTA-locally, each ended by one barrier that
+                                 carries its totals instead of shared lists (0 = never):
+                                 AC-4, in+out: from a round with at most this many edges to
+                                   push on (in+out: and at most two removed vertices to a
+                                   warp), each CTA queues the vertices it removes in shared
+                                   memory and pushes them itself in the next round; a round
+                                   whose removals overflow the queues returns to ordinary
+                                   rounds
+                                 AC-6: from a round with at most this many removed vertices,
+                                   and at most one to a warp, on
+                                 AC-3: every round, each CTA on a live list of its own
+                                   vertices, whatever the value                          */
   float sched_commit_confidence; /* LEARNED: a choice whose softmax probability (among the
                                  variants the run can use) is at least this commits the
                                  run at once, as sched_commit_rounds unchanged choices do

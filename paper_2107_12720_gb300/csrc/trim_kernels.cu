@@ -1304,6 +1304,11 @@ __device__ __forceinline__ bool local_start(const Dev& D, const Sched& S) {
   // with the schedulers: inside a committed stretch only, whose last round
   // (the one the scheduler reads features of) runs as an ordinary round
   if ((MODES & M_SCHED) && !(S.cstop != 0u && S.round + 1u < S.cstop)) return false;
+  // In+out trimming takes one entry to a warp in a stretch's first round, so it starts one
+  // with at most two each; wider rounds are better spread by inout_round (kernel us with any
+  // number / with this bound: R-MAT of 2^22 vertices 149 and 145, of 2^23 269 and 258, 80
+  // packed graphs 289 and 278, planted 4,000,000 362 and 349; deep cascades the same).
+  if ((MODES & M_INOUT) && S.w_end - S.c4w > 2u * gridDim.x * (blockDim.x >> 5)) return false;
   const uint32_t edges = S.e_end - S.e_c4;
   return edges <= D.local_edges_max && S.bmax <= 256u;
 #endif
@@ -1500,7 +1505,7 @@ __device__ __noinline__ bool local_stretch() {
       // G entries to a warp (one where there are enough warps), their edges end to
       // end: a stretch may begin with many more entries than warps. 4,096 packed
       // graphs, kernel us: 1,990 against 2,041 with one entry after the other.
-      // (In+out keeps one: a stretch begins about every 30 rounds there.)
+      // (In+out keeps one: it starts with at most two entries to a warp.)
       constexpr bool kOne = (MODES & M_INOUT) != 0;
       const uint32_t G = kOne ? 1u : min(32u, (ib - ia + nw - 1u) / nw);
       auto of = [&](uint32_t x, unsigned o) { return kOne ? x : __shfl_sync(FULL, x, o); };
