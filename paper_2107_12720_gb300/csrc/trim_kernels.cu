@@ -3487,17 +3487,21 @@ __device__ __forceinline__ uint32_t lane_range(uint32_t a, uint32_t b) {  // bit
 }
 
 constexpr uint32_t kMaskHeavy = 512;
-constexpr uint32_t kMaskGiant = 4096;
+constexpr uint32_t kMaskGiant = 2048;
 constexpr uint32_t kMaskHeavyCap = LW - MAX_WARPS;  // list + per-warp sums in one slice
+constexpr uint32_t kMaskOnce = 1u << 21;  // from here on targets pass by the L1
 
 // The mask comes as one bit per vertex: the pass is bound by the look-ups of the
 // targets' marks (random accesses), and the bits of the targets that skewed graphs
-// keep asking for stay in the L1, which the streamed targets pass by. R-MAT of
-// 3,000,017 vertices, half of them masked, 21 million look-ups, initial pass in us: 213
-// with a byte per vertex, one 32-vertex block after the other and heavy rows (over
-// 1,024) by the CTA; 191 with bits, 178 with heavy rows by warps, 159 with the next block's loads
-// (and its G^T rows) ahead. Bounds of 128 / 256 / 512 for the heavy rows: 217, 207, 178;
-// of 2,048 / 4,096 / 8,192 / 16,384 for the giant ones (at 256): 201, 207, 205, 242.
+// keep asking for stay in the L1, which the streamed targets pass by where the bits fill
+// it (from kMaskOnce vertices on; below, the targets' next sectors are worth keeping).
+// There, blocks of 32 vertices go to the CTAs in turn, so that a small graph of long rows
+// has all SMs at work. Kernel us, a byte per vertex and rows over 1,024 by the CTA / bits,
+// always passing by and blocks next to each other / as here: R-MAT of 3,000,017 vertices,
+// half of them masked, 264 / 194 / 186, 1,000,000 118 / 82 / 79, 1,000,000 vertices with 16
+// random successors 50 / 55 / 44, 20,000 with 800 161 / 235 / 34.
+// kMaskHeavy of 256 / 512 / 1,024: R-MAT of 3,000,017 201 / 191 / 191, 20,000 with 800 34 / 34 / 149;
+// kMaskGiant of 2,048 / 4,096 / 16,384: R-MAT 186 / 191 / 223, 5,000 vertices with 3,000 33 / 41 / 41.
 __device__ __forceinline__ bool is_masked(const Dev& D, uint32_t v) {
   return __ldg(&D.mask[v >> 5]) >> (v & 31u) & 1u;
 }
@@ -3507,10 +3511,13 @@ __device__ __forceinline__ uint32_t ld_once(const uint32_t* p) {
   return v;
 }
 
-__device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
-                                           uint32_t nwarps) {
+__device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B) {
   const unsigned lane = lane_id();
   const uint32_t n = D.n;
+  const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+  const bool once = n >= kMaskOnce;
+  const uint32_t gwarp = once ? blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)
+                              : (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const bool w4 = (D.flags & F_AC4_POSSIBLE) != 0;
   // the CTA's deferred heavy rows and its reduction scratch: warp 0's live-list
   // slice, which no append of this pass uses (its work-list slices stay in
@@ -3551,13 +3558,22 @@ __device__ ROUND_FN void init_round_masked(const Dev& D, Cta& B, uint32_t gwarp,
       const uint32_t incl = warp_incl_scan(dd), excl = incl - dd;
       const uint32_t total = __shfl_sync(FULL, incl, 31);
       for (uint32_t k0 = 0; k0 < total; k0 += 128u) {  // warp-uniform
-        uint32_t t[4];
+        uint32_t at[4], t[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t k = k0 + (uint32_t)q * 32u + lane;
           const unsigned o = owner_of(excl, k);
           const uint32_t so = __shfl_sync(FULL, s, o), xo = __shfl_sync(FULL, excl, o);
-          t[q] = k < total ? ld_once(&D.tgt[so + (k - xo)]) : 0u;
+          at[q] = so + (k - xo);
+        }
+        if (once) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            t[q] = k0 + (uint32_t)q * 32u + lane < total ? ld_once(&D.tgt[at[q]]) : 0u;
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            t[q] = k0 + (uint32_t)q * 32u + lane < total ? __ldg(&D.tgt[at[q]]) : 0u;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -3762,7 +3778,7 @@ __global__ void __launch_bounds__(512, TRIM_MIN_BLOCKS) TRIM_KERNEL(const __grid
     if (threadIdx.x == 0) B.w4_wide = ((MODES & M_INOUT) || D.mask != nullptr) ? 0u : 1u;
     __syncthreads();
 #if !(TRIM_MODES & 48)
-    if (D.mask != nullptr) init_round_masked(D, B, gwarp, nwarps);
+    if (D.mask != nullptr) init_round_masked(D, B);
     else
 #endif
       init_round(D, B, gwarp, nwarps);
