@@ -2632,8 +2632,8 @@ __device__ ROUND_FN void ac3_round(const Dev& D, Cta& B, const Sched& S, uint32_
 
 #if TRIM_LOCAL && TRIM_AC3_ONLY
 // A run of AC-3 alone, from round 1 to the end: each CTA sweeps its own vertices
-// (every nwarps-th block of 32 per warp) and keeps its survivors in its own part of
-// the live lists, in the part's order of blocks. A round needs no shared list, no space
+// (every block of 32 in turn, so that the vertices of a level, often neighbours, are
+// spread over the CTAs) and keeps its survivors in its own part of the live lists. A round needs no shared list, no space
 // reservation, no dead log and no read of the control block; it ends at a fenced
 // local barrier that carries the removals. A list entry has all that a sweep needs:
 // the vertex, its support, the support's position and the row's end; while the
@@ -2649,12 +2649,12 @@ __device__ __noinline__ bool local_stretch() {
   const Dev& D = cta_dev;
   Cta& B = cta_state;
   Counters K;
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  const uint32_t n = D.n, blocks = (n + 31u) / 32u, nwarps = gridDim.x * wpb;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint32_t n = D.n, blocks = (n + 31u) / 32u;
   // first entry of the CTA's part, and its blocks
-  const uint32_t turns = blocks / nwarps, left = blocks % nwarps;
-  const uint32_t part = 32u * (turns * wpb * blockIdx.x + min(left, blockIdx.x * wpb));
-  const uint32_t own = turns * wpb + min(wpb, left - min(left, blockIdx.x * wpb));
+  const uint32_t turns = blocks / gridDim.x, left = blocks % gridDim.x;
+  const uint32_t part = 32u * (turns * blockIdx.x + min(left, blockIdx.x));
+  const uint32_t own = turns + (blockIdx.x < left ? 1u : 0u);
   bool first = true;
   while (true) {
     const uint32_t r = B.S.round;
@@ -2667,9 +2667,8 @@ __device__ __noinline__ bool local_stretch() {
       const uint32_t k = base + lane;
       bool alive = k < N, stays = false;
       uint4 x = make_uint4(0u, 0u, 0u, 0u);
-      if (first) {  // block q of the CTA is its warp q % wpb's, in turn q / wpb
-        const uint32_t q = base / 32u;
-        x.x = 32u * ((q / wpb) * nwarps + blockIdx.x * wpb + q % wpb) + lane;
+      if (first) {
+        x.x = 32u * (base / 32u * gridDim.x + blockIdx.x) + lane;
         alive = x.x < n;
         K.swept += alive ? 1 : 0;
         alive = alive && ldcg(&D.level[x.x]) == LIVE;
