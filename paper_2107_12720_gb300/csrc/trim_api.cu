@@ -62,6 +62,7 @@ struct trim_ctx {
   uint32_t* mask_bits = nullptr;  // ... and the same as one bit per vertex
   bool has_mask = false;
   bool implicit = false;      // trim_create_implicit: successors computed, no CSR
+  bool rows_far = false;      // csr_out is TRIM_MEM_HOST_MAPPED
   trim_implicit_graph_t ig{};
   // trim_run_scc: component labels, propagated labels, search marks, two
   // frontiers (one allocation), control block, launch size (made on first use)
@@ -647,6 +648,7 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   } else if (g->on_device == TRIM_MEM_HOST_MAPPED) {
     TRY(map_host(c, g->offsets, &c->off));
     TRY(map_host(c, c->m ? g->targets : nullptr, &c->tgt));
+    c->rows_far = true;
   } else {
     c->off = g->offsets;
     c->tgt = g->targets;
@@ -825,6 +827,7 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   if (ac4) { f |= trimk::F_AC4_POSSIBLE; TRY(ensure_work_list(c)); }
   if (ac6) f |= trimk::F_AC6_POSSIBLE;
   if (ac3) f |= trimk::F_AC3_POSSIBLE;
+  if (c->rows_far) f |= trimk::F_ROWS_FAR;
   c->cont_mode = -1;
   c->sched_mode = (variant >= TRIM_SCHED_HEURISTIC) ? (int)variant : -1;
   c->last_launches = 0;

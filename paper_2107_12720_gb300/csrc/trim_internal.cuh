@@ -42,6 +42,7 @@ constexpr uint32_t F_AC6_POSSIBLE = 0x400;
 constexpr uint32_t F_AC3_POSSIBLE = 0x800;
 constexpr uint32_t F_LIVE_EDGES = 0x1000;    // scheduled run: keep the live-edge count in every flavour
 constexpr uint32_t F_CONTINUE = 0x2000;      // continuation launch: resume the run if a segment handed it over
+constexpr uint32_t F_ROWS_FAR = 0x4000;      // the out-CSR is host memory read in place
 
 // Per-round accumulators, filled while round r runs (ring slot r & 3). CTA 0
 // zeroes slot (k+2) & 3 at the start of round k: that slot was last read at the

@@ -2797,6 +2797,15 @@ __device__ unsigned block_sum(unsigned x) {
 // scatter needs no atomics. The table lies in append slices that AC-6 does not use:
 // keys, counts, and the CTA's first rank of each support.
 constexpr uint32_t AC6_HEADS = 4;
+// Rows in host memory come over the link, entry by entry as they are needed: a record then
+// holds UNREAD instead of the next successor (ids are below 2^31), and row bounds are
+// read once. AC-6 of R-MAT of 2^22 vertices read in place, call us: 785 with the next
+// successors read ahead, 608 without, 574 with the bounds
+// read once as well (581 before the records).
+constexpr uint32_t UNREAD = 0xFFFFFFFEu;
+__device__ __forceinline__ bool rows_far(const Dev& D) {
+  return !(MODES & M_IMPLICIT) && (D.flags & F_ROWS_FAR) != 0u;
+}
 __device__ __forceinline__ uint32_t* set_head(const Dev& D, uint32_t w, uint32_t q) {
   return reinterpret_cast<uint32_t*>(&D.s_heads[w]) + q;
 }
@@ -2819,6 +2828,7 @@ __device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, u
   Counters K;
   const unsigned lane = lane_id();
   const uint32_t n = D.n;
+  const bool far = rows_far(D);
   for (uint32_t e = threadIdx.x; e < sort_slots(); e += blockDim.x) {
     *sort_word(e, 1) = NIL;
     *sort_word(e, 2) = 0u;
@@ -2862,7 +2872,7 @@ __device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, u
         if (alive[q]) row_bounds(D, v, s[q], d[q]);
 #endif
         t[q] = alive[q] ? row_target(D, v, s[q], 0u) : 0u;
-        after[q] = alive[q] && d[q] > 1u ? row_target(D, v, s[q], 1u) : NIL;
+        after[q] = !(alive[q] && d[q] > 1u) ? NIL : far ? UNREAD : row_target(D, v, s[q], 1u);
       }
 #pragma unroll
       for (int q = 0; q < U; ++q) {
@@ -2874,6 +2884,7 @@ __device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, u
         const bool slow = alive[q] && x[q] < r;
         const unsigned mask = __ballot_sync(FULL, slow);
         if (slow) list[nl + __popc(mask & ((1u << lane) - 1u))] = base + q * 32u + lane;
+        if (slow && far) D.s_rec[base + q * 32u + lane] = make_uint4(s[q], d[q], 0u, 0u);
         nl += __popc(mask);
         alive[q] = alive[q] && !slow;
         x[q] = alive[q] ? count(t[q]) : 0u;
@@ -2892,15 +2903,20 @@ __device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, u
       nl -= take;
       uint32_t s = 0, d = 0, i = 0;
       bool resolved = true;
-      if (has) {
+      if (has && far) {  // (its bounds, not to read them again)
+        const uint4 x = __ldcg(&D.s_rec[v]);
+        s = x.x;
+        d = x.y;
+      } else if (has) {
         row_bounds(D, v, s, d);
-        i = scan_thread(D, v, s, d, 1u, r, 2, resolved, K);
       }
+      if (has) i = scan_thread(D, v, s, d, 1u, r, 2, resolved, K);
       scan_warp_finish(D, resolved, v, s, d, i, r, K);
       const bool found = has && i < d;
       if (found) {
         const uint32_t t = row_target(D, v, s, i);
-        store(v, t, count(t), i + 1u < d ? row_target(D, v, s, i + 1u) : NIL, s + i + 1u, s + d);
+        store(v, t, count(t), i + 1u >= d ? NIL : far ? UNREAD : row_target(D, v, s, i + 1u),
+              s + i + 1u, s + d);
       } else if (has) {
         D.s_heads[v] = make_uint4(NIL, NIL, NIL, NIL);
       }
@@ -3112,6 +3128,8 @@ __device__ __forceinline__ void log_removed(const Dev& D, unsigned mask, uint32_
 template <bool LOCAL>
 __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uint32_t v, uint32_t t,
                                            uint32_t pos, uint32_t end, uint32_t r, Counters& K) {
+  const bool far = rows_far(D);
+  if (valid && t == UNREAD) t = row_target(D, v, 0u, pos);
   const bool cand = valid && t != NIL;
   // members without a successor left die: their log space is asked for first
   const unsigned now = __ballot_sync(FULL, valid && !cand);
@@ -3119,7 +3137,7 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
   uint32_t lv = 0, after = NIL;
   if (cand) {
     lv = ldcg(&D.level[t]);
-    if (pos + 1u < end) after = row_target(D, v, 0u, pos + 1u);
+    if (pos + 1u < end) after = far ? UNREAD : row_target(D, v, 0u, pos + 1u);
     K.edges += 1;
   }
   bool found = cand && lv >= r;
@@ -3128,14 +3146,14 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
     uint32_t i = pos + 1u;
     bool resolved = !(cand && !found);
     // one or two rows: the whole warp scans each, 32 successors in one step; more of
-    // them: each lane its own first, four successors in a step
-    if (__popc(scan) > 2 && !resolved) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
+    // them (and rows read over the link): each lane its own first, four successors in a step
+    if ((far || __popc(scan) > 2) && !resolved) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
     scan_warp_finish(D, resolved, v, 0u, end, i, r, K);
     if (cand && !found && i < end) {
       found = true;
       pos = i;
       t = row_target(D, v, 0u, i);
-      after = i + 1u < end ? row_target(D, v, 0u, i + 1u) : NIL;
+      after = i + 1u >= end ? NIL : far ? UNREAD : row_target(D, v, 0u, i + 1u);
     }
   }
   if (found) {
