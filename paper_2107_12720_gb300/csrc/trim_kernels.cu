@@ -77,10 +77,12 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int MAX_WARPS = 16;   // blockDim.x <= 512
 constexpr int WBUF = 64;        // per-warp staging of supporting-set members
 
-// Work counters (TRIM_FLAG_STATS). Each round function keeps its own in
-// registers and adds them to the global totals when it returns.
+// Work counters (TRIM_FLAG_STATS). Each round function keeps its own in registers and
+// adds a warp's to the CTA's 64-bit totals (stats_flush) before they can pass 2^32: at its
+// end where an edge or a vertex counts once, after every round where each round counts
+// them again (AC-3).
 struct Counters {
-  unsigned edges = 0, pushed = 0, cand = 0, swept = 0;  // one round: each at most m < 2^32
+  unsigned edges = 0, pushed = 0, cand = 0, swept = 0;
 };
 
 // Per-warp append slices. Each warp buffers what it removes (and, in AC-3
@@ -791,7 +793,7 @@ __device__ bool grid_barrier(const Dev& D, Cta& B, bool read_err = true) {
 // atomics per warp and round.
 __device__ __forceinline__ void stats_flush(const Dev& D, Cta& B, const Counters& K) {
   if (!(D.flags & F_STATS)) return;
-  // a round's counts of a whole warp are counts of distinct edges or vertices
+  // (a warp's counts since the last call: below 2^32, see Counters)
   const unsigned e = __reduce_add_sync(FULL, K.edges), p = __reduce_add_sync(FULL, K.pushed),
                  c = __reduce_add_sync(FULL, K.cand), s = __reduce_add_sync(FULL, K.swept);
   if (lane_id() == 0) {
@@ -2712,11 +2714,12 @@ __device__ __noinline__ bool local_stretch() {
       __syncthreads();
       if (threadIdx.x == 0) D.C->t_work[r & 3] = globaltimer();
     }
+    stats_flush(D, B, K);
+    K = Counters();
     if (!local_barrier(D, B, b, r)) break;
     if (B.lq_next != LQ_GO) break;  // done (a round cannot overflow)
     first = false;
   }
-  stats_flush(D, B, K);
   return B.err == 0u;
 }
 #endif
