@@ -222,8 +222,9 @@ typedef struct trim_ctx trim_ctx;
  * when TRIM_FLAG_VALIDATE is set); without it the AC-4 variant builds G^T on the
  * device on first use (a counting sort; its time is not part of trim_run).
  * cuda_stream: a cudaStream_t (NULL = the legacy default stream).
- * On success *out receives the context. Allocates device memory ~ (40 n + 4 m) B,
- * plus ~ (12 n + m / 21) B + 96 B per resident GPU thread for the asynchronous
+ * On success *out receives the context. Allocates device memory ~ (56 n + m / 8) B,
+ * 4 (n + m) B more for each CSR that is copied from host memory and for G^T built here,
+ * and ~ (12 n + m / 21) B + 96 B per resident GPU thread for the asynchronous
  * AC-4 tail once G^T exists (given here, or built on first use). */
 trim_err_t trim_create(const trim_csr_t* csr_out, const trim_csr_t* csr_in, void* cuda_stream,
                        uint32_t flags, trim_ctx** out);

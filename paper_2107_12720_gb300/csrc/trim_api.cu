@@ -39,7 +39,7 @@ struct trim_ctx {
   uint64_t allocated = 0;
   uint32_t *level = nullptr, *cnt = nullptr, *supp = nullptr, *s_head = nullptr,
            *s_next = nullptr, *s_cnt = nullptr, *s_off = nullptr, *s_list = nullptr,
-           *log = nullptr, *roff = nullptr, *live0 = nullptr, *live1 = nullptr, *bsum = nullptr;
+           *log = nullptr, *s_rank = nullptr, *live0 = nullptr, *live1 = nullptr, *bsum = nullptr;
   uint32_t *w4_row = nullptr, *w4_eoff = nullptr, *chunk_first = nullptr;
   // asynchronous AC-4 tail: per-vertex records (over supp, s_head, s_next and
   // s_list), the global list of G^T row pieces and the two pairs of rebalance
@@ -630,7 +630,7 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   const size_t a_snext = A.add<uint32_t>(n), a_slist = A.add<uint32_t>(n);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_log = A.add<uint32_t>(n);
-  const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
+  const size_t a_rank = A.add<uint32_t>(n), a_bsum = A.add<uint32_t>(8192);
   const size_t a_ctrl = A.add<Ctrl>(1);
   // (next to each other: together they hold the four list heads per vertex of a
   // run of AC-6 alone)
@@ -672,7 +672,7 @@ trim_err_t create_impl(const trim_csr_t* g, const trim_csr_t* gi, void* stream, 
   }
   c->level = at(a_level); c->cnt = at(a_cnt); c->supp = at(a_supp);
   c->s_head = at(a_shead); c->s_next = at(a_snext); c->s_cnt = at(a_scnt);
-  c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->roff = at(a_roff);
+  c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->s_rank = at(a_rank);
   c->live0 = at(a_live0); c->live1 = at(a_live1); c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
   c->aw = reinterpret_cast<uint4*>(c->supp);
@@ -720,7 +720,7 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   const size_t a_level = A.add<uint32_t>(n), a_rec = A.add<uint4>(n + 32);
   const size_t a_scnt = A.add<uint32_t>(n), a_soff = A.add<uint32_t>(n + 1);
   const size_t a_slist = A.add<uint32_t>(n), a_log = A.add<uint32_t>(n);
-  const size_t a_roff = A.add<uint32_t>(n + 2), a_bsum = A.add<uint32_t>(8192);
+  const size_t a_rank = A.add<uint32_t>(n), a_bsum = A.add<uint32_t>(8192);
   const size_t a_heads = A.add<uint4>(n + 32);
   const size_t a_ctrl = A.add<Ctrl>(1), a_m = A.add<unsigned long long>(1);
   const size_t a_rlog = c->rlog_cap ? A.add<trim_round_rec_t>(c->rlog_cap) : 0;
@@ -730,7 +730,7 @@ trim_err_t create_implicit_impl(const trim_implicit_graph_t* g, void* stream, ui
   c->level = at(a_level); c->supp = at(a_rec); c->cnt = nullptr;
   c->s_rec = reinterpret_cast<uint4*>(c->supp);
   c->s_cnt = at(a_scnt);
-  c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->roff = at(a_roff);
+  c->s_off = at(a_soff); c->s_list = at(a_slist); c->log = at(a_log); c->s_rank = at(a_rank);
   c->live0 = at(a_heads); c->live1 = c->live0 + ((n + 63) & ~(size_t)63); c->bsum = at(a_bsum);
   c->ctrl = reinterpret_cast<Ctrl*>(base + a_ctrl);
   if (c->rlog_cap) c->rlog = reinterpret_cast<trim_round_rec_t*>(base + a_rlog);
@@ -857,7 +857,7 @@ trim_err_t enqueue_run(trim_ctx* c, trim_variant_t variant, int seg_flavour = -1
   D.off = c->off; D.tgt = c->tgt; D.ioff = c->ioff; D.itgt = c->itgt;
   D.level = c->level; D.cnt = c->cnt; D.supp = c->supp;
   D.s_head = c->s_head; D.s_next = c->s_next; D.s_cnt = c->s_cnt; D.s_off = c->s_off;
-  D.s_list = c->s_list; D.log = c->log; D.roff = c->roff; D.live0 = c->live0;
+  D.s_list = c->s_list; D.log = c->log; D.s_rank = c->s_rank; D.live0 = c->live0;
   D.live1 = c->live1; D.w4_row = c->w4_row; D.w4_eoff = c->w4_eoff;
   D.chunk_first = c->chunk_first; D.bsum = c->bsum; D.C = c->ctrl;
   D.cnt_io = c->cnt_io; D.w4_dir = c->w4_dir;

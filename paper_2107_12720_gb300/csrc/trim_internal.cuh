@@ -171,7 +171,7 @@ struct Dev {
   uint32_t* s_off;    // AC-6 bulk supporting sets: CSR by support vertex (n+1)
   uint32_t* s_list;
   uint32_t* log;      // dead log: F_0 | F_1 | ... (n)
-  uint32_t* roff;     // roff[r] = start of F_r in the log (n+2)
+  uint32_t* s_rank;   // AC-6 alone, first build: every member's rank in its support's set
   uint32_t* live0;    // AC-3 live lists
   uint32_t* live1;
   // AC-4 work list: one entry per removed vertex with in-edges, in removal order:

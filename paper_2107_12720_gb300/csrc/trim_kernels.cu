@@ -1048,8 +1048,6 @@ __device__ ROUND_FN void advance(const Dev& D, Cta& B) {
   }
   L.bmax = max(L.bmax, max_din);  // the entries of F_r join the AC-4 backlog
   if (cta0) {
-    D.roff[r] = L.fe;
-    D.roff[r + 1] = len;
     C->rounds = nF ? r + 1 : r;
     C->n_dead = len;
   }
@@ -2844,12 +2842,11 @@ __device__ __forceinline__ void ac6_supports(const Dev& D, Cta& B, uint32_t r, u
     if (key == NIL) key = atomicCAS(sort_word(e, 1), NIL, t);
     return atomicAdd(key == NIL || key == t ? sort_word(e, 2) : &D.s_cnt[t], 1u);
   };
-  // (support and rank are parked in the link and, as the frontier offsets are read
-  // by nothing on the device, in roff until the scatter)
+  // (the support is parked in the link until the scatter)
   auto store = [&](uint32_t v, uint32_t t, uint32_t rank, uint32_t after, uint32_t pos,
                    uint32_t end) {
     D.s_rec[v] = make_uint4(t, after, pos, end);
-    D.roff[v] = rank;
+    D.s_rank[v] = rank;
   };
   uint32_t* list = slice(threadIdx.x >> 5, 3);  // at most 31 + 32 * U entries
   uint32_t nl = 0;
@@ -3051,7 +3048,7 @@ __device__ ROUND_FN bool ac6_entry(const Dev& D, Cta& B, const Sched& S, uint32_
       const uint32_t v = base + q * 32u + lane;
 #if TRIM_AC6_ONLY
       t[q] = alive[q] ? ldcg(&D.s_rec[v].x) : 0u;
-      pos[q] = alive[q] ? ldcg(&D.roff[v]) : 0u;
+      pos[q] = alive[q] ? ldcg(&D.s_rank[v]) : 0u;
 #else
       t[q] = alive[q] ? ldcg(&D.s_next[v]) : 0u;
 #endif

@@ -29,8 +29,7 @@ constexpr size_t round_up(size_t x) { return (x + kAlignWords - 1) / kAlignWords
 constexpr size_t kCtrlWords = round_up((sizeof(trimk::Ctrl) + 3) / 4);
 constexpr size_t kOffCnt = kCtrlWords;
 constexpr size_t kOffLog = kOffCnt + round_up(kMaxN);
-constexpr size_t kOffRoff = kOffLog + round_up(kMaxN);
-constexpr size_t kOffRow = kOffRoff + round_up(kMaxN + 2);
+constexpr size_t kOffRow = kOffLog + round_up(kMaxN);
 constexpr size_t kOffEoff = kOffRow + round_up(kMaxN);
 constexpr size_t kOffChunk = kOffEoff + round_up(kMaxN);
 constexpr size_t kOffSpare = kOffChunk + round_up((kMaxM >> 5) + 2);
@@ -134,7 +133,6 @@ extern "C" trim_err_t trim_run_ac4_noalloc(const uint32_t* offsets, const uint32
   D.level = level_out;
   D.cnt = base + kOffCnt;
   D.log = base + kOffLog;
-  D.roff = base + kOffRoff;
   D.w4_row = base + kOffRow;
   D.w4_eoff = base + kOffEoff;
   D.chunk_first = base + kOffChunk;
