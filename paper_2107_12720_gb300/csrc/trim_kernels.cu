@@ -234,7 +234,7 @@ __device__ __forceinline__ bool feats_on(const Dev& D, const Sched& S) {
 
 // dynamic shared memory: per warp w, 4 slices of LW words at w * 4 * LW:
 // dead-log entries | work-list rows | work-list edge offsets (warp-local) | live-list entries
-extern __shared__ uint32_t dyn_smem[];
+extern __shared__ __align__(16) uint32_t dyn_smem[];  // (AC-6 stages 16-byte records there)
 __device__ __forceinline__ uint32_t* slice(unsigned warp, int which) {
   return dyn_smem + (warp * 4u + (unsigned)which) * LW;
 }
