@@ -29,7 +29,8 @@ constexpr size_t round_up(size_t x) { return (x + kAlignWords - 1) / kAlignWords
 constexpr size_t kCtrlWords = round_up((sizeof(trimk::Ctrl) + 3) / 4);
 constexpr size_t kOffCnt = kCtrlWords;
 constexpr size_t kOffLog = kOffCnt + round_up(kMaxN);
-constexpr size_t kOffRow = kOffLog + round_up(kMaxN);
+// (one array of kMaxN + 2 words unused: the size is part of the interface)
+constexpr size_t kOffRow = kOffLog + round_up(kMaxN) + round_up(kMaxN + 2);
 constexpr size_t kOffEoff = kOffRow + round_up(kMaxN);
 constexpr size_t kOffChunk = kOffEoff + round_up(kMaxN);
 constexpr size_t kOffSpare = kOffChunk + round_up((kMaxM >> 5) + 2);
