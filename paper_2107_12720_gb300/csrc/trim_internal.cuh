@@ -95,6 +95,9 @@ struct Sched {
   uint32_t skew;
   uint32_t supp_valid;           // 1 once an AC-6 or AC-3 round set the support positions
   uint32_t lround;               // local rounds run so far (parity picks the barrier slot)
+  // the asynchronous tail handed the run back to rounds: it may start again from this
+  // round on, and waits twice as long after the next time
+  uint32_t async_from, async_wait;
   unsigned long long lbase[2];   // value of each local-barrier slot after its last round
 };
 
@@ -138,7 +141,9 @@ struct Ctrl {
   unsigned int a_round;
   unsigned int a_beat;
   unsigned int a_rebalances;
-  unsigned int _p5[16];
+  unsigned int a_hand;            // rows that workers handed on
+  unsigned int a_bmax;            // longest row among the vertices parked
+  unsigned int _p5[14];
   // segmented runs: a kernel that lacks the variant its scheduler picked saves
   // the schedule state here and exits; the kernel that has it resumes from it
   unsigned int resume;            // 1: a segment ended early, state in `saved`

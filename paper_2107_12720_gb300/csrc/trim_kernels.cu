@@ -141,6 +141,9 @@ constexpr uint32_t ASYNC_MIN_ROUND = 128;  // rounds before the tail may take ov
 constexpr uint32_t ASYNC_RETRY = 64;       // local stretches end for it at multiples of this
 constexpr uint32_t AQ_LOCAL_DMAX = 1024; // larger in-degrees always go to the global pieces
 constexpr uint32_t AQ_PIECE = 32;        // in-edges per piece of a CTA's ring (one batch)
+constexpr uint32_t ASYNC_LOOK = 128;     // rows handed on by a CTA before the first look at the tail's worth
+constexpr uint32_t ASYNC_PATIENCE = 16;  // ... and turns of its control warp with a crowded ring
+constexpr uint32_t ASYNC_WAIT = 128;     // rounds before a tail that was not may start again
 #endif
 
 // Per-CTA shared state.
@@ -185,7 +188,7 @@ struct Cta {
   // entries, rows and pieces); removals and top level not yet published;
   // entries and rows written out by a rebalance; whether the CTA holds a
   // token, asks for a rebalance; rebalances passed; first piece of the global
-  // list not yet shared out; the last batch's time (shows progress); bases of
+  // list not yet shared out; batches so far (shows progress); bases of
   // the entries and rows it writes out; its channels' last tags
   uint32_t r_head, r_tail;
   uint32_t a_idle;
@@ -201,6 +204,17 @@ struct Cta {
   uint32_t a_plo;
   uint32_t a_prog;
   uint32_t a_ebase, a_rbase;
+  // is the tail worth it (see async_rebalance): the level above which vertices are parked
+  // (NIL: none yet); rows handed on since the last rebalance, how many at least bring the
+  // next, and the batches before it;
+  // the run's removals before the tail; totals of removals and rows at the last look; turns
+  // of the control warp with a crowded ring that bring the next one
+  uint32_t a_cap;
+  uint32_t a_hand, a_look;
+  uint32_t a_base;
+  uint32_t a_seen_removed, a_seen_hand;
+  uint32_t a_prog0;
+  uint32_t a_patience;
   uint32_t ch_sent[32], ch_taken[32];
 #endif
 };
@@ -1420,7 +1434,8 @@ __device__ bool local_barrier(const Dev& D, Cta& B, uint32_t b, uint32_t r) {
     const bool last = (MODES & M_SCHED) && r + 1u >= S.cstop;
 #if TRIM_ASYNC
     const bool ask = D.async_edges_max != 0u && !(D.flags & F_ROUND_LOG) && !S.mixed &&
-                     r + 1u >= ASYNC_MIN_ROUND && (r + 1u) % ASYNC_RETRY == 0u;
+                     r + 1u >= ASYNC_MIN_ROUND && r + 1u >= S.async_from &&
+                     (r + 1u) % ASYNC_RETRY == 0u;
 #endif
     const uint64_t t0 = globaltimer();
     // relaxed polls: an acquiring load would also invalidate this SM's L1 on
@@ -1659,15 +1674,32 @@ __device__ __noinline__ bool local_stretch() {
 // ring are empty and its rows sent are acknowledged, and a count of zero (with
 // no rebalance asked for) ends the run.
 //
+// What it gains it gains where a batch removes one vertex, whose row stays in its warp
+// (chains). Where batches remove several or none, rows change hands all the time, and they
+// gather in few CTAs, as every row stays where the last of its vertex's successors went;
+// where a level has many more vertices than there are workers, every row waits for one.
+// Rounds are faster there, so the tail looks at itself: a CTA that has handed on more than a
+// row for every four batches, or whose ring stays crowded, asks for a rebalance, and that
+// compares the totals. If the tail does not pay, it goes on up to the top level removed so
+// far only; vertices of the next level are parked in the AC-4 work list, and once no CTA has
+// work, the counters return to their array and ordinary rounds go on from that list
+// (async_leave). A later tail waits ASYNC_WAIT rounds, twice as long each time.
+//
+// Measured (ms per trim; rounds only / tail as one step per CTA / without leaving / as
+// here): 3,000 levels of 100 vertices with three random successors each in the level below 8.8 /
+// 12.3 / 30.1 / 8.6; 400 levels of 3,000 with 40 8.0 / 17.6 / 28.6 / 8.3; 1,000 chains of 200
+// below 40 levels of 300,000 1.6 / 2.9 / 6.9 / 1.9; 1,000 chains of 2,000 6.1 / 5.8 / 3.0 / 3.1. The look
+// costs chains 1 to 2 per cent. (Alternating levels of one vertex with 2,000 predecessors and
+// those go through rebalances of the global pieces: 5.3 / 6.4 / 8.2 / 7.4.)
+//
 // It takes over at the start of an AC-4 round r (r >= ASYNC_MIN_ROUND) whose
 // pending work-list entries are exactly the vertices removed in round r - 1,
-// at most async_edges_max in-edges, and runs the rest of the run (with the
-// schedulers: only inside a committed stretch, as the scheduler is not
-// consulted again). Rounds before ASYNC_MIN_ROUND stay rounds (local ones
+// at most async_edges_max in-edges, and runs the rest of the run or until it leaves (with
+// the schedulers: it starts only inside a committed stretch). Rounds before ASYNC_MIN_ROUND stay rounds (local ones
 // where they can): on graphs that peel in fewer rounds they were faster.
 __device__ __forceinline__ bool async_start(const Dev& D, const Sched& S) {
   if (D.async_edges_max == 0u || S.variant != TRIM_AC4_PUSH || S.mixed) return false;
-  if ((D.flags & F_ROUND_LOG) || S.round < ASYNC_MIN_ROUND) return false;
+  if ((D.flags & F_ROUND_LOG) || S.round < ASYNC_MIN_ROUND || S.round < S.async_from) return false;
   if (S.prev_variant != TRIM_AC4_PUSH) return false;
   if ((MODES & M_SCHED) && D.mode > TRIM_AC3_PULL && !(S.cstop != 0u && S.round < S.cstop))
     return false;
@@ -1703,6 +1735,7 @@ struct AsyncWarp {
   uint32_t pr, pl, pv;
   uint32_t wj;
   uint32_t removed, top;
+  uint32_t cap;
   uint32_t phase;
   bool share;
 };
@@ -2042,6 +2075,28 @@ __device__ __forceinline__ void async_fill(const Dev& D, Cta& B, AsyncWarp& A, u
   }
 }
 
+// Warp-collective: lanes with park removed a vertex of the level after the tail's last one:
+// its row (row start, length) joins the AC-4 work list, for the round after that level.
+__device__ __noinline__ void async_park(bool park, uint32_t row, uint32_t len) {
+  const Dev& D = cta_dev;
+  const unsigned lane = lane_id(), m = __ballot_sync(FULL, park);
+  const uint32_t ew = park ? len : 0u, incl = warp_incl_scan(ew);
+  const uint32_t longest = __reduce_max_sync(FULL, ew);
+  unsigned long long o = 0;
+  if (lane == 31) {
+    o = atomicAdd(&D.C->w4, ((unsigned long long)incl << 32) | __popc(m));
+    atomicMax(&D.C->a_bmax, longest);
+  }
+  o = __shfl_sync(FULL, o, 31);
+  const uint32_t at = (uint32_t)o + __popc(m & ((1u << lane) - 1u));
+  const uint32_t eo = (uint32_t)(o >> 32) + incl - ew;
+  if (park) {
+    D.w4_row[at] = row;
+    D.w4_eoff[at] = eo;
+  }
+  mark_chunks(D, park, at, eo, eo + ew);
+}
+
 // Warp-collective: one batch. The compare-and-swaps are issued before the rows
 // of the vertices they should remove are loaded, and checked after: the row
 // accesses do not wait for them. A word whose counter is zero belongs to a
@@ -2060,7 +2115,7 @@ __device__ __forceinline__ void async_batch(const Dev& D, Cta& B, AsyncWarp& A, 
   unsigned long long prev = a.x;
   if (live) prev = atomicCAS(word, a.x, ((unsigned long long)lev << 32) | (cnt - 1u));
   uint32_t total = 0;
-  const unsigned seen = __ballot_sync(FULL, live && cnt == 1u && len != 0u);
+  const unsigned seen = __ballot_sync(FULL, live && cnt == 1u && len != 0u && lev < A.cap);
   // One row per batch: a warp that keeps several is slower (it waits for the
   // latest of more accesses), and every level waits for the slowest. Only where
   // rows pile up in the ring (more than there are warps for) are batches filled.
@@ -2093,7 +2148,7 @@ __device__ __forceinline__ void async_batch(const Dev& D, Cta& B, AsyncWarp& A, 
   if (!clean) {
     // not all as foreseen: rows of vertices that another push removed leave the
     // batch, rows of vertices removed after all join it
-    const unsigned rows = __ballot_sync(FULL, removed && len != 0u);
+    const unsigned rows = __ballot_sync(FULL, removed && len != 0u && lev < A.cap);
     if (seen & ~rows) {
       total = 0u;
       left = async_pick(A, rows, row, len, lev + 1u, many, total);
@@ -2109,7 +2164,17 @@ __device__ __forceinline__ void async_batch(const Dev& D, Cta& B, AsyncWarp& A, 
     A.removed += __popc(rm);
   }
   A.cnt = total;
-  if (left) async_surplus(D, B, left, row, len, lev + 1u);
+  if (left != 0u || A.cap != NIL) {
+    const bool park = removed && len != 0u && lev >= A.cap;
+    if (left) {
+      // rows beyond the batch's first (one that is too long, or that makes way for the last
+      // rebalance's share, tells nothing of the graph)
+      const uint32_t more = (uint32_t)__popc(left) - (total == 0u ? 1u : 0u);
+      if (lane == 0 && !A.share && more) atomicAdd(&B.a_hand, more);
+      async_surplus(D, B, left, row, len, lev + 1u);
+    }
+    if (__any_sync(FULL, park)) async_park(park, row, len);
+  }
 }
 
 // A worker warp: batches until the control warp ends the stretch (and the last
@@ -2125,13 +2190,13 @@ __device__ __forceinline__ void async_work(const Dev& D, Cta& B, AsyncWarp& A, u
       continue;
     }
     async_batch(D, B, A, K);
-    if (lane_id() == 0) set_vol(B.a_prog, (uint32_t)clock());  // (shows that this CTA goes on)
+    if (lane_id() == 0) atomicAdd(&B.a_prog, 1u);
   }
 }
 
-// One thread: releases this CTA's token, after publishing its removals and top
-// level (CTA 0 reads the totals once the token count is zero).
-__device__ __forceinline__ void async_release(const Dev& D, Cta& B) {
+// One thread: publishes this CTA's removals and top level; releases its token after
+// that (CTA 0 reads the totals once the token count is zero).
+__device__ __forceinline__ void async_publish(const Dev& D, Cta& B) {
   Ctrl* C = D.C;
   if (B.a_removed) {
     atomicAdd(&C->a_removed, B.a_removed);
@@ -2139,6 +2204,10 @@ __device__ __forceinline__ void async_release(const Dev& D, Cta& B) {
     B.a_removed = 0u;
     B.a_maxlev = 0u;
   }
+}
+__device__ __forceinline__ void async_release(const Dev& D, Cta& B) {
+  Ctrl* C = D.C;
+  async_publish(D, B);
   fence_acq_rel();  // the counts before the release
   atomicSub(&C->a_tokens, 1u);
   B.a_token = 0u;
@@ -2183,13 +2252,15 @@ __device__ __noinline__ void async_control() {
   const ulonglong2* in = &D.ch_msg[32u * blockIdx.x + lane];
   uint64_t t0 = globaltimer(), tb = t0;
   uint32_t beat = ld_relaxed(&C->a_beat), prog = vol(B.a_prog), next = AS_STEP;
-  uint32_t load = 0xFFFFFFFFu;
+  uint32_t load = 0xFFFFFFFFu, crowded = 0;
   for (uint32_t turn = 0; next == AS_STEP; ++turn) {
     // everything this turn looks at, under way together
     unsigned long long m0, m1;
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(m0), "=l"(m1) : "l"(in) : "memory");
     const uint32_t ack = ld_relaxed(&D.ch_ack[32u * blockIdx.x + lane]);
-    const bool watch = (turn & 3u) == 0u || __shfl_sync(FULL, B.a_token, 0) == 0u;
+    // (a CTA with hardly any work looks for requests every turn: others wait for it)
+    const bool watch = (turn & 3u) == 0u || __shfl_sync(FULL, B.a_token, 0) == 0u ||
+                       __popc(warp_vol(B.a_idle)) + 2u >= nwk;
     uint32_t err = 0, req = 0, tok = 0, bt = 0;
     if (watch && lane == 0) {
       err = ld_relaxed(&C->err);
@@ -2228,6 +2299,7 @@ __device__ __noinline__ void async_control() {
     __threadfence_block();
     const uint32_t head = __shfl_sync(FULL, B.r_head, 0), rows = warp_vol(B.r_tail) - head;
     const bool idle = mask == all && rows == 0u && !__any_sync(FULL, ack != ch.sent);
+    crowded = rows > 2u * nwk ? crowded + 1u : 0u;
     const uint32_t now_load = nwk - __popc(mask) + min(rows, 255u);
     if (now_load != load) {
       load = now_load;
@@ -2277,11 +2349,13 @@ __device__ __noinline__ void async_control() {
     __syncwarp();
     if (lane == 0 && (watch || idle)) {
       const uint64_t now = globaltimer();
-      const uint32_t pr = vol(B.a_prog);
+      const uint32_t pr = vol(B.a_prog), hand = vol(B.a_hand);
       if (err != 0u) {
         B.err = err;
         next = AS_DONE;
-      } else if (vol(B.a_want) || rows > QR / 2u) {
+      } else if (vol(B.a_want) || rows > QR / 2u ||
+                 (B.a_cap == NIL && ((hand >= B.a_look && hand > (pr - B.a_prog0) / 4u) ||
+                                     crowded >= B.a_patience))) {
         atomicMax(&C->a_req, B.a_gen + 1u);
         next = AS_REBALANCE;
       } else if (watch && (int)(req - B.a_gen) > 0) {
@@ -2357,6 +2431,10 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
   __syncthreads();
   const uint32_t head = B.r_head, nring = B.r_tail - head, ne = B.a_ne, nr = B.a_nr + nring;
   if (threadIdx.x == 0) {
+    async_publish(D, B);
+    if (B.a_hand) atomicAdd(&C->a_hand, B.a_hand);
+    B.a_hand = 0u;
+    B.a_prog0 = B.a_prog;
     B.a_ebase = ne ? atomicAdd(&C->e_n[par], ne) : 0u;
     B.a_rbase = nr ? atomicAdd(&C->er_n[par], nr) : 0u;
     // (cannot fail: the lists hold what every CTA can hold)
@@ -2399,6 +2477,16 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
     B.sh_plo = B.a_plo + (uint32_t)(b * tP / G);
     B.sh_phi = B.a_plo + (uint32_t)((b + 1u) * tP / G);
     B.a_plo = p_hi;
+    if (B.a_cap == NIL) {  // (the same decision in every CTA)
+      const uint32_t removed = ld_relaxed(&C->a_removed), hand = ld_relaxed(&C->a_hand);
+      const uint32_t dr = removed - B.a_seen_removed, dh = hand - B.a_seen_hand;
+      if (tR + tP > async_workers() || (dh >= ASYNC_LOOK && dh > dr / 4u))
+        B.a_cap = max(ld_relaxed(&C->a_maxlev), B.S.round - 1u);
+      B.a_seen_removed = removed;
+      B.a_seen_hand = hand;
+      B.a_look = min(2u * B.a_look, 1u << 20);
+      B.a_patience = min(2u * B.a_patience, 1u << 20);
+    }
     B.r_head = B.r_tail;  // the ring went to the list
     B.a_ne = 0u;
     B.a_nr = 0u;
@@ -2417,7 +2505,74 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
       C->a_rebalances = B.a_gen;
     }
   }
-  return grid_barrier(D, B);
+  const bool ok = grid_barrier(D, B);
+  A.cap = B.a_cap;
+  return ok;
+}
+
+// End of a tail whose last level was a_cap (all threads): the counters go back to their
+// array, and the schedule goes on with round a_cap + 2, which pushes the vertices of level
+// a_cap + 1, parked in the work list. *over: nothing was parked, the run has ended. Returns
+// false on an error.
+__device__ __noinline__ bool async_leave(bool& over) {
+  const Dev& D = cta_dev;
+  Cta& B = cta_state;
+  Ctrl* C = D.C;
+  const uint32_t stride = gridDim.x * blockDim.x;
+  unsigned long long pushed = 0;  // by the tail, for vertices without work-list entries
+  for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < D.n; v += stride) {
+    const uint4 x = __ldcg(&D.aw[v]);
+    D.cnt[v] = x.x;
+    if (MODES & M_SCHED) {
+      const uint32_t l = ldcg(&D.level[v]);
+      pushed += l >= B.S.round && l <= B.a_cap ? x.w : 0u;
+    }
+  }
+  if (MODES & M_SCHED) {
+    pushed = warp_sum(pushed);
+    if (lane_id() == 0 && pushed) atomicAdd(&C->local_edges, pushed);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    // the next rounds' accumulators (rounds cleared them two ahead)
+    for (int k = 0; k < 4; ++k) {
+      RoundStat* z = &C->rs[k];
+      z->sum_in = 0; z->sum_out = 0;
+      z->hist[0] = z->hist[1] = z->hist[2] = 0;
+      z->live_count = 0;
+      z->max_din = 0;
+    }
+  }
+  if (!grid_barrier(D, B)) return false;
+  const unsigned long long w4 = ld_relaxed64(&C->w4);
+  over = (uint32_t)w4 == B.S.w_end;
+  if (threadIdx.x == 0 && !over) {
+    Sched& S = B.S;
+    const uint32_t removed = ld_relaxed(&C->a_removed) - B.a_base, next = B.a_cap + 2u;
+    S.vcount[TRIM_AC4_PUSH] += next - S.round;
+    S.prev_variant = TRIM_AC4_PUSH;
+    S.fprev = S.fe - S.fb;
+    S.round = next;
+    S.fe += removed;
+    S.fb = S.fe - ((uint32_t)w4 - S.w_end);  // (those with in-edges)
+    S.skew += removed;
+    S.c4w = S.w_end;
+    S.e_c4 = S.e_end;
+    S.w_end = (uint32_t)w4;
+    S.e_end = (uint32_t)(w4 >> 32);
+    S.bmax = ld_relaxed(&C->a_bmax);
+    S.stable = D.commit_after ? D.commit_after - 1u : 0u;
+    if (MODES & M_SCHED)
+      for (int i = 0; i < NFEAT; ++i) S.feat[i] = 0.0f;
+    S.async_wait = S.async_wait ? min(2u * S.async_wait, 1u << 20) : ASYNC_WAIT;
+    S.async_from = next + S.async_wait;
+    if (blockIdx.x == 0) {
+      C->vcount[TRIM_AC4_PUSH] = S.vcount[TRIM_AC4_PUSH];
+      C->rounds = next;
+      C->n_dead = S.fe;
+    }
+  }
+  __syncthreads();
+  return true;
 }
 
 // Runs the rest of the run asynchronously from round B.S.round = r0 (all
@@ -2425,7 +2580,8 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
 // the workers push the pending work-list entries (level r0 - 1) and what
 // follows from them until the token count is zero. CTA 0 then publishes the
 // run's totals: alpha = top level + 1 (r0 if the tail removed nothing), and
-// one AC-4 round for each of rounds r0 .. alpha. Returns false on an error.
+// one AC-4 round for each of rounds r0 .. alpha; or, where the tail left (see async_leave),
+// rounds go on. Returns false on an error.
 __device__ __noinline__ bool async_tail() {
   const Dev& D = cta_dev;
   Cta& B = cta_state;
@@ -2472,13 +2628,20 @@ __device__ __noinline__ bool async_tail() {
     B.a_ne = B.a_nr = 0u;
     B.a_token = 1u;
     B.a_want = 0u;
-    B.a_gen = 0u;
-    B.a_plo = 0u;
-    B.a_prog = 0u;
+    // (what an earlier tail of the run left: nothing changes it between tails)
+    B.a_plo = ld_relaxed(&C->oq_res);
+    B.a_base = B.a_seen_removed = ld_relaxed(&C->a_removed);
+    B.a_seen_hand = ld_relaxed(&C->a_hand);
+    B.a_prog = B.a_prog0 = 0u;
+    B.a_cap = NIL;
+    B.a_hand = 0u;
+    B.a_look = ASYNC_LOOK;
+    B.a_patience = ASYNC_PATIENCE;
     D.ch_load[blockIdx.x] = nwk;
     if (blockIdx.x == 0) {
       C->a_tokens = gridDim.x;
-      C->a_round = r0;
+      C->a_bmax = 0u;
+      if (C->a_round == 0u) C->a_round = r0;
     }
   }
   if (!grid_barrier(D, B, false)) return false;
@@ -2490,6 +2653,7 @@ __device__ __noinline__ bool async_tail() {
   A.pr = A.pl = A.pv = 0u;
   A.wj = warp < nwk ? B.S.c4w + warp * gridDim.x + blockIdx.x : B.S.w_end;
   A.removed = A.top = 0u;
+  A.cap = NIL;
   A.phase = 0u;
   A.share = true;
   bool ok = true;
@@ -2504,10 +2668,18 @@ __device__ __noinline__ bool async_tail() {
     }
   }
   stats_flush(D, B, K);
-  if (threadIdx.x == 0) {
+  __syncthreads();
+  if (threadIdx.x == 0)  // (the next tail initialises them again)
+    for (uint32_t w = 0; w < MAX_WARPS; ++w)
+      asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(&B.w_bar[w])) : "memory");
+  bool over = true;
+  if (ok && B.err == 0u && B.a_cap != NIL) {
+    if (!async_leave(over)) return false;
+  }
+  if (threadIdx.x == 0 && over) {
     if (blockIdx.x == 0 && ok && B.err == 0u) {
       fence_acq_rel();  // every CTA published its counts before its last release
-      const uint32_t removed = ld_relaxed(&C->a_removed);
+      const uint32_t removed = ld_relaxed(&C->a_removed) - B.a_base;
       const uint32_t top = ld_relaxed(&C->a_maxlev);
       Sched& S = B.S;
       const uint32_t alpha = removed ? max(r0, top + 1u) : r0;
@@ -3755,6 +3927,7 @@ __global__ void __launch_bounds__(512, TRIM_MIN_BLOCKS) TRIM_KERNEL(const __grid
     S.supp_valid = 0;
     S.lround = 0;
     S.lbase[0] = S.lbase[1] = 0;
+    S.async_from = S.async_wait = 0;
 
     for (int w = 0; w < MAX_WARPS; ++w) {
       WarpSlice& x = B.ws[w];
@@ -3771,6 +3944,9 @@ __global__ void __launch_bounds__(512, TRIM_MIN_BLOCKS) TRIM_KERNEL(const __grid
     B.lq_cnt[0] = B.lq_cnt[1] = 0;
     B.lq_vend[0] = B.lq_vend[1] = 0;
     B.lq_k = B.lq_ovf = B.lq_pushed = 0;
+#if TRIM_ASYNC
+    B.a_gen = 0;
+#endif
 #if TRIM_AC3_ONLY
     B.live_n[0] = B.live_n[1] = 0;
 #endif
