@@ -143,6 +143,7 @@ constexpr uint32_t AQ_LOCAL_DMAX = 1024; // larger in-degrees always go to the g
 constexpr uint32_t AQ_PIECE = 32;        // in-edges per piece of a CTA's ring (one batch)
 constexpr uint32_t ASYNC_LOOK = 128;     // rows handed on by a CTA before the first look at the tail's worth
 constexpr uint32_t ASYNC_PATIENCE = 16;  // ... and turns of its control warp with a crowded ring
+constexpr uint32_t ASYNC_CLOSE = 192;  // ... and rebalances in a row at most four levels apart that end it
 constexpr uint32_t ASYNC_WAIT = 128;     // rounds before a tail that was not may start again
 #endif
 
@@ -207,12 +208,14 @@ struct Cta {
   // is the tail worth it (see async_rebalance): the level above which vertices are parked
   // (NIL: none yet); rows handed on since the last rebalance, how many at least bring the
   // next, and the batches before it;
-  // the run's removals before the tail; totals of removals and rows at the last look; turns
-  // of the control warp with a crowded ring that bring the next one
+  // the run's removals before the tail; totals of removals and rows and the top level at the
+  // last rebalance, and how many of them came soon after each other; turns of the control
+  // warp with a crowded ring that bring the next one
   uint32_t a_cap;
   uint32_t a_hand, a_look;
   uint32_t a_base;
   uint32_t a_seen_removed, a_seen_hand;
+  uint32_t a_seen_top, a_close;
   uint32_t a_prog0;
   uint32_t a_patience;
   uint32_t ch_sent[32], ch_taken[32];
@@ -1689,8 +1692,9 @@ __device__ __noinline__ bool local_stretch() {
 // here): 3,000 levels of 100 vertices with three random successors each in the level below 8.8 /
 // 12.3 / 30.1 / 8.6; 400 levels of 3,000 with 40 8.0 / 17.6 / 28.6 / 8.3; 1,000 chains of 200
 // below 40 levels of 300,000 1.6 / 2.9 / 6.9 / 1.9; 1,000 chains of 2,000 6.1 / 5.8 / 3.0 / 3.1. The look
-// costs chains 1 to 2 per cent. (Alternating levels of one vertex with 2,000 predecessors and
-// those go through rebalances of the global pieces: 5.3 / 6.4 / 8.2 / 7.4.)
+// costs chains 1 to 2 per cent. Rows over AQ_LOCAL_DMAX in-edges at every other level bring a
+// rebalance each, slower than a round: ASYNC_CLOSE of those in a row end the tail as well (800
+// levels, every other one a vertex with 2,000 predecessors: 5.3 / 6.4 / 8.2 / 7.1).
 //
 // It takes over at the start of an AC-4 round r (r >= ASYNC_MIN_ROUND) whose
 // pending work-list entries are exactly the vertices removed in round r - 1,
@@ -2167,10 +2171,10 @@ __device__ __forceinline__ void async_batch(const Dev& D, Cta& B, AsyncWarp& A, 
   if (left != 0u || A.cap != NIL) {
     const bool park = removed && len != 0u && lev >= A.cap;
     if (left) {
-      // rows beyond the batch's first (one that is too long, or that makes way for the last
-      // rebalance's share, tells nothing of the graph)
+      // rows beyond the batch's first (a single one that is too long, or that makes way for
+      // the last rebalance's share, tells nothing of the graph)
       const uint32_t more = (uint32_t)__popc(left) - (total == 0u ? 1u : 0u);
-      if (lane == 0 && !A.share && more) atomicAdd(&B.a_hand, more);
+      if (lane == 0 && more) atomicAdd(&B.a_hand, more);
       async_surplus(D, B, left, row, len, lev + 1u);
     }
     if (__any_sync(FULL, park)) async_park(park, row, len);
@@ -2480,8 +2484,12 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
     if (B.a_cap == NIL) {  // (the same decision in every CTA)
       const uint32_t removed = ld_relaxed(&C->a_removed), hand = ld_relaxed(&C->a_hand);
       const uint32_t dr = removed - B.a_seen_removed, dh = hand - B.a_seen_hand;
-      if (tR + tP > async_workers() || (dh >= ASYNC_LOOK && dh > dr / 4u))
-        B.a_cap = max(ld_relaxed(&C->a_maxlev), B.S.round - 1u);
+      const uint32_t top = max(ld_relaxed(&C->a_maxlev), B.S.round - 1u);
+      B.a_close = top - B.a_seen_top <= 4u ? B.a_close + 1u : 0u;
+      if (tR + tP > async_workers() || (dh >= ASYNC_LOOK && dh > dr / 4u) ||
+          B.a_close >= ASYNC_CLOSE)
+        B.a_cap = top;
+      B.a_seen_top = top;
       B.a_seen_removed = removed;
       B.a_seen_hand = hand;
       B.a_look = min(2u * B.a_look, 1u << 20);
@@ -2632,6 +2640,8 @@ __device__ __noinline__ bool async_tail() {
     B.a_plo = ld_relaxed(&C->oq_res);
     B.a_base = B.a_seen_removed = ld_relaxed(&C->a_removed);
     B.a_seen_hand = ld_relaxed(&C->a_hand);
+    B.a_seen_top = r0 - 1u;
+    B.a_close = 0u;
     B.a_prog = B.a_prog0 = 0u;
     B.a_cap = NIL;
     B.a_hand = 0u;
