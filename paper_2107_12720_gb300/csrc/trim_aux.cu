@@ -228,6 +228,7 @@ trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n, uin
   uint32_t* first = mark + kGtTile;
   uint32_t* dist = first + nb;
   __shared__ uint32_t wmax[kGtThreads / 32];
+  __shared__ uint32_t far;  // the tile spans more rows than are looked at
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
   const uint32_t e0 = gt_piece(blockIdx.x, piece, m), e1 = gt_piece(blockIdx.x + 1ull, piece, m);
   // a row that starts at or before the piece: the last of those tried, narrowed down
@@ -245,6 +246,7 @@ trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n, uin
     const uint32_t tile = (uint32_t)t0, size = min((uint32_t)kGtTile, e1 - tile);
     for (uint32_t i = threadIdx.x; i < kGtTile; i += kGtThreads) mark[i] = i ? 0u : ra;
     for (uint32_t b = threadIdx.x; b < nb; b += kGtThreads) first[b] = 0u;
+    if (threadIdx.x == 0) far = 0u;
     uint32_t t[U], rank[U], row[U];
 #pragma unroll
     for (int q = 0; q < U; ++q)
@@ -258,12 +260,15 @@ trim_gt_scatter_kernel(const uint32_t* off, const uint32_t* tgt, uint32_t n, uin
       if (o >= tile + size) break;
       atomicMax(&mark[o > tile ? o - tile : 0u], (uint32_t)r);
     }
-    const bool far = __syncthreads_or(r >= r_end && r_end < n) != 0;
+    if (r >= r_end && r_end < n) far = 1u;
 #pragma unroll
     for (int q = 0; q < U; ++q)
       rank[q] = t[q] < n ? atomicAdd(&first[t[q] >> shift], 1u) : 0u;
-    if (far) gt_far_rows(off, n, ra, tile, size, mark);
     __syncthreads();
+    if (far) {  // block-uniform
+      gt_far_rows(off, n, ra, tile, size, mark);
+      __syncthreads();
+    }
     // running maximum of the marks
     uint32_t carry = 0;
 #pragma unroll
