@@ -1502,12 +1502,12 @@ __device__ __noinline__ bool local_stretch() {
   // (about 12 us) spreads the work evenly again. Kernel ms, with the bound and
   // with queues filled to LQ_EDGES: in+out of 2^23 vertices 6.73 and 7.52, of 2^20
   // 1.354 and 1.510; AC-4 of 2^24 (rounds only) 12.4 and 13.2, of 2^20 1.205 and
-  // 1.283; 256 packed graphs 0.616 and 0.601. Multiples of 2 to 6 on an in+out
-  // cascade of 5,000,011: 4.61, 4.45, 4.54, 4.68, 4.85 (2: packed graphs 0.84). Where few
-  // edges are pending a full queue is cheaper than leaving, so the bound has a floor:
-  // kernel us with 256 / 512 / 768 / 1,024, packed graphs, 64 402 / 350 / 348 / 356, 80 462 / 405 /
-  // 396 / 400, 256 570 / 556 / 552 / 552; in+out of 2^20 1,055 / 1,049 / 1,145 / 1,202, of
-  // 5,000,011 4,218 / 4,218 / 4,575 / 4,835.
+  // 1.283. Multiples of 3 / 4 / 6: in+out of 5,000,011 4.15 / 4.21 / 4.52, of 2^20 1.049 /
+  // 1.045 / 1.083, 200 packed graphs 0.581 / 0.554 / 0.537. Where few edges are pending a
+  // full queue is cheaper than leaving, so the bound has a floor: kernel us with 256 / 512 /
+  // 768 / 1,024, packed graphs, 64 402 / 350 / 348 / 356, 80 462 / 405 / 396 / 400, 256 570 / 556 /
+  // 552 / 552; in+out of 2^20 1,055 / 1,049 / 1,145 / 1,202, of 5,000,011 4,218 / 4,218 / 4,575 /
+  // 4,835.
   const float mean = __fdividef((float)(B.S.e_end - B.S.e_c4), (float)gridDim.x);
   const uint32_t cap = min(LQ_EDGES, max(LQ_FLOOR, (uint32_t)((float)LQ_SKEW * mean)));
   const bool late = D.n > LQ_LATE_MIN;
@@ -1661,11 +1661,11 @@ __device__ __noinline__ bool local_stretch() {
 // each, to CTAs with idle workers (channels, see async_control).
 //
 // Measured (ms per trim, kernel only; chains of 2,867 and 10,000 levels): the
-// deep cascade 2^24 6.7, the large mixed graph 21.0. As one step per CTA, two
-// pushes per thread, with a rebalance of all CTAs when a queue grew: 11.4 and
-// 36.2 (a level paid for the word, the swap, the row and two CTA barriers in
-// turn). With batches of several rows, up to 32 pushes: 8.9 and 29.4; 16: 7.8
-// and 25.1.
+// deep cascade 2^24 6.45, the large mixed graph 20.5. As one step per CTA, two
+// pushes per thread, with a rebalance of all CTAs when a queue grew: 11.3 and
+// 36.1 (a level paid for the word, the swap, the row and two CTA barriers in
+// turn). With batches of several rows (first build, one row 6.7 and 21.0), up to 32
+// pushes: 8.9 and 29.4; 16: 7.8 and 25.1.
 //
 // Rows in the global pieces, or a ring half full, need a rebalance: every CTA's
 // workers stop after their batch, write what they hold (entries of their batch,
@@ -2719,10 +2719,10 @@ __device__ __noinline__ bool async_tail() {
 // one word, and the push sees both. Edges are balanced over the warps in
 // 32-edge chunks as in ac4_round.
 //
-// Measured (ms per run, deep cascades of 5,000,011 vertices and 1,001 rounds /
-// 2^20 and 501 / 2^22 and 151): 4.26 / 2.0 / 1.4 with local rounds; before, with
-// both rows pushed, a compare-and-swap of the level and every round through the
-// global lists, 7.94 / 3.79 / 1.76.
+// Measured (kernel ms, deep cascades of 5,000,011 vertices and 1,001 rounds / 2^20
+// and 251 / R-MAT 2^22 / 2^23): 4.21 / 1.05 / 0.139 / 0.251; with both rows pushed, a
+// compare-and-swap of the level and every round through the global lists 8.32 /
+// 2.02 / 0.155 / 0.268.
 __device__ ROUND_FN void inout_round(const Dev& D, Cta& B, const Sched& S, uint32_t gwarp,
                                      uint32_t nwarps) {
   constexpr int U = 4;

@@ -28,10 +28,10 @@
 // and rows over kSccHeavy edges, cut into pieces and those laid end to end, over the
 // whole grid (one warp on a hub's row was what a level waited for).
 //
-// Measured (ms, in+out trimming included; before: one launch and one host read
-// per level and pass, a warp per row, searches from every vertex in every step):
-// R-MAT scale 14 0.13 (0.80), 20 0.29 (5.9), 22 0.65 (16.7); 4,096 planted graphs
-// in one call 17.7 (51.1); a planted graph of 100,000 0.47 (0.89).
+// Measured (ms per call, in+out trimming included; before: one launch and one host
+// read per level and pass, a warp per row, searches from every vertex in every step):
+// R-MAT scale 20 0.34 (6.3), 22 0.71 (17.4); 1,024 packed planted graphs 5.1 (15.2); a
+// planted graph of 100,000 0.43 (0.95); 20 dense parts joined in a row 20 (42).
 #include "trim_internal.cuh"
 
 using namespace trimk;
@@ -41,6 +41,9 @@ constexpr uint32_t SCC_OPEN = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t CLOSED = 0xFFFFFFFFu;  // search mark of a vertex with a component
 constexpr unsigned FULL = 0xFFFFFFFFu;
+// (20 parts of 2,000 vertices with 1,500 / 1,000 edges each, ms: kSccHeavy of 512, 1,024, 4,096
+// 0.93 / 0.76, 0.93 / 1.00, 1.28 / 0.94, 2,000 hubs of 3,000 leaves 1.43, 1.43, 2.30; kSccChunk of
+// 128, 256, 1,024 0.92 / 0.99, 0.93 / 1.00, 1.18 / 1.07, R-MAT 2^20 0.333, 0.343, 0.414)
 constexpr uint32_t kSccHeavy = 1024;   // longer rows go to the whole grid ...
 constexpr uint32_t kSccChunk = 256;    // ... in pieces of this many edges
 constexpr uint32_t kBuf = 256;         // entries staged per warp before a flush
@@ -373,7 +376,8 @@ __device__ __forceinline__ void close_vertex(const SccArgs& A, uint32_t v, uint3
 // (off, tgt), whose transpose is (roff, rtgt), among the open vertices in
 // `allow` (where given: those whose mark there is allowed). A small frontier
 // offers its rows; once it is large, the vertices not yet marked look for a
-// marked neighbour instead (usually within a few entries). Returns false on an
+// marked neighbour instead (usually within a few entries; large from 1/4, 1/16, 1/64 of
+// them on: R-MAT 2^20 0.597, 0.343, 0.342 ms, dense parts 0.94, 0.93, 1.16). Returns false on an
 // error.
 __device__ bool search(const SccArgs& A, Scc& S, const uint32_t* off, const uint32_t* tgt,
                        const uint32_t* roff, const uint32_t* rtgt, uint32_t* mark, uint32_t stamp,
