@@ -2980,11 +2980,12 @@ __device__ unsigned block_sum(unsigned x) {
 // scatter needs no atomics. The table lies in append slices that AC-6 does not use:
 // keys, counts, and the CTA's first rank of each support.
 constexpr uint32_t AC6_HEADS = 4;
-// Rows in host memory come over the link, entry by entry as they are needed: a record then
-// holds UNREAD instead of the next successor (ids are below 2^31), and row bounds are
-// read once. AC-6 of R-MAT of 2^22 vertices read in place, call us: 785 with the next
-// successors read ahead, 608 without, 574 with the bounds
-// read once as well (581 before the records).
+// Rows in host memory come over the link, entry by entry as they are needed: after the
+// first build a record then holds UNREAD instead of the next successor (ids are below 2^31),
+// and row bounds are read once there. (Later re-scans, far fewer, read ahead as elsewhere;
+// the check there cost AC-6 of packed graphs 0.7 per cent.) AC-6 of R-MAT of 2^22 vertices
+// read in place, call us: 785 with all next successors read ahead, 567 so (574 before the
+// records), 2^20 242, 189 (212).
 constexpr uint32_t UNREAD = 0xFFFFFFFEu;
 __device__ __forceinline__ bool rows_far(const Dev& D) {
   return !(MODES & M_IMPLICIT) && (D.flags & F_ROWS_FAR) != 0u;
@@ -3310,8 +3311,7 @@ __device__ __forceinline__ void log_removed(const Dev& D, unsigned mask, uint32_
 template <bool LOCAL>
 __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uint32_t v, uint32_t t,
                                            uint32_t pos, uint32_t end, uint32_t r, Counters& K) {
-  const bool far = rows_far(D);
-  if (valid && t == UNREAD) t = row_target(D, v, 0u, pos);
+  if (!(MODES & M_IMPLICIT) && valid && t == UNREAD) t = row_target(D, v, 0u, pos);
   const bool cand = valid && t != NIL;
   // members without a successor left die: their log space is asked for first
   const unsigned now = __ballot_sync(FULL, valid && !cand);
@@ -3319,7 +3319,7 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
   uint32_t lv = 0, after = NIL;
   if (cand) {
     lv = ldcg(&D.level[t]);
-    if (pos + 1u < end) after = far ? UNREAD : row_target(D, v, 0u, pos + 1u);
+    if (pos + 1u < end) after = row_target(D, v, 0u, pos + 1u);
     K.edges += 1;
   }
   bool found = cand && lv >= r;
@@ -3328,14 +3328,14 @@ __device__ __forceinline__ void ac6_rescan(const Dev& D, Cta& B, bool valid, uin
     uint32_t i = pos + 1u;
     bool resolved = !(cand && !found);
     // one or two rows: the whole warp scans each, 32 successors in one step; more of
-    // them (and rows read over the link): each lane its own first, four successors in a step
-    if ((far || __popc(scan) > 2) && !resolved) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
+    // them: each lane its own first, four successors in a step
+    if (__popc(scan) > 2 && !resolved) i = scan_thread(D, v, 0u, end, i, r, 2, resolved, K);
     scan_warp_finish(D, resolved, v, 0u, end, i, r, K);
     if (cand && !found && i < end) {
       found = true;
       pos = i;
       t = row_target(D, v, 0u, i);
-      after = i + 1u >= end ? NIL : far ? UNREAD : row_target(D, v, 0u, i + 1u);
+      after = i + 1u < end ? row_target(D, v, 0u, i + 1u) : NIL;
     }
   }
   if (found) {
