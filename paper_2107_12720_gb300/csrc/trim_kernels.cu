@@ -2520,9 +2520,9 @@ __device__ __forceinline__ bool async_rebalance(const Dev& D, Cta& B, AsyncWarp&
 
 // End of a tail whose last level was a_cap (all threads): the counters go back to their
 // array, and the schedule goes on with round a_cap + 2, which pushes the vertices of level
-// a_cap + 1, parked in the work list. *over: nothing was parked, the run has ended. Returns
-// false on an error.
-__device__ __noinline__ bool async_leave(bool& over) {
+// a_cap + 1, parked in the work list; where nothing was parked the run has ended (B.S stays
+// as it was). Returns false on an error.
+__device__ __noinline__ bool async_leave() {
   const Dev& D = cta_dev;
   Cta& B = cta_state;
   Ctrl* C = D.C;
@@ -2552,8 +2552,7 @@ __device__ __noinline__ bool async_leave(bool& over) {
   }
   if (!grid_barrier(D, B)) return false;
   const unsigned long long w4 = ld_relaxed64(&C->w4);
-  over = (uint32_t)w4 == B.S.w_end;
-  if (threadIdx.x == 0 && !over) {
+  if (threadIdx.x == 0 && (uint32_t)w4 != B.S.w_end) {
     Sched& S = B.S;
     const uint32_t removed = ld_relaxed(&C->a_removed) - B.a_base, next = B.a_cap + 2u;
     S.vcount[TRIM_AC4_PUSH] += next - S.round;
@@ -2682,11 +2681,8 @@ __device__ __noinline__ bool async_tail() {
   if (threadIdx.x == 0)  // (the next tail initialises them again)
     for (uint32_t w = 0; w < MAX_WARPS; ++w)
       asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(&B.w_bar[w])) : "memory");
-  bool over = true;
-  if (ok && B.err == 0u && B.a_cap != NIL) {
-    if (!async_leave(over)) return false;
-  }
-  if (threadIdx.x == 0 && over) {
+  if (ok && B.err == 0u && B.a_cap != NIL && !async_leave()) return false;
+  if (threadIdx.x == 0 && B.S.round == r0) {  // (not handed back to rounds)
     if (blockIdx.x == 0 && ok && B.err == 0u) {
       fence_acq_rel();  // every CTA published its counts before its last release
       const uint32_t removed = ld_relaxed(&C->a_removed) - B.a_base;
